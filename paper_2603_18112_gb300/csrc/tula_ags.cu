@@ -58,43 +58,29 @@
 
 namespace {
 
-// A stage ring: kStages shared-memory stages of kStageBytes each (one tile of
-// every stream), one producer warp and kConsumers consumer warps.  A consumer
-// must own whole stages: the tile it waits for on a stage is then always the
-// one after its own previous tile there, so a parity wait never sees a phase
-// two ahead.
-template <int StageKB, int Stages, int Consumers>
+// The stages of a streaming kernel's CTA: one per warp, each holding one tile of every stream.  A
+// warp refills its own stage (see "Streaming warps" below), so a CTA is nothing but warps that
+// stream for themselves.
+template <int StageKB, int Warps>
 struct Ring {
     static constexpr int kStageBytes = StageKB * 1024;
-    static constexpr int kStages = Stages;
-    static constexpr int kConsumers = Consumers;
-    static constexpr int kThreads = 32 * (1 + Consumers);
-    static constexpr int kSmemBytes = Stages * kStageBytes + 2 * Stages * 8 + Stages * 4;
-    static_assert(Stages % Consumers == 0, "consumers own whole stages");
+    static constexpr int kWarps = Warps;
+    static constexpr int kThreads = 32 * Warps;
+    static constexpr int kSmemBytes = Warps * (kStageBytes + 8);
     static_assert(kSmemBytes <= 227 * 1024, "one CTA per SM");
     // Elements per tile when `streams` tensors share one stage (multiple of 128).
     __host__ __device__ static constexpr int tile_elems(int streams) {
         return (kStageBytes / (4 * streams)) / 128 * 128;
     }
 };
-// Pass 1 streams K (+1, +2) tensors through 36 KB stages.  Six consumer warps, two per
-// scheduler: the precise norms spend ~13 dependent FP32 instructions per element and norm, and
-// the default ones add their tile sums into the accumulators at the end of each batch; with
-// three warps the reduction ran 0.8 % slower alone (the same step time).
-using Ring1 = Ring<36, 6, 6>;
-// Pass 1 when it also reads w (LARS, tula_layer_stats) streams through five 45 KB stages with
-// five consumers: the larger tiles (1280 elements for K = 8 and w) make every bulk copy 5 KB
-// instead of 4 KB, and the LARS step ran 2.5 % faster (ResNet-50, 248.1 -> 241.9 us); without
-// w (8 streams) the same ring measured 0.5 % slower.
-using Ring1W = Ring<45, 5, 5>;
+// Pass 1 streams K (+1, +2) tensors through 36 KB stages.
+using Ring1 = Ring<36, 6>;
+// Pass 1 when it also reads w (LARS, tula_layer_stats): five 45 KB stages.
+using Ring1W = Ring<45, 5>;
 template <bool RW>
 using Ring1Of = std::conditional_t<RW, Ring1W, Ring1>;
-// Pass 2 does ~11 flops per element over 3-4 streams: with three consumer warps they, not HBM,
-// set its pace, so it runs four.
-using Ring2 = Ring<24, 8, 4>;
-constexpr int kDynTiles = 64;            // tiles per CTA from which a launch claims its tiles
-constexpr unsigned kClaim = 4;           // tiles per claim
-constexpr unsigned kClaimTail = 16;      // single-tile claims for the last kClaimTail per CTA
+// Pass 2: eight 24 KB stages.
+using Ring2 = Ring<24, 8>;
 constexpr int kPend = 4;                // tiles whose warp reductions run together
 constexpr int kFinWarps = 4;            // k_finish: one warp per tensor, 4 per CTA
 constexpr int kParamBudget = 31 * 1024; // kernel parameter bytes per launch (limit 32764)
@@ -512,9 +498,6 @@ __device__ __forceinline__ void mbar_arrive_tx(uint64_t *bar, uint32_t bytes) {
                  "r"(bytes)
                  : "memory");
 }
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
-}
 __device__ __forceinline__ bool mbar_test(uint64_t *bar, uint32_t parity) {
     uint32_t ok;
     asm volatile(
@@ -571,8 +554,8 @@ __device__ __forceinline__ void report_timeout(const Scalars &sc) {
 // Tile table lookups
 // ----------------------------------------------------------------------------
 
-__device__ __forceinline__ int find_tensor(const int *cstart, int n, int c) {
-    int lo = 0, hi = n;  // cstart[lo] <= c < cstart[hi]
+__device__ __forceinline__ int find_tensor(const int *cstart, int lo, int hi, int c) {
+    // cstart[lo] <= c < cstart[hi]
     while (hi - lo > 1) {
         int mid = (lo + hi) >> 1;
         if (cstart[mid] <= c) lo = mid; else hi = mid;
@@ -580,16 +563,17 @@ __device__ __forceinline__ int find_tensor(const int *cstart, int n, int c) {
     return lo;
 }
 
-// Follows the tensor index along a monotone sequence of tiles (one CTA's tiles,
-// ascending or descending): O(1) per tile instead of a search.
+// Follows the tensor index along one warp's tiles, which ascend: the next two tensors are tried
+// first, then a search over the rest.
 struct Walker {
     int t = -1;
     template <int NP>
     __device__ __forceinline__ int to(const Table<NP> &tab, int c) {
-        if (t < 0) return t = find_tensor(tab.cstart, tab.n, c);
-        while (c >= tab.cstart[t + 1]) ++t;
-        while (c < tab.cstart[t]) --t;
-        return t;
+        if (t < 0) return t = find_tensor(tab.cstart, 0, tab.n, c);
+        if (c < tab.cstart[t + 1]) return t;
+        ++t;
+        if (c < tab.cstart[t + 1]) return t;
+        return t = find_tensor(tab.cstart, t + 1, tab.n, c);
     }
 };
 
@@ -652,172 +636,110 @@ struct TensorCache {
 };
 
 // ----------------------------------------------------------------------------
-// The producer: TMA bulk copies of each tile's streams into the stage ring
+// Streaming warps: TMA bulk copies of each tile's streams into a warp's own stage
 // ----------------------------------------------------------------------------
 //
-// Two ways to deal a launch's tiles to its persistent CTAs:
-//  * round-robin (tile blockIdx.x + j * gridDim.x), for launches of fewer than
-//    kDynTiles tiles per CTA: nothing to claim, nothing to wait for;
-//  * claimed, for larger launches: the producer warp of each CTA takes kClaim
-//    consecutive tiles at a time from a global counter (ctr[0]), with one
-//    claim in flight while it issues the range before (see produce()).  SMs
-//    do not stream at equal rates (on
-//    large launches the last CTA of a round-robin deal finished 15-30% after
-//    the median), so claiming lets the faster SMs take more tiles and the
-//    launch end with the memory system rather than with its slowest SM.  The
-//    last CTA to finish puts both counters (ctr[0], ctr[1]) back to zero.
-// Where a tile is processed never changes its result: each tile's partial sums
-// are added exactly, in integers, into its tensor's accumulators.  The j-th
-// tile of a CTA goes to stage j % kStages and is consumed by consumer warp
-// j % kConsumers; its launch tile index is left in stage_tile[stage] before the
-// stage's full barrier is armed (the barrier's release/acquire orders it), and
-// -1 there tells a consumer that no tile is left.  Lane i < ns of the producer
-// fetches stream i's pointer (role roles[i]) and issues that stream's copy to
-// offset i * chunk floats of the stage.  Both passes walk the tiles in the same
-// order (measured: walking pass 2 backwards, to start on the mean pass 1 wrote
-// last, was 1 % slower per step).
+// Each warp streams for itself: it has one stage of shared memory and one mbarrier, waits for the
+// tile in it, computes, and issues its next tile into the same stage as soon as every lane has read
+// the last one, before it adds that tile's sums up.  Lane i < ns fetches stream i's pointer (role
+// roles[i]) and issues that stream's copy to offset i * chunk floats of the stage.  While one warp
+// of a CTA computes, the others' copies are in flight; nothing is handed from warp to warp.
+// A producer warp that issues for all of them, as here before, is what bounded the passes: one
+// warp issues a bulk copy every ~27 ns (the lanes of one instruction go in turn), so 16 streams
+// of 2 KB took 0.83 us of a 36 KB stage's 0.80 us at the HBM rate, and 8 streams delayed every
+// refill.  Streams read this way alone run at 6.95-6.99 TB/s whatever the copy size (512 B to
+// 18 KB), against 6.09 TB/s with one producer warp and 16 copies of 2 KB.
+//
+// Dealing: a launch has V = gridDim.x * kWarps streaming warps; warp v first takes tile v, then,
+// when there are more tiles than warps, tiles claimed one at a time from a global counter
+// (ctr[0]), the claim made a whole tile ahead so that its round trip is never waited for.  SMs
+// stream at unequal rates; with 36 KB tiles claims run at 7.19-7.25 TB/s where a fixed deal runs
+// at 6.95.  (Tiles under ~18 KB would be bound by the counter: one atomic every 1.5-2.8 ns.)  The
+// last warp to finish puts both counters (ctr[0], ctr[1]) back to zero.  Where a tile is processed
+// never changes its result: each tile's partial sums are added exactly, in integers, into its
+// tensor's accumulators.
+template <typename R>
+struct Stream {
+    uint32_t stage;  // shared-memory address of this warp's stage
+    uint64_t *bar;   // its mbarrier: one arrival, which arms the bytes of all streams
+    uint32_t phase = 0;
+    unsigned nc, V;
+    bool claims;
+    unsigned *ctr;
+    unsigned pend = 0;  // lane 0: the claim in flight
+    uint64_t policy;
+    bool hint;
+    TensorCache tc;  // of the tile in the stage (or on its way there)
 
-__device__ __forceinline__ unsigned claim_tiles(unsigned *ctr, unsigned n) {
-    return atomicAdd(ctr, n);
-}
-
-// Round-robin tiles of this CTA (0 when the launch claims its tiles).
-__device__ __forceinline__ int static_tiles(int nc) {
-    const int g = (int)gridDim.x, b = (int)blockIdx.x;
-    if (nc >= kDynTiles * g) return 0;
-    return b < nc ? (nc - b + g - 1) / g : 0;
-}
-__device__ __forceinline__ bool claims_tiles(int nc) { return nc >= kDynTiles * (int)gridDim.x; }
-__device__ __forceinline__ int static_tile(int j) { return (int)blockIdx.x + j * (int)gridDim.x; }
-
-template <typename R, int NP, int NS>
-__device__ __forceinline__ void produce(const Table<NP> &tab, const Scalars &sc,
-                                        const int (&roles)[NS], int ns, int chunk,
-                                        int js, unsigned *ctr, uint32_t ring,
-                                        uint64_t *full, uint64_t *empty, int *stage_tile) {
-    const int lane = threadIdx.x & 31;
-    const int role = lane < ns ? roles[lane] : 0;
-    const unsigned nc = (unsigned)tab.nc;
-    const bool claim = claims_tiles(tab.nc);
-    const bool hint = sc.evict_first != 0;
-    const uint64_t policy = policy_evict_first();
-    TensorCache tc;
-    // Claiming (lane 0): tiles [cur, cur_end) are being issued, [nxt, nxt_end) come next and
-    // one claim is in flight.  The first two ranges of each CTA are dealt, not claimed (152
-    // CTAs claiming at once would queue on the counter at the start); claimed ranges begin
-    // after them.  Near the end, claims shrink to one tile so that CTAs do not hold tiles
-    // others could have taken.
-    const unsigned G = gridDim.x, b = blockIdx.x;
-    const unsigned base = 2u * G * kClaim;
-    unsigned cur = b * kClaim, cur_end = cur + kClaim;
-    unsigned nxt = (G + b) * kClaim, nxt_end = nxt + kClaim;
-    unsigned pend = 0u, pend_k = kClaim;
-    if (claim && lane == 0) pend = claim_tiles(ctr, kClaim);
-    int issued = 0, ending = 0;
-    for (int j = 0; ending < R::kConsumers; ++j) {
-        const int s = j % R::kStages;
-        unsigned i = nc;  // past the end: an end marker
-        if (j < js) {
-            i = blockIdx.x + (unsigned)j * gridDim.x;
-        } else if (claim) {
-            if (lane == 0) {
-                if (cur == cur_end) {
-                    cur = nxt;
-                    cur_end = nxt_end;
-                    if (nxt < nc) {  // the counter only grows: no more claims once past the end
-                        nxt = base + pend;
-                        nxt_end = nxt + pend_k;
-                        if (nxt < nc) {
-                            pend_k = nxt + kClaimTail * G >= nc ? 1u : kClaim;
-                            pend = claim_tiles(ctr, pend_k);
-                        }
-                    }
-                }
-                i = cur++;
-            }
-            i = __shfl_sync(kFull, i, 0);
-        }
-        if (j >= R::kStages) {
-            int w = 1;
-            if (lane == 0) w = mbar_wait(&empty[s], (uint32_t)((j / R::kStages - 1) & 1));
-            if (!__shfl_sync(kFull, w, 0)) {
-                if (lane == 0) report_timeout(sc);
-                break;
-            }
-        }
-        if (i >= nc) {  // one end marker per consumer warp
-            if (lane == 0) {
-                stage_tile[s] = -1;
-                mbar_arrive_tx(&full[s], 0u);
-            }
-            ++ending;
-            issued = j + 1;
-            continue;
-        }
-        const int c = (int)i;
-        const TilePos q = tc.at(tab, c, chunk, role, ns);
-        const uint32_t bytes = 16u * (uint32_t)tc.nv;
-        if (lane == 0) {
-            stage_tile[s] = c;
-            mbar_arrive_tx(&full[s], bytes * (uint32_t)ns);
+    // Barrier init; returns this warp's first tile (-1: none).  Called by the whole CTA.
+    __device__ __forceinline__ int start(unsigned char *smem, int n_tiles, unsigned *counter,
+                                         bool evict_first) {
+        const int warp = threadIdx.x >> 5;
+        stage = smem_addr(smem) + (uint32_t)warp * R::kStageBytes;
+        bar = reinterpret_cast<uint64_t *>(smem + R::kWarps * R::kStageBytes) + warp;
+        if ((threadIdx.x & 31) == 0) {
+            mbar_init(bar, 1);
+            mbar_fence_init();
         }
         __syncwarp();
-        if (bytes && lane < ns) {
-            const uint32_t dst = ring + (uint32_t)s * R::kStageBytes + (uint32_t)(lane * chunk * 4);
-            if (hint) bulk_g2s_hint(dst, tc.mine + q.begin, bytes, &full[s], policy);
-            else bulk_g2s(dst, tc.mine + q.begin, bytes, &full[s]);
-        }
-        issued = j + 1;
+        nc = (unsigned)n_tiles;
+        V = gridDim.x * (unsigned)R::kWarps;
+        claims = nc > V;
+        ctr = counter;
+        hint = evict_first;
+        policy = policy_evict_first();
+        if (claims && (threadIdx.x & 31) == 0) pend = atomicAdd(ctr, 1u);
+        const unsigned v = (unsigned)warp * gridDim.x + blockIdx.x;
+        return v < nc ? (int)v : -1;
     }
-    // Drain: never leave the CTA with a copy still writing into its shared memory.
-    if (lane == 0) {
-        for (int s = 0; s < R::kStages && s < issued; ++s) {
-            const int jl = s + ((issued - 1 - s) / R::kStages) * R::kStages;  // last tile on stage s
-            if (!mbar_wait(&full[s], (uint32_t)((jl / R::kStages) & 1))) report_timeout(sc);
+    // The tile after the last one taken (-1: none left).
+    __device__ __forceinline__ int next() {
+        if (!claims) return -1;
+        const unsigned c = __shfl_sync(kFull, pend, 0) + V;
+        if (c >= nc) return -1;
+        if ((threadIdx.x & 31) == 0) pend = atomicAdd(ctr, 1u);
+        return (int)c;
+    }
+    // Issues tile c; every lane has read what the stage held (a __syncwarp ago).
+    template <int NP>
+    __device__ __forceinline__ TilePos issue(const Table<NP> &tab, int c, int chunk, int role,
+                                             int ns) {
+        const int lane = threadIdx.x & 31;
+        const TilePos q = tc.at(tab, c, chunk, role, ns);
+        const uint32_t bytes = 16u * (uint32_t)tc.nv;
+        if (lane == 0) mbar_arrive_tx(bar, bytes * (uint32_t)ns);
+        __syncwarp();
+        if (bytes && lane < ns) {
+            const uint32_t dst = stage + (uint32_t)(lane * chunk * 4);
+            if (hint) bulk_g2s_hint(dst, tc.mine + q.begin, bytes, bar, policy);
+            else bulk_g2s(dst, tc.mine + q.begin, bytes, bar);
         }
-        // Every claim of this CTA is performed before it counts itself finished;
-        // the last CTA re-arms the counters for the next launch.
-        if (claim) {
+        return q;
+    }
+    // Waits for the tile in the stage.  false: the wait ran out (reported); the copies are then
+    // given as long again to land, so that the CTA does not end with them in flight, and the
+    // warp must stop.  The same in every lane.
+    __device__ __forceinline__ bool arrived(const Scalars &sc) {
+        const bool ok = __all_sync(kFull, mbar_wait(bar, phase));
+        if (!ok) {
+            if ((threadIdx.x & 31) == 0) report_timeout(sc);
+            mbar_wait(bar, phase);
+            claims = false;
+        }
+        phase ^= 1u;
+        return ok;
+    }
+    // After the warp's last tile: the last warp of the launch re-arms the counters.
+    __device__ __forceinline__ void finish() {
+        if (claims && (threadIdx.x & 31) == 0) {
             __threadfence();
-            if (atomicAdd(ctr + 1, 1u) == gridDim.x - 1u) {
+            if (atomicAdd(ctr + 1, 1u) == V - 1u) {
                 atomicExch(ctr, 0u);
                 atomicExch(ctr + 1, 0u);
             }
         }
     }
-}
-
-// Shared prologue of the streaming kernels: barrier init.
-template <typename R>
-__device__ __forceinline__ void ring_setup(unsigned char *smem, uint64_t *&full, uint64_t *&empty,
-                                           int *&stage_tile) {
-    full = reinterpret_cast<uint64_t *>(smem + R::kStages * R::kStageBytes);
-    empty = full + R::kStages;
-    stage_tile = reinterpret_cast<int *>(empty + R::kStages);
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < R::kStages; ++s) {
-            mbar_init(&full[s], 1);
-            mbar_init(&empty[s], 1);
-        }
-        mbar_fence_init();
-    }
-    __syncthreads();
-}
-
-// A consumer's wait for its j-th tile: the launch tile index, -1 when no tile
-// is left, -2 when the wait ran out (reported).  Called by the whole warp; the
-// result is the same in every lane (a lane whose bounded wait ran out makes
-// the warp stop), so the warp stays converged for its shuffles and votes.
-template <typename R>
-__device__ __forceinline__ int next_tile(const Scalars &sc, int j, uint64_t *full,
-                                         const int *stage_tile) {
-    const int s = j % R::kStages;
-    if (!__all_sync(kFull, mbar_wait(&full[s], (uint32_t)((j / R::kStages) & 1)))) {
-        if ((threadIdx.x & 31) == 0) report_timeout(sc);
-        return -2;
-    }
-    return *reinterpret_cast<const volatile int *>(stage_tile + s);
-}
+};
 
 // ----------------------------------------------------------------------------
 // Pass 1: replica mean + per-tile squared norms
@@ -1136,7 +1058,6 @@ template <int KT, bool WM, bool RW, bool SS, bool PR>
 __global__ void __launch_bounds__(Ring1Of<RW>::kThreads, 1)
     k_reduce(const __grid_constant__ Table<P1<KT>::NP> tab, const __grid_constant__ Scalars sc) {
     constexpr int KS = P1<KT>::KS;
-    constexpr int NSMAX = KS + 2;
     extern __shared__ __align__(128) unsigned char smem[];
     // In a step that does not read w, the first launch of the pass starts at
     // once.  It can only have been started early by the previous step's pass-2
@@ -1151,41 +1072,26 @@ __global__ void __launch_bounds__(Ring1Of<RW>::kThreads, 1)
     grid_launch_dependents();
     const bool early = !RW && !SS && sc.mode == kModeStep && tab.first;
     if (!early) grid_wait();
-    uint64_t *full, *empty;
-    int *stage_tile;
-    using R1 = Ring1Of<RW>;
-    ring_setup<R1>(smem, full, empty, stage_tile);
-    const int js = static_tiles(tab.nc);
-    const uint32_t ring = smem_addr(smem);
-    const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     const int K = KT > 0 ? KT : sc.K;
     const int chunk = tab.chunk;
-    int roles[NSMAX];
-    int ns = 0;
-    for (int k = 0; k < K; ++k) roles[ns++] = k;
-    if (RW) roles[ns++] = KS;
-    if (SS) roles[ns++] = KS + 1;
-    if (warp == 0) {
-        produce<R1, P1<KT>::NP, NSMAX>(tab, sc, roles, ns, chunk, js, sc.tiles, ring, full,
-                                          empty, stage_tile);
-        return;
-    }
-    const int my_role = lane < ns ? roles[lane] : 0;
-
-    const int cw = warp - 1;
-    TensorCache tc;
-    bool stop = false;
+    // Stage streams: replicas 0 .. K - 1, then w (RW), then g_small (SS).
+    const int ns = K + (RW ? 1 : 0) + (SS ? 1 : 0);
+    const int role = lane < K ? lane : (RW && lane == K ? KS : KS + 1);
+    Stream<Ring1Of<RW>> st;
+    int c = st.start(smem, tab.nc, sc.tiles, sc.evict_first != 0);
+    TilePos q = {};
+    if (c >= 0) q = st.issue(tab, c, chunk, role, ns);
     const bool step_g2 = sc.mode == kModeStep;  // |gbar|^2 also goes into |G|^2
     // The partial sums of a batch of kPend tiles are reduced across the warp together
     // (reduce-scatter, kRS values with padding) and added into the accumulators by the lanes
     // that own them.
     constexpr int kRS = 16;
     static_assert(kPend * kAcc <= kRS, "one reduce-scatter per batch");
-    for (int jb = cw; !stop; jb += R1::kConsumers * kPend) {
+    while (c >= 0) {
         // PR: the lanes' fp64 sums.  Default: fp32 sums of the shared-memory columns, scaled by
         // 2^(2e) with e coded in two bits per value in `ecode` (same in every lane); a tile with
-        // elements loaded one by one (fp64, rare) is stored at once instead (store_tile_now).
+        // elements loaded one by one (fp64, rare) is stored at once instead (add_tile_now).
         double pendd[PR ? kRS : 1];
         float pendf[PR ? 1 : kRS];
         unsigned ecode = 0u;
@@ -1196,46 +1102,43 @@ __global__ void __launch_bounds__(Ring1Of<RW>::kThreads, 1)
             else pendf[i] = 0.f;
         }
 #pragma unroll
-        for (int p = 0; p < kPend; ++p) {
-            const int j = jb + p * R1::kConsumers;
-            ptensor[p] = -1;
-            if (stop) continue;
-            // A round-robin tile is located before its wait, a claimed one after.
-            int c = j < js ? static_tile(j) : -1;
-            TilePos q;
-            if (c >= 0) q = tc.at(tab, c, chunk, my_role, ns);
-            const int got = next_tile<R1>(sc, j, full, stage_tile);
-            if (got < 0) {
-                stop = true;
-                continue;
+        for (int p = 0; p < kPend; ++p) ptensor[p] = -1;
+        // One copy of the tile's code for the whole batch: the sums go to their places by
+        // predicated moves.
+#pragma unroll 1
+        for (int p = 0; p < kPend && c >= 0; ++p) {
+            if (!st.arrived(sc)) {
+                c = -1;
+                break;
             }
-            if (c < 0) {
-                c = got;
-                q = tc.at(tab, c, chunk, my_role, ns);
-            }
-            const int s = j % R1::kStages;
             const float *const *ptr = tab.ptr[q.t];
             double accd[kAcc];
             float accf[kAcc];
             int acce[kAcc];
             unsigned tcode;
             bool tile_tail;
-            reduce_tile<KT, WM, RW, SS, PR>(ring + (uint32_t)s * R1::kStageBytes, chunk, ptr, q,
-                                            tc.nv, sc, accd, accf, acce, tcode, tile_tail);
+            reduce_tile<KT, WM, RW, SS, PR>(st.stage, chunk, ptr, q, st.tc.nv, sc, accd, accf, acce,
+                                            tcode, tile_tail);
             __syncwarp();
-            if (lane == 0) mbar_arrive(&empty[s]);
-            if constexpr (PR) {
-                ptensor[p] = q.tg;
-#pragma unroll
-                for (int a = 0; a < kAcc; ++a) pendd[p * kAcc + a] = accd[a];
-            } else if (tile_tail) {
-                add_tile_now(sc, q.tg, accf, acce, accd);
-            } else {
-                ptensor[p] = q.tg;
-#pragma unroll
-                for (int a = 0; a < kAcc; ++a) pendf[p * kAcc + a] = accf[a];
-                ecode |= tcode << (2 * kAcc * p);
+            const int tg = q.tg;
+            c = st.next();
+            if (c >= 0) q = st.issue(tab, c, chunk, role, ns);
+            if (!PR && tile_tail) {
+                add_tile_now(sc, tg, accf, acce, accd);
+                continue;
             }
+#pragma unroll
+            for (int i = 0; i < kPend; ++i) {
+                if (p == i) {
+                    ptensor[i] = tg;
+#pragma unroll
+                    for (int a = 0; a < kAcc; ++a) {
+                        if constexpr (PR) pendd[i * kAcc + a] = accd[a];
+                        else pendf[i * kAcc + a] = accf[a];
+                    }
+                }
+            }
+            if constexpr (!PR) ecode |= tcode << (2 * kAcc * p);
         }
         int idx;
         double vd = 0.0;
@@ -1258,9 +1161,9 @@ __global__ void __launch_bounds__(Ring1Of<RW>::kThreads, 1)
                 }
             }
         }
-        if (stop) break;
     }
-    if (early && threadIdx.x == 32) grid_wait();  // see the top of the kernel
+    st.finish();
+    if (early && threadIdx.x == 0) grid_wait();  // see the top of the kernel
 }
 
 // ----------------------------------------------------------------------------
@@ -1587,75 +1490,54 @@ __global__ void __launch_bounds__(Ring2::kThreads, 1)
     if (sc.fin2) grid_launch_dependents();
     const bool early = !PE && tab.first;
     if (!early) grid_wait();
-    uint64_t *full, *empty;
-    int *stage_tile;
-    ring_setup<Ring2>(smem, full, empty, stage_tile);
-    const int js = static_tiles(tab.nc);
-    const uint32_t ring = smem_addr(smem);
-    const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     const int chunk = tab.chunk;
-    int roles[4] = {0, 1, 2, 3};
-    if (!HM) roles[2] = 3;
-    if (warp == 0) {
-        const bool se = PE && sc.flags[0];
-        produce<Ring2, kNP2, 4>(tab, sc, roles, 2 + (HM ? 1 : 0) + (se ? 1 : 0), chunk, js,
-                                sc.tiles + 2, ring, full, empty, stage_tile);
-        return;
-    }
-    if (early) grid_wait();
-    const int scaled = sc.flags[0];
-    const bool gated = sc.rule == TULA_RULE_AGS || sc.rule == TULA_RULE_STATIC;
-    const bool use_se = PE && scaled;
+    const bool use_se = PE && sc.flags[0];  // PE: after the wait above
     const int ns = 2 + (HM ? 1 : 0) + (use_se ? 1 : 0);
-    const int my_role = lane < ns ? roles[lane] : 0;
+    const int role = !HM && lane == 2 ? 3 : (lane < 4 ? lane : 0);
     constexpr int CH = Ring2::tile_elems(2 + (HM ? 1 : 0) + (PE ? 1 : 0));
     constexpr int COLS = CH / 128;
     const uint32_t w_off = (uint32_t)(CH * 4);
     const uint32_t m_off = (uint32_t)(2 * CH * 4);
     const uint32_t se_off = (uint32_t)((HM ? 3 : 2) * CH * 4);
+    Stream<Ring2> st;
+    int c = st.start(smem, tab.nc, sc.tiles + 2, sc.evict_first != 0);
+    TilePos q = {};
+    if (c >= 0) q = st.issue(tab, c, chunk, role, ns);
+    if (early) grid_wait();
+    const int scaled = sc.flags[0];
+    const bool gated = sc.rule == TULA_RULE_AGS || sc.rule == TULA_RULE_STATIC;
+    const uint32_t stage = st.stage;
 
-    TensorCache tc;
-    const int cw = warp - 1;
     int cand_t = -1;
     float cand = 0.f;
-    bool stop = false;
-    for (int jb = cw; !stop; jb += Ring2::kConsumers * kPend) {
+    while (c >= 0) {
         // fp32 |w|^2 of the tiles' shared-memory columns, scaled by 2^(2e) (e coded in `ecode`);
         // a tile with elements loaded one by one (fp64, rare) is stored at once instead.
         float pend[kPend];
         unsigned ecode = 0u;
         int ptensor[kPend];  // global index of each pending tile's tensor, -1: none
 #pragma unroll
-        for (int p = 0; p < kPend; ++p) {
-            const int j = jb + p * Ring2::kConsumers;
-            ptensor[p] = -1;
-            pend[p] = 0.f;
-            if (stop) continue;
-            int c = j < js ? static_tile(j) : -1;
-            TilePos q;
-            if (c >= 0) q = tc.at(tab, c, chunk, my_role, ns);
-            const int got = next_tile<Ring2>(sc, j, full, stage_tile);
-            if (got < 0) {
-                stop = true;
-                continue;
-            }
-            if (c < 0) {
-                c = got;
-                q = tc.at(tab, c, chunk, my_role, ns);
-            }
-            const int s = j % Ring2::kStages;
-            const float *const *ptr = tab.ptr[q.t];
-            const int nv = tc.nv;
+        for (int i = 0; i < kPend; ++i) {
+            ptensor[i] = -1;
+            pend[i] = 0.f;
+        }
+#pragma unroll 1
+        for (int p = 0; p < kPend && c >= 0; ++p) {
             if (q.tg != cand_t) {  // c_p changes only with the tensor
                 cand = sc.cand[q.tg];
                 cand_t = q.tg;
             }
+            if (!st.arrived(sc)) {
+                c = -1;
+                break;
+            }
+            const float *const *ptr = tab.ptr[q.t];
+            const int nv = st.tc.nv;
             const float ct = gated ? (scaled ? cand : 1.0f) : cand;
             if (sc.stats && q.c_in_t == 0 && lane == 0)
                 sc.stats[(size_t)q.tg * TULA_STATS_LEN + TULA_STAT_COEF] =
                     PE ? (scaled ? (double)NAN : 1.0) : (double)ct;
-            const uint32_t stage = ring + (uint32_t)s * Ring2::kStageBytes;
             float *wp = const_cast<float *>(ptr[1]) + q.begin;
             float *mp = HM ? const_cast<float *>(ptr[2]) + q.begin : nullptr;
             const float4 cdef = PE ? make_float4(1.f, 1.f, 1.f, 1.f) : make_float4(ct, ct, ct, ct);
@@ -1704,7 +1586,6 @@ __global__ void __launch_bounds__(Ring2::kThreads, 1)
                 if (ew) aw = w_cols_scaled(stage + w_off, nv, pow2f(ew));
             }
             __syncwarp();
-            if (lane == 0) mbar_arrive(&empty[s]);
             const long long n = q.end - q.begin;
             const bool tile_tail = 4 * (long long)nv < n;  // the same in every lane
             for (long long jj = 4 * (long long)nv + lane; jj < n; jj += 32) {
@@ -1717,12 +1598,20 @@ __global__ void __launch_bounds__(Ring2::kThreads, 1)
                 wp[jj] = w;
                 if (HM) mp[jj] = m;
             }
+            const int tg = q.tg;
+            c = st.next();
+            if (c >= 0) q = st.issue(tab, c, chunk, role, ns);
             if (SW) {
                 if (tile_tail) {
-                    add_w_tile_now(acc2_of(sc, q.tg), aw, ew, awt);
+                    add_w_tile_now(acc2_of(sc, tg), aw, ew, awt);
                 } else {
-                    ptensor[p] = q.tg;
-                    pend[p] = aw;
+#pragma unroll
+                    for (int i = 0; i < kPend; ++i) {
+                        if (p == i) {
+                            ptensor[i] = tg;
+                            pend[i] = aw;
+                        }
+                    }
                     if (ew) ecode |= scale_code(ew) << (2 * p);
                 }
             }
@@ -1738,8 +1627,8 @@ __global__ void __launch_bounds__(Ring2::kThreads, 1)
                                 -2 * scale_exp((ecode >> (2 * idx)) & 3u));
             }
         }
-        if (stop) break;
     }
+    st.finish();
 }
 
 // ----------------------------------------------------------------------------
