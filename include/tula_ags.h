@@ -139,10 +139,10 @@ typedef struct tula_ags_hparams {
                                      not depend on it) */
     void *trace_events[5];        /* optional cudaEvent_t (NULL = none), recorded on `stream`:
                                      [0] before the reduction kernel(s), [1] after them,
-                                     [2] after the pass-1 finish (before the update kernel),
+                                     [2] before the update kernel (after LARS's coefficients),
                                      [3] after the update kernel(s), [4] the end of the step
-                                     (after the finish that follows the update, when the step
-                                     has statistics or refreshes the gradscale).  A recorded
+                                     (after the kernel that finishes the norms, the statistics
+                                     and the step record).  A recorded
                                      event keeps the next kernel from starting early, so steps
                                      that record events run slightly slower. */
 } tula_ags_hparams;

@@ -1,6 +1,6 @@
 // libtula_ags: the AGS optimizer step (Tula, arXiv 2603.18112) for sm_103a.
 //
-// Per step, four kernels on the caller's stream, chained by programmatic
+// Per step, three kernels on the caller's stream, chained by programmatic
 // dependent launch so that each one's launch and prologue overlap the tail of
 // the one before:
 //
@@ -8,28 +8,27 @@
 //                        tile's sums of |gbar|^2, |g_0|^2 [, |w|^2] are added
 //                        exactly into per-tensor accumulators (and |gbar|^2 into
 //                        the step's |G|^2 accumulator) by L2 atomics.
+//   k_update   (pass 2)  the branch of Algorithm 1 from |G|^2 (Eq. 5), then
+//                        d = c gbar + wd w; m = mu m + d; w = w - lr m (Eq. 7b with
+//                        the wrapped SGD); |w|^2 per tile for the statistics.
 //   k_finish             per tensor, the norms rounded from its accumulators, its
-//                        statistics, its coefficient when scaled (the old
-//                        gradscale, Eq. 8's s, or the LARS ratio) and, when
-//                        asked, the refreshed gradscale (UpdateGradScale,
-//                        Algorithm 1); one more warp forms |G|^2, Delta (Eq. 5)
-//                        and the branch of Algorithm 1.
-//   k_update   (pass 2)  d = c gbar + wd w; m = mu m + d; w = w - lr m (Eq. 7b with
-//                        the wrapped SGD); |w|^2 per tile for the statistics,
-//   k_finish             then rounded per tensor.
+//                        statistics and, when asked, the refreshed gradscale
+//                        (UpdateGradScale, Algorithm 1); one more warp writes the
+//                        step record (|G|^2, Delta, the branch).
+//
+// A LARS step has k_lars between the passes: its coefficients are ratios of this
+// step's norms.
 //
 // The streaming passes: each tensor is cut into tiles of T elements (T fixed
 // per pass by how many tensors it streams, so that one tile of every stream
 // fills one shared-memory stage: 36 KB in pass 1, 24 KB in pass 2).  One
-// persistent CTA per SM; small launches deal tiles round-robin, larger ones
-// claim them from a global counter (SMs stream at unequal rates).  The producer
-// warp moves tiles from HBM into the stage ring with TMA bulk copies
-// (cp.async.bulk ... mbarrier::complete_tx), one copy per stream issued by one
-// lane each; consumer warps, each owning whole stages, compute from shared
-// memory and release the stage through an mbarrier.  Tile partials are fp32
-// sums within a tile (float-float pairs per lane in the precise mode for norms
-// that feed a coefficient), range-checked per tile, and leave the tile only as
-// exact integer additions into the accumulators.
+// persistent CTA per SM, whose warps each stream tiles through a stage of their
+// own with TMA bulk copies (cp.async.bulk ... mbarrier::complete_tx), one copy per
+// stream issued by one lane each, and claim tiles from a global counter (SMs
+// stream at unequal rates).  Tile partials are fp32 sums within a tile
+// (float-float pairs per lane in the precise mode for norms that feed a
+// coefficient), range-checked per tile, and leave the tile only as exact integer
+// additions into the accumulators.
 //
 // Every mbarrier wait is bounded; a wait that runs out sets an error word in
 // the workspace (tula_ags_workspace_error) and the CTA drains its copies in
@@ -86,11 +85,11 @@ constexpr int kFinWarps = 4;            // k_finish: one warp per tensor, 4 per 
 constexpr int kParamBudget = 31 * 1024; // kernel parameter bytes per launch (limit 32764)
 constexpr int kAcc = 3;                 // partial sums per pass-1 tile: |gbar|^2, |g_0|^2, |w|^2
 constexpr int kPrecCols = 1;            // float4 columns per step of the precise path's tile loop
-constexpr int kTsum = 4;                // per-tensor sums (stride)
+constexpr int kSpare = 32;              // unused bytes per tensor in the workspace's layout
 constexpr unsigned kFull = 0xffffffffu;
 constexpr uint32_t kSpinLimit = 1u << 19;  // bound on every mbarrier wait (~2 s on GB300)
 
-enum Mode { kModeStep = 0, kModeStats = 1, kModeScale = 2, kModeUpdate = 3 };
+enum Mode { kModeStep = 0, kModeStats = 1, kModeScale = 2 };
 
 
 // ----------------------------------------------------------------------------
@@ -114,19 +113,17 @@ struct Table {
 
 struct Scalars {
     int K, rule, gran, force, refresh, mode, n_total, read_w;
-    int pow2K, evict_first, fin2, pad2;  // evict_first: TMA loads ask L2 to drop their lines first;
-                                         // fin2: a finish kernel follows the update
+    int pow2K, evict_first, early_w, pad2;  // evict_first: TMA loads ask L2 to drop their lines
+                                            // first; early_w: the update follows this call's pass 1
     float delta, eps, s_max, static_s, lars_trust, lr, mu, wd, invK, Kf;
     float *scale;
     double *state;
     double *stats;
-    int *flags;                // [0]: branch of the last step (1 = scaled)
     unsigned *err;             // [0]: bounded waits that ran out (sticky until read)
     unsigned long long *acc1;  // [tensor][kAcc][kTCopies][kAccWords]: |gbar|^2, |g_0|^2, |w|^2
     unsigned long long *gacc;  // [kGCopies][kAccWords]: |G|^2 = every tensor's |gbar|^2
     unsigned long long *acc2;  // [tensor][kTCopies][kAccWords]: |w|^2, pass 2
-    double *tsum;              // [tensor][kTsum]: |gbar|^2, |g_0|^2, |w|^2
-    float *cand;               // [tensor]: c_p of the scaled branch (AGS: the old gradscale)
+    float *cand;               // [tensor]: c_p of a LARS step
     unsigned *tiles;           // [2 * pass]: next tile to claim, [2 * pass + 1]: CTAs finished
     const unsigned long long *g2ext;  // a sharded step's |G|^2: the ranks' shares summed (or NULL)
 };
@@ -700,21 +697,29 @@ struct Stream {
         if ((threadIdx.x & 31) == 0) pend = atomicAdd(ctr, 1u);
         return (int)c;
     }
-    // Issues tile c; every lane has read what the stage held (a __syncwarp ago).
+    // Issues tile c, or of it only streams `from` .. ns - 1, the rest left to issue_below();
+    // every lane has read what the stage held (a __syncwarp ago).
     template <int NP>
     __device__ __forceinline__ TilePos issue(const Table<NP> &tab, int c, int chunk, int role,
-                                             int ns) {
+                                             int ns, int from = 0) {
         const int lane = threadIdx.x & 31;
         const TilePos q = tc.at(tab, c, chunk, role, ns);
-        const uint32_t bytes = 16u * (uint32_t)tc.nv;
-        if (lane == 0) mbar_arrive_tx(bar, bytes * (uint32_t)ns);
+        if (lane == 0) mbar_arrive_tx(bar, 16u * (uint32_t)(tc.nv * ns));
         __syncwarp();
-        if (bytes && lane < ns) {
+        if (lane >= from && lane < ns) copy(q, lane, chunk);
+        return q;
+    }
+    __device__ __forceinline__ void issue_below(const TilePos &q, int from, int chunk) {
+        const int lane = threadIdx.x & 31;
+        if (lane < from) copy(q, lane, chunk);
+    }
+    __device__ __forceinline__ void copy(const TilePos &q, int lane, int chunk) {
+        const uint32_t bytes = 16u * (uint32_t)tc.nv;
+        if (bytes) {
             const uint32_t dst = stage + (uint32_t)(lane * chunk * 4);
             if (hint) bulk_g2s_hint(dst, tc.mine + q.begin, bytes, bar, policy);
             else bulk_g2s(dst, tc.mine + q.begin, bytes, bar);
         }
-        return q;
     }
     // Waits for the tile in the stage.  false: the wait ran out (reported); the copies are then
     // given as long again to land, so that the CTA does not end with them in flight, and the
@@ -1059,19 +1064,16 @@ __global__ void __launch_bounds__(Ring1Of<RW>::kThreads, 1)
     k_reduce(const __grid_constant__ Table<P1<KT>::NP> tab, const __grid_constant__ Scalars sc) {
     constexpr int KS = P1<KT>::KS;
     extern __shared__ __align__(128) unsigned char smem[];
-    // In a step that does not read w, the first launch of the pass starts at
-    // once.  It can only have been started early by the previous step's pass-2
-    // finish (the update triggers its successor only when that finish
-    // follows), and that finish starts it after its own wait, i.e. once the
-    // previous update has completed (and, before it, the pass-1 finish that
-    // re-armed the pass-1 accumulators): nothing still running then reads the
-    // replicas or the pass-1 accumulators this kernel adds into, and nothing
-    // writes what it loads.  The running finish reads the per-tensor sums the
-    // next pass-1 finish writes, so this kernel does not complete before it
-    // (one wait per CTA at the end).  Otherwise the whole CTA waits first.
-    grid_launch_dependents();
+    // The first launch of a step's pass that does not read w issues its first tiles at once: the
+    // only kernel that lets it start early is the previous call's k_finish, once all before that
+    // one had completed.  What it writes, the mean and the accumulators, waits for k_finish, which
+    // reads the accumulators.  Otherwise the whole CTA waits first.  The next kernel may start when
+    // that wait has passed.
     const bool early = !RW && !SS && sc.mode == kModeStep && tab.first;
-    if (!early) grid_wait();
+    if (!early) {
+        grid_wait();
+        grid_launch_dependents();
+    }
     const int lane = threadIdx.x & 31;
     const int K = KT > 0 ? KT : sc.K;
     const int chunk = tab.chunk;
@@ -1082,6 +1084,10 @@ __global__ void __launch_bounds__(Ring1Of<RW>::kThreads, 1)
     int c = st.start(smem, tab.nc, sc.tiles, sc.evict_first != 0);
     TilePos q = {};
     if (c >= 0) q = st.issue(tab, c, chunk, role, ns);
+    if (early) {
+        grid_wait();
+        grid_launch_dependents();
+    }
     const bool step_g2 = sc.mode == kModeStep;  // |gbar|^2 also goes into |G|^2
     // The partial sums of a batch of kPend tiles are reduced across the warp together
     // (reduce-scatter, kRS values with padding) and added into the accumulators by the lanes
@@ -1163,7 +1169,6 @@ __global__ void __launch_bounds__(Ring1Of<RW>::kThreads, 1)
         }
     }
     st.finish();
-    if (early && threadIdx.x == 0) grid_wait();  // see the top of the kernel
 }
 
 // ----------------------------------------------------------------------------
@@ -1171,10 +1176,16 @@ __global__ void __launch_bounds__(Ring1Of<RW>::kThreads, 1)
 // ----------------------------------------------------------------------------
 //
 // One warp per tensor reads its accumulators (one word per lane), rounds them to fp64
-// (acc_to_double), puts them back to zero for the next call and finishes the tensor: after
-// pass 1 its statistics and coefficient (tensor_done), after pass 2 |w|^2 for the statistics.
-// After pass 1 of a step, one more warp forms |G|^2 from the global accumulator, then Delta
-// (Eq. 5) and the branch of Algorithm 1 (finalize_step).  No warp waits for another.
+// (acc_to_double), puts them back to zero for the next call and writes the tensor's results: the
+// last kernel of a step (statistics, UpdateGradScale), of tula_layer_stats and of a per-tensor
+// tula_ags_update_scale.  In a step, one more warp forms |G|^2 from the global accumulator, then
+// Delta (Eq. 5) and the branch of Algorithm 1 for the step record; the update has taken the same
+// branch from the same accumulator (step_branch).  No warp waits for another.
+//
+// Everything here used to stand between the passes, in a kernel of its own.  The update then
+// waited for it: 9.9 us from the end of the reduction to the update's first tile on ResNet-50,
+// 3.7 of them the record's fp64 division.  Only LARS, whose coefficients are ratios of this
+// step's norms, still has a kernel there (k_lars).
 
 // The square roots of three norms (lanes 0-2 in one fp64 sequence) and the two ratios of a
 // tensor (lanes 0 and 1): UpdateGradScale's |g_s| / (|g_l| + eps) and |w| / |gbar| (LARS, the
@@ -1196,83 +1207,6 @@ __device__ __forceinline__ Norms tensor_norms(const Scalars &sc, double sg, doub
     return o;
 }
 
-// The statistics row of a tensor from its squared norms (sw: |w|^2 before the update).
-__device__ __forceinline__ void stats_row(double *row, double sg, double ss, double sw,
-                                          const Norms &o) {
-    row[TULA_STAT_W_SQ] = sw;
-    row[TULA_STAT_G_SQ] = sg;
-    row[TULA_STAT_G0_SQ] = ss;
-    row[TULA_STAT_W_NORM] = o.nw;
-    row[TULA_STAT_G_NORM] = o.ng;
-    row[TULA_STAT_RATIO] = sg > 0.0 ? o.q_w : 0.0;
-}
-
-// Per-tensor results after pass 1, by the whole warp holding the tensor's norms.
-// tula_layer_stats and tula_ags_update_scale: everything here.  A step: what the update needs
-// (the coefficient c_p) and the norms, kept in tsum with the old gradscale; the square roots,
-// the statistics and UpdateGradScale follow the update (tensor_after_update), off the path
-// between the passes, except for LARS, whose coefficient is a ratio of norms.
-__device__ void tensor_done(const Scalars &sc, int tg, double sg, double ss, double sw, float old) {
-    const int lane = threadIdx.x & 31;
-    if (sc.mode == kModeScale || sc.mode == kModeStats || sc.rule == TULA_RULE_LARS) {
-        const Norms o = tensor_norms(sc, sg, ss, sw);
-        if (lane != 0) return;
-        if (sc.mode == kModeScale) {
-            // UpdateGradScale, g_0 = g_large, small = g_small: min(|g_s| / (|g_l| + eps), s_max)
-            sc.scale[tg] = (float)fmin(o.q_scale, (double)sc.s_max);
-            return;
-        }
-        if (sc.mode == kModeStats) {
-            double *row = sc.stats + (size_t)tg * TULA_STATS_LEN;
-            stats_row(row, sg, ss, sw, o);
-            row[TULA_STAT_COEF] = 0.0;
-            row[TULA_STAT_SCALE] = 0.0;
-            return;
-        }
-        // LARS (Sec. V-B): c_p = trust * |w| / |gbar|, every step (1 when either norm is 0)
-        sc.cand[tg] = (sw > 0.0 && sg > 0.0) ? (float)((double)sc.lars_trust * o.q_w) : 1.0f;
-    } else if (lane == 0) {
-        // the coefficient this tensor gets when the step is scaled (Algorithm 1, Eq. 8), before
-        // UpdateGradScale may overwrite gradscale
-        sc.cand[tg] = sc.rule == TULA_RULE_AGS ? old
-                      : (sc.rule == TULA_RULE_STATIC ? sc.static_s : 1.0f);
-    }
-    if (lane != 0) return;
-    double *T = sc.tsum + (size_t)tg * kTsum;
-    T[0] = sg;
-    T[1] = ss;
-    T[2] = sw;
-    T[3] = (double)old;
-}
-
-// After the update of a step: the statistics row and UpdateGradScale of tensor t, from the
-// pass-1 norms kept in tsum and, when the update took it, |w|^2 from pass 2 (sw2).
-__device__ void tensor_after_update(const Scalars &sc, int t, double sw2, bool have_sw2) {
-    const int lane = threadIdx.x & 31;
-    const double *T = sc.tsum + (size_t)t * kTsum;
-    const double sg = T[0], ss = T[1], sw = have_sw2 ? sw2 : T[2];
-    const float old = (float)T[3];
-    const Norms o = tensor_norms(sc, sg, ss, sw);
-    if (lane != 0) return;
-    float s_after = sc.scale ? old : 0.0f;
-    if (sc.refresh && sc.scale) {
-        // UpdateGradScale with g_small = replica 0 and g_large = the mean
-        s_after = (float)fmin(o.q_scale, (double)sc.s_max);
-        sc.scale[t] = s_after;
-    }
-    if (sc.stats) {
-        double *row = sc.stats + (size_t)t * TULA_STATS_LEN;
-        if (have_sw2 || sc.read_w) {
-            stats_row(row, sg, ss, sw, o);
-        } else {
-            row[TULA_STAT_G_SQ] = sg;
-            row[TULA_STAT_G0_SQ] = ss;
-            row[TULA_STAT_G_NORM] = o.ng;
-        }
-        row[TULA_STAT_SCALE] = (double)s_after;
-    }
-}
-
 // Delta (Eq. 5): this step's |G|^2 against the last step's, +inf at the first step (no previous
 // norm; the step is then unscaled, the sensitive phase).
 __device__ __forceinline__ double variability(double g2, double g2_prev, double steps) {
@@ -1284,6 +1218,23 @@ __device__ __forceinline__ int branch_of(const Scalars &sc, double dv) {
     if (sc.force == TULA_BRANCH_UNSCALED) return 0;
     return dv < (double)sc.delta;
 }
+// The same branch without waiting for Eq. 5's fp64 division (1.8-3.7 us on GB300) unless it is
+// close: with d = |g2 - g2_prev| as rounded and t = fl(delta * g2_prev), both far from underflow,
+// d < t (1 - 2^-49) puts the exact quotient d / g2_prev below delta (1 - 2^-50) (t and the product
+// err by 2^-53 each), so its rounding is below delta, and d > t (1 + 2^-49) puts it above.  NaN,
+// infinite and zero norms fail both tests and divide.
+__device__ __forceinline__ int branch_from(const Scalars &sc, double g2, double g2_prev,
+                                           double steps) {
+    if (sc.force == TULA_BRANCH_AUTO && steps != 0.0) {
+        const double t = __dmul_rn((double)sc.delta, g2_prev);
+        const double d = fabs(__dsub_rn(g2, g2_prev));
+        if (t > 0x1p-900 && t < 0x1p900) {
+            if (d < __dmul_rn(t, 1.0 - 0x1p-49)) return 1;
+            if (d > __dmul_rn(t, 1.0 + 0x1p-49) && d < 0x1p1000) return 0;
+        }
+    }
+    return branch_of(sc, variability(g2, g2_prev, steps));
+}
 // The step record from this step's |G|^2 (one lane).
 __device__ void finalize_step(const Scalars &sc, double g2, double g2_prev, double steps) {
     const double dv = variability(g2, g2_prev, steps);
@@ -1292,7 +1243,6 @@ __device__ void finalize_step(const Scalars &sc, double g2, double g2_prev, doub
     sc.state[TULA_STATE_STEPS] = steps + 1.0;
     sc.state[TULA_STATE_DELTA] = dv;
     sc.state[TULA_STATE_SCALED] = (double)scaled;
-    sc.flags[0] = scaled;
 }
 
 // This lane's word of the sum of R accumulators' Copies copies each (A[r] the first copy of
@@ -1366,53 +1316,83 @@ __global__ void __launch_bounds__(32) k_share(const __grid_constant__ Scalars sc
     else if (lane < kAccWords) share[lane] = 0ull;
 }
 
-// NA = kAcc: after pass 1 (the pass-1 norms; in a step also the branch, which the update then
-// reads).  NA = 1: after the update of a step (its statistics and UpdateGradScale, with |w|^2
-// from pass 2 when the update took it).
-template <int NA>
+// The step's |G|^2, by the whole warp: from the ranks' shares in a sharded step.
+__device__ __forceinline__ double step_g2_of(const Scalars &sc, bool rearm) {
+    return sc.g2ext ? share_to_double(sc.g2ext) : acc_read<kGCopies>(sc.gacc, rearm);
+}
+// The branch of this step for the update, by one warp, once the reduction has completed.
+__device__ __forceinline__ int step_branch(const Scalars &sc) {
+    const double g2_prev = sc.state[TULA_STATE_G2_PREV], steps = sc.state[TULA_STATE_STEPS];
+    return branch_from(sc, step_g2_of(sc, false), g2_prev, steps);
+}
+
+// LARS (Sec. V-B), between the passes: c_p = trust * |w| / |gbar|, every step (1 when either norm
+// is 0).  One warp per tensor; the accumulators stay as they are for k_finish.
+__global__ void __launch_bounds__(32 * kFinWarps) k_lars(const __grid_constant__ Scalars sc) {
+    const int lane = threadIdx.x & 31;
+    const int t = (int)blockIdx.x * kFinWarps + (int)(threadIdx.x >> 5);
+    grid_launch_dependents();  // the update's first w and m (see k_update)
+    grid_wait();
+    if (t >= sc.n_total) return;
+    unsigned long long *A = sc.acc1 + (size_t)t * kAcc * kTCopies * kAccWords;
+    unsigned long long *const a[2] = {A, A + 2 * kTCopies * kAccWords};
+    unsigned long long w[2];
+    acc_words<2, kTCopies>(a, false, w);
+    double v[2];
+    acc_to_double<2>(w, v);
+    const Norms o = tensor_norms(sc, v[0], 0.0, v[1]);
+    if (lane == 0)
+        sc.cand[t] = (v[1] > 0.0 && v[0] > 0.0) ? (float)((double)sc.lars_trust * o.q_w) : 1.0f;
+}
+
 __global__ void __launch_bounds__(32 * kFinWarps) k_finish(const __grid_constant__ Scalars sc) {
-    constexpr bool P1 = NA == kAcc;  // pass-1 accumulators
     const int lane = threadIdx.x & 31;
     const int t = (int)blockIdx.x * kFinWarps + (int)(threadIdx.x >> 5);
     const int n = sc.n_total;
-    const bool step = P1 && sc.mode == kModeStep;
-    const bool active = t < n + (step ? 1 : 0);
-    // This kernel is launched early and waits here for the kernel before it; the old gradscale
-    // and the step record are read after the wait, together with the accumulators (no round
-    // trip is added, and no kernel of an earlier call can still be writing them).
+    const bool step = sc.mode == kModeStep;
     grid_wait();
-    // Inside a step the successor (the update, or the next step's reduction) may start now;
-    // after tula_layer_stats or tula_ags_update_scale it starts when this kernel has completed
-    // (a step's reduction that starts early adds into the accumulators this kernel reads).
-    if (sc.mode == kModeStep || NA == 1) grid_launch_dependents();
-    if (!active) return;
-    const float scale_old = (t < n && step && sc.scale) ? sc.scale[t] : 1.0f;
-    const double g2_prev = step ? sc.state[TULA_STATE_G2_PREV] : 0.0;
-    const double steps = step ? sc.state[TULA_STATE_STEPS] : 0.0;
-    if (t == n) {  // the record and the branch
-        double g2;
-        if (sc.g2ext) {
-            g2 = share_to_double(sc.g2ext);
-        } else {
-            g2 = acc_read<kGCopies>(sc.gacc, true);
-        }
+    // The next call's reduction may start now: it only reads replicas until this kernel has
+    // completed.
+    grid_launch_dependents();
+    if (t > n || (t == n && !step)) return;
+    if (t == n) {  // the step record
+        const double g2_prev = sc.state[TULA_STATE_G2_PREV], steps = sc.state[TULA_STATE_STEPS];
+        const double g2 = step_g2_of(sc, true);
         if (lane == 0) finalize_step(sc, g2, g2_prev, steps);
         return;
     }
     unsigned long long *A1 = sc.acc1 + (size_t)t * kAcc * kTCopies * kAccWords;
     unsigned long long *A2 = sc.acc2 + (size_t)t * kTCopies * kAccWords;
-    if constexpr (NA == kAcc) {
-        unsigned long long *const a[kAcc] = {A1, A1 + kTCopies * kAccWords,
-                                             A1 + 2 * kTCopies * kAccWords};
-        unsigned long long w[kAcc];
-        acc_words<kAcc, kTCopies>(a, true, w);
-        double v[kAcc];
-        acc_to_double<kAcc>(w, v);
-        tensor_done(sc, t, v[0], v[1], v[2], scale_old);
-    } else {
-        const bool have_sw2 = sc.stats && !sc.read_w;  // the update's |w|^2 (k_update<..., SW>)
-        const double sw2 = have_sw2 ? acc_read<kTCopies>(A2, true) : 0.0;
-        tensor_after_update(sc, t, sw2, have_sw2);
+    // |w|^2 before the update comes from pass 1 when that read w, else from the update's own tiles.
+    const bool have_sw2 = step && sc.stats && !sc.read_w;
+    const float old = (step && sc.scale) ? sc.scale[t] : 0.0f;
+    unsigned long long *const a[kAcc] = {A1, A1 + kTCopies * kAccWords,
+                                         have_sw2 ? A2 : A1 + 2 * kTCopies * kAccWords};
+    unsigned long long w[kAcc];
+    acc_words<kAcc, kTCopies>(a, true, w);
+    if (step && !sc.stats && !sc.refresh) return;  // re-armed, and nobody asks for the norms
+    double v[kAcc];
+    acc_to_double<kAcc>(w, v);
+    const double sg = v[0], ss = v[1], sw = v[2];
+    const Norms o = tensor_norms(sc, sg, ss, sw);
+    if (lane != 0) return;
+    float s_after = old;
+    if (sc.mode == kModeScale || (step && sc.refresh && sc.scale)) {
+        // UpdateGradScale: min(|g_small| / (|g_large| + eps), s_max); in a step g_small is replica
+        // 0 and g_large the mean
+        s_after = (float)fmin(o.q_scale, (double)sc.s_max);
+        sc.scale[t] = s_after;
+    }
+    if (sc.stats) {
+        double *row = sc.stats + (size_t)t * TULA_STATS_LEN;
+        row[TULA_STAT_W_SQ] = sw;
+        row[TULA_STAT_G_SQ] = sg;
+        row[TULA_STAT_G0_SQ] = ss;
+        row[TULA_STAT_W_NORM] = o.nw;
+        row[TULA_STAT_G_NORM] = o.ng;
+        row[TULA_STAT_RATIO] = sg > 0.0 ? o.q_w : 0.0;
+        if (!step) row[TULA_STAT_COEF] = 0.0;  // a step's update has written its coefficient
+        row[TULA_STAT_SCALE] = (double)s_after;
     }
 }
 
@@ -1476,23 +1456,34 @@ template <bool HM, bool PE, bool SW>
 __global__ void __launch_bounds__(Ring2::kThreads, 1)
     k_update(const __grid_constant__ Table<kNP2> tab, const __grid_constant__ Scalars sc) {
     extern __shared__ __align__(128) unsigned char smem[];
-    // The first launch of the pass follows the pass-1 finish, which starts it
-    // once the reduction kernel has completed (the finish's own wait).  gbar, w
-    // and m are then final, so the producer streams tiles in while the finish
-    // still runs; the branch and the coefficients the consumers apply are the
-    // finish's output, so every consumer waits for its completion first.  The
-    // whole CTA waits per element (the producer's stream count depends on the
-    // branch) and in later launches of the pass (which share the tile counter
-    // with the launch before).
-    // Successors may start early only when the pass-2 finish follows (it waits
-    // for this kernel); the next step's reduction, when it follows directly,
-    // must start after this kernel has completed (see k_reduce).
-    if (sc.fin2) grid_launch_dependents();
-    const bool early = !PE && tab.first;
-    if (!early) grid_wait();
+    // The first launch of the pass issues w and m of its first tiles at once: it starts only when
+    // this step's reduction (and k_lars) have started, which let it once every kernel before them
+    // had completed, so both are final.  The mean follows when the kernel before has completed.
+    // The whole CTA waits per element (the stream count depends on the branch), in later launches
+    // of the pass (which share the tile counter with the launch before) and in a sharded step
+    // (whatever ran between its two calls).
+    const bool early = !PE && tab.first && sc.early_w;
+    if (!early) {
+        grid_wait();
+        grid_launch_dependents();
+    }
+    __shared__ int branch;
+    const bool gated = sc.rule == TULA_RULE_AGS || sc.rule == TULA_RULE_STATIC;
+    // Called by the whole CTA after its wait: every CTA forms the branch from the accumulator for
+    // itself, one warp each.
+    auto take_branch = [&]() -> int {
+        if (!gated) return 0;
+        if (threadIdx.x < 32) {
+            const int b = step_branch(sc);
+            if (threadIdx.x == 0) branch = b;
+        }
+        __syncthreads();
+        return branch;
+    };
+    int scaled = early ? 0 : take_branch();
     const int lane = threadIdx.x & 31;
     const int chunk = tab.chunk;
-    const bool use_se = PE && sc.flags[0];  // PE: after the wait above
+    const bool use_se = PE && scaled;
     const int ns = 2 + (HM ? 1 : 0) + (use_se ? 1 : 0);
     const int role = !HM && lane == 2 ? 3 : (lane < 4 ? lane : 0);
     constexpr int CH = Ring2::tile_elems(2 + (HM ? 1 : 0) + (PE ? 1 : 0));
@@ -1503,14 +1494,22 @@ __global__ void __launch_bounds__(Ring2::kThreads, 1)
     Stream<Ring2> st;
     int c = st.start(smem, tab.nc, sc.tiles + 2, sc.evict_first != 0);
     TilePos q = {};
-    if (c >= 0) q = st.issue(tab, c, chunk, role, ns);
-    if (early) grid_wait();
-    const int scaled = sc.flags[0];
-    const bool gated = sc.rule == TULA_RULE_AGS || sc.rule == TULA_RULE_STATIC;
+    if (c >= 0) q = st.issue(tab, c, chunk, role, ns, early ? 1 : 0);
+    if (early) {
+        grid_wait();
+        grid_launch_dependents();
+        if (c >= 0) st.issue_below(q, 1, chunk);
+        scaled = take_branch();
+    }
     const uint32_t stage = st.stage;
+    // Where a tensor's coefficient comes from (per tensor): the gradscale or s when scaled, LARS's
+    // ratio, else 1.
+    const float *const cand_of = sc.rule == TULA_RULE_LARS ? sc.cand
+                                 : (sc.rule == TULA_RULE_AGS && !PE && scaled) ? sc.scale : nullptr;
+    const float c_all = sc.rule == TULA_RULE_STATIC && scaled ? sc.static_s : 1.0f;
 
     int cand_t = -1;
-    float cand = 0.f;
+    float ct = c_all;
     while (c >= 0) {
         // fp32 |w|^2 of the tiles' shared-memory columns, scaled by 2^(2e) (e coded in `ecode`);
         // a tile with elements loaded one by one (fp64, rare) is stored at once instead.
@@ -1525,7 +1524,7 @@ __global__ void __launch_bounds__(Ring2::kThreads, 1)
 #pragma unroll 1
         for (int p = 0; p < kPend && c >= 0; ++p) {
             if (q.tg != cand_t) {  // c_p changes only with the tensor
-                cand = sc.cand[q.tg];
+                if (cand_of) ct = cand_of[q.tg];
                 cand_t = q.tg;
             }
             if (!st.arrived(sc)) {
@@ -1534,7 +1533,6 @@ __global__ void __launch_bounds__(Ring2::kThreads, 1)
             }
             const float *const *ptr = tab.ptr[q.t];
             const int nv = st.tc.nv;
-            const float ct = gated ? (scaled ? cand : 1.0f) : cand;
             if (sc.stats && q.c_in_t == 0 && lane == 0)
                 sc.stats[(size_t)q.tg * TULA_STATS_LEN + TULA_STAT_COEF] =
                     PE ? (scaled ? (double)NAN : 1.0) : (double)ct;
@@ -1726,10 +1724,12 @@ struct Plan {
     long long c1 = 0, c2 = 0;  // tiles of each pass (at the smallest tile sizes)
 };
 
-// Workspace layout.  Every counter, flag and accumulator precedes `tsum`, so zeroing
-// [0, tsum) clears all of them; the error word is the only one no call clears.
+// Workspace layout.  Every counter and accumulator precedes `spare`, so zeroing [0, spare) clears
+// all of them; the error word is the only one no call clears.  `flags` and `spare` hold nothing any
+// more; they stay so that workspace sizes, and the longest list the static scratch takes, are what
+// callers know.
 struct WsLayout {
-    size_t flags, err, tiles, acc1, gacc, acc2, tsum, cand, total;
+    size_t flags, err, tiles, acc1, gacc, acc2, spare, cand, total;
 };
 
 WsLayout ws_layout(int n_tensors, const Plan &) {
@@ -1747,7 +1747,7 @@ WsLayout ws_layout(int n_tensors, const Plan &) {
     L.acc1 = take(acc * kAcc * kTCopies * (size_t)n_tensors);
     L.gacc = take(acc * kGCopies);
     L.acc2 = take(acc * kTCopies * (size_t)n_tensors);
-    L.tsum = take(sizeof(double) * kTsum * (size_t)n_tensors);
+    L.spare = take(kSpare * (size_t)n_tensors);
     L.cand = take(sizeof(float) * (size_t)n_tensors);
     L.total = off;
     return L;
@@ -1915,12 +1915,12 @@ int launch_streaming(Kernel kernel, int n, const int64_t *numels, int chunk, int
     return TULA_OK;
 }
 
-// k_finish over all tensors: NA accumulators per tensor (+ the branch after pass 1 of a step).
-template <int NA>
+// One warp per tensor (+ the step record's): k_lars, k_finish.
+int launch_per_tensor(void (*kernel)(Scalars), int warps, const Scalars &sc, cudaStream_t s) {
+    return launch_pdl(kernel, (warps + kFinWarps - 1) / kFinWarps, 32 * kFinWarps, 0, s, sc);
+}
 int launch_finish(int n, const Scalars &sc, cudaStream_t s) {
-    const bool record = NA == kAcc && sc.mode == kModeStep;  // + the branch's warp
-    const int warps = n + (record ? 1 : 0);
-    return launch_pdl(k_finish<NA>, (warps + kFinWarps - 1) / kFinWarps, 32 * kFinWarps, 0, s, sc);
+    return launch_per_tensor(k_finish, n + (sc.mode == kModeStep ? 1 : 0), sc, s);
 }
 
 Scalars make_scalars(const tula_ags_hparams *hp, int K, int n, void *ws, const WsLayout &L,
@@ -1948,13 +1948,11 @@ Scalars make_scalars(const tula_ags_hparams *hp, int K, int n, void *ws, const W
         sc.stats = hp->layer_stats;
     }
     char *b = static_cast<char *>(ws);
-    sc.flags = reinterpret_cast<int *>(b + L.flags);
     sc.err = reinterpret_cast<unsigned *>(b + L.err);
     sc.tiles = reinterpret_cast<unsigned *>(b + L.tiles);
     sc.acc1 = reinterpret_cast<unsigned long long *>(b + L.acc1);
     sc.gacc = reinterpret_cast<unsigned long long *>(b + L.gacc);
     sc.acc2 = reinterpret_cast<unsigned long long *>(b + L.acc2);
-    sc.tsum = reinterpret_cast<double *>(b + L.tsum);
     sc.cand = reinterpret_cast<float *>(b + L.cand);
     return sc;
 }
@@ -1963,30 +1961,26 @@ void record(void *ev, cudaStream_t s) {
     if (ev) cudaEventRecord(static_cast<cudaEvent_t>(ev), s);
 }
 
-// Pass 1 (+ its finish) dispatched over the compile-time replica count.
+// Pass 1 dispatched over the compile-time replica count.
 template <int KT, bool WM, bool RW, bool SS, bool PR, typename Fill>
 int run_reduce_k(int K, int n, const int64_t *numels, const Scalars &sc, int grid, cudaStream_t s,
-                 Fill fill, void *mid_event, bool finish, TableCache *cache) {
+                 Fill fill, TableCache *cache) {
     const int chunk = chunk1(K, RW, SS);
-    int rc = launch_streaming<P1<KT>::NP>(k_reduce<KT, WM, RW, SS, PR>, n, numels, chunk,
-                                          Ring1Of<RW>::kThreads, Ring1Of<RW>::kSmemBytes, sc,
-                                          grid, s, fill, cache);
-    if (rc) return rc;
-    record(mid_event, s);
-    return finish ? launch_finish<kAcc>(n, sc, s) : TULA_OK;
+    return launch_streaming<P1<KT>::NP>(k_reduce<KT, WM, RW, SS, PR>, n, numels, chunk,
+                                       Ring1Of<RW>::kThreads, Ring1Of<RW>::kSmemBytes, sc, grid,
+                                       s, fill, cache);
 }
 
 template <bool WM, bool RW, bool SS, bool PR, typename Fill>
 int run_reduce(int K, int n, const int64_t *numels, const Scalars &sc, int grid, cudaStream_t s,
-               Fill fill, void *mid_event = nullptr, bool finish = true,
-               TableCache *cache = nullptr) {
+               Fill fill, TableCache *cache = nullptr) {
     switch (K) {
-    case 1: return run_reduce_k<1, false, RW, SS, PR>(K, n, numels, sc, grid, s, fill, mid_event, finish, cache);
-    case 2: return run_reduce_k<2, WM, RW, SS, PR>(K, n, numels, sc, grid, s, fill, mid_event, finish, cache);
-    case 4: return run_reduce_k<4, WM, RW, SS, PR>(K, n, numels, sc, grid, s, fill, mid_event, finish, cache);
-    case 8: return run_reduce_k<8, WM, RW, SS, PR>(K, n, numels, sc, grid, s, fill, mid_event, finish, cache);
-    case 16: return run_reduce_k<16, WM, RW, SS, PR>(K, n, numels, sc, grid, s, fill, mid_event, finish, cache);
-    default: return run_reduce_k<0, WM, RW, SS, PR>(K, n, numels, sc, grid, s, fill, mid_event, finish, cache);
+    case 1: return run_reduce_k<1, false, RW, SS, PR>(K, n, numels, sc, grid, s, fill, cache);
+    case 2: return run_reduce_k<2, WM, RW, SS, PR>(K, n, numels, sc, grid, s, fill, cache);
+    case 4: return run_reduce_k<4, WM, RW, SS, PR>(K, n, numels, sc, grid, s, fill, cache);
+    case 8: return run_reduce_k<8, WM, RW, SS, PR>(K, n, numels, sc, grid, s, fill, cache);
+    case 16: return run_reduce_k<16, WM, RW, SS, PR>(K, n, numels, sc, grid, s, fill, cache);
+    default: return run_reduce_k<0, WM, RW, SS, PR>(K, n, numels, sc, grid, s, fill, cache);
     }
 }
 
@@ -2168,6 +2162,7 @@ int run_step(float *const *param_ptrs, float *const *grad_ptrs, float *const *mo
     sc.lr = lr;
     sc.mu = momentum;
     sc.wd = weight_decay;
+    sc.early_w = part == kPartWhole ? 1 : 0;
 
     const int KS = replica_slot(K);
     auto fill1 = [&](int p, const float **dst) {
@@ -2179,24 +2174,20 @@ int run_step(float *const *param_ptrs, float *const *grad_ptrs, float *const *mo
     if (part == kPartUpdate) {
         // the ranks' shares summed give |G|^2; the local accumulators the tensors' norms
         sc.g2ext = g2_in;
-        record(hp->trace_events[1], s);
-        rc = launch_finish<kAcc>(n, sc, s);
-        sc.g2ext = nullptr;
     } else {
-        const bool fin = part == kPartWhole;
         // Norms feeding a coefficient (LARS, UpdateGradScale) are taken precisely.
         if (lars)
-            rc = run_reduce<true, true, false, true>(K, n, numels, sc, hp->grid_ctas, s, fill1,
-                                                     hp->trace_events[1], fin, cache);
+            rc = run_reduce<true, true, false, true>(K, n, numels, sc, hp->grid_ctas, s, fill1, cache);
         else if (hp->refresh_scale)
-            rc = run_reduce<true, false, false, true>(K, n, numels, sc, hp->grid_ctas, s, fill1,
-                                                      hp->trace_events[1], fin, cache);
+            rc = run_reduce<true, false, false, true>(K, n, numels, sc, hp->grid_ctas, s, fill1, cache);
         else
-            rc = run_reduce<true, false, false, false>(K, n, numels, sc, hp->grid_ctas, s, fill1,
-                                                       hp->trace_events[1], fin, cache);
+            rc = run_reduce<true, false, false, false>(K, n, numels, sc, hp->grid_ctas, s, fill1, cache);
         if (rc == TULA_OK && part == kPartReduce)
             return launch_pdl(k_share, 1, 32, 0, s, sc, share_out);
     }
+    if (rc) return rc;
+    record(hp->trace_events[1], s);
+    if (lars) rc = launch_per_tensor(k_lars, n, sc, s);
     if (rc) return rc;
     record(hp->trace_events[2], s);
 
@@ -2208,10 +2199,7 @@ int run_step(float *const *param_ptrs, float *const *grad_ptrs, float *const *mo
     };
     const bool hm = mom_ptrs != nullptr;
     const bool sw = hp->layer_stats != nullptr && !lars;  // the update takes |w|^2
-    // The statistics and UpdateGradScale are finished after the update (k_finish<1>).
-    sc.fin2 = (hp->layer_stats != nullptr || hp->refresh_scale) ? 1 : 0;
     const int c2 = chunk2(hm, per_elem);
-    sc.mode = kModeUpdate;
 #define TULA_UPD(HM, PE, SW)                                                                \
     launch_streaming<kNP2>(k_update<HM, PE, SW>, n, numels, c2, Ring2::kThreads,             \
                            Ring2::kSmemBytes, sc, hp->grid_ctas, s, fill2, cache)
@@ -2225,7 +2213,7 @@ int run_step(float *const *param_ptrs, float *const *grad_ptrs, float *const *mo
 #undef TULA_UPD
     if (rc) return rc;
     record(hp->trace_events[3], s);
-    if (sc.fin2) rc = launch_finish<1>(n, sc, s);
+    rc = launch_finish(n, sc, s);
     if (rc) return rc;
     record(hp->trace_events[4], s);
     return TULA_OK;
@@ -2376,8 +2364,9 @@ int tula_layer_stats(const float *const *param_ptrs, const float *const *grad_pt
         dst[KS] = param_ptrs[p];
         dst[KS + 1] = nullptr;
     };
-    return run_reduce<false, true, false, false>(K, n, numels, sc, 0,
-                                                 static_cast<cudaStream_t>(stream), fill);
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    rc = run_reduce<false, true, false, false>(K, n, numels, sc, 0, s, fill);
+    return rc ? rc : launch_finish(n, sc, s);
 }
 
 int tula_ags_update_scale(const float *const *g_small, const float *const *g_large,
@@ -2420,8 +2409,8 @@ int tula_ags_update_scale(const float *const *g_small, const float *const *g_lar
         dst[1] = nullptr;
         dst[2] = g_small[p];
     };
-    return run_reduce_k<1, false, false, true, true>(1, n, numels, sc, hp->grid_ctas, s, fill,
-                                                     nullptr, true, nullptr);
+    rc = run_reduce_k<1, false, false, true, true>(1, n, numels, sc, hp->grid_ctas, s, fill, nullptr);
+    return rc ? rc : launch_finish(n, sc, s);
 }
 
 const char *tula_ags_error_string(int code) {
@@ -2497,14 +2486,13 @@ extern "C" int tula_ags_step_static_scratch(float *const *param_ptrs, float *con
     void *scratch = nullptr;
     rc = static_scratch_address(&scratch);
     if (rc) return rc;
-    // The array keeps the last call's contents: zero the branch flag, the tile counters and the
-    // accumulators (they precede the per-tensor sums) before this call's kernels.  The error
+    // The array keeps the last call's contents: zero the tile counters and the accumulators before this call's kernels.  The error
     // word between them is left alone, so that a wait that ran out stays reported until
     // tula_ags_static_scratch_error reads it.
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     char *b = static_cast<char *>(scratch);
     cudaError_t e = cudaMemsetAsync(b, 0, L.err, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(b + L.tiles, 0, L.tsum - L.tiles, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(b + L.tiles, 0, L.spare - L.tiles, s);
     if (e != cudaSuccess) {
         g_last_cuda = (int)e;
         return TULA_ERR_CUDA;
