@@ -96,9 +96,10 @@ enum Mode { kModeStep = 0, kModeStats = 1, kModeScale = 2 };
 // Launch tables (kernel parameters)
 // ----------------------------------------------------------------------------
 
+constexpr int kHints = 160, kHintTiles = 8;  // covers the first tiles of 152 SMs' 8 warps
 template <int NP>
 struct Table {
-    static constexpr int kMaxT = (kParamBudget - 64) / (NP * 8 + 12);
+    static constexpr int kMaxT = (kParamBudget - 64 - 2 * kHints) / (NP * 8 + 12);
     int n;      // tensors in this launch
     int t0;     // global index of its first tensor
     int c0;     // global index of its first tile
@@ -108,6 +109,7 @@ struct Table {
     int pad[2];
     long long numel[kMaxT];
     int cstart[kMaxT + 1];  // first tile of each tensor, relative to c0; cstart[n] = nc
+    unsigned short hint[kHints];  // tensor of tile min(i * kHintTiles, nc - 1)
     const float *ptr[kMaxT][NP];
 };
 
@@ -566,7 +568,14 @@ struct Walker {
     int t = -1;
     template <int NP>
     __device__ __forceinline__ int to(const Table<NP> &tab, int c) {
-        if (t < 0) return t = find_tensor(tab.cstart, 0, tab.n, c);
+        if (t < 0) {
+            // The warp's first tile: the table is not in the constant cache yet, and the eight
+            // or so steps of a search, each a miss, took 2 us.  Two with the hint.
+            if (c >= kHints * kHintTiles) return t = find_tensor(tab.cstart, 0, tab.n, c);
+            t = tab.hint[c / kHintTiles];
+            while (c >= tab.cstart[t + 1]) ++t;  // at most kHintTiles - 1 steps
+            return t;
+        }
         if (c < tab.cstart[t + 1]) return t;
         ++t;
         if (c < tab.cstart[t + 1]) return t;
@@ -685,9 +694,12 @@ struct Stream {
         ctr = counter;
         hint = evict_first;
         policy = policy_evict_first();
-        if (claims && (threadIdx.x & 31) == 0) pend = atomicAdd(ctr, 1u);
         const unsigned v = (unsigned)warp * gridDim.x + blockIdx.x;
         return v < nc ? (int)v : -1;
+    }
+    // The first claim, once the first tile has been issued.
+    __device__ __forceinline__ void claim_first() {
+        if (claims && (threadIdx.x & 31) == 0) pend = atomicAdd(ctr, 1u);
     }
     // The tile after the last one taken (-1: none left).
     __device__ __forceinline__ int next() {
@@ -1084,6 +1096,7 @@ __global__ void __launch_bounds__(Ring1Of<RW>::kThreads, 1)
     int c = st.start(smem, tab.nc, sc.tiles, sc.evict_first != 0);
     TilePos q = {};
     if (c >= 0) q = st.issue(tab, c, chunk, role, ns);
+    st.claim_first();
     if (early) {
         grid_wait();
         grid_launch_dependents();
@@ -1495,6 +1508,7 @@ __global__ void __launch_bounds__(Ring2::kThreads, 1)
     int c = st.start(smem, tab.nc, sc.tiles + 2, sc.evict_first != 0);
     TilePos q = {};
     if (c >= 0) q = st.issue(tab, c, chunk, role, ns, early ? 1 : 0);
+    st.claim_first();
     if (early) {
         grid_wait();
         grid_launch_dependents();
@@ -1893,6 +1907,10 @@ int launch_streaming(Kernel kernel, int n, const int64_t *numels, int chunk, int
                 tab->n = cnt;
                 tab->nc = nc;
                 tab->cstart[cnt] = nc;
+                for (int i = 0, t = 0; i < kHints; ++i) {
+                    while (t + 1 < cnt && i * kHintTiles >= tab->cstart[t + 1]) ++t;
+                    tab->hint[i] = (unsigned short)t;
+                }
                 c_global += nc;
                 built.push_back(std::move(tab));
             }
