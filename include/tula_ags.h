@@ -14,9 +14,9 @@
  *      SGD optimizer with momentum and weight decay (Sec. IV-A, IV-B).
  *
  * Conventions for every entry point:
- *   - Tensors are fp32, in caller-owned DEVICE memory, 4-byte aligned; the
- *     fast path wants them 16-byte aligned (misaligned tensors take a scalar
- *     path with the same results).
+ *   - Tensors are fp32, in caller-owned DEVICE memory, 4-byte aligned; every
+ *     buffer of a tensor at a 16-byte boundary is fastest (a step over
+ *     misaligned ones, views into packed buckets say, takes about 20 % longer).
  *   - Arrays of pointers (param_ptrs, grad_ptrs, ...) and numels are HOST
  *     arrays, read during the call only.
  *   - Calls are asynchronous on `stream` (a cudaStream_t; NULL = the legacy
@@ -41,8 +41,9 @@
  *     once to fp64.  A tile whose fp32 sums would overflow (a lane sum above
  *     2^120) or lose precision to underflow (every lane sum below 2^-100, zero
  *     included) is summed again with its elements scaled by an exact power of two,
- *     and elements loaded one by one (tails, misaligned tensors) are squared in
- *     fp64, so these norms hold over the whole fp32 range.  Norms that feed a
+ *     the last n % 4 elements of a tensor are squared in fp64, and the tensors with
+ *     a buffer off a 16-byte boundary have their squares added as below, so these
+ *     norms hold over the whole fp32 range.  Norms that feed a
  *     coefficient (gradscale refresh, LARS) split every square exactly into two
  *     fp32 parts, add them as float-float pairs per lane and in fp64 across lanes
  *     (relative error ~1e-14), then exactly across tiles; a tile whose pairs cannot hold that (a

@@ -57,29 +57,57 @@
 
 namespace {
 
+// Tensors off a 16-byte boundary: a stream's tile starts up to 12 bytes into its part of the
+// stage, which is kShiftBytes longer; the stages have room for that.
+constexpr int kShiftBytes = 16;
 // The stages of a streaming kernel's CTA: one per warp, each holding one tile of every stream.  A
 // warp refills its own stage (see "Streaming warps" below), so a CTA is nothing but warps that
 // stream for themselves.
-template <int StageKB, int Warps>
+template <int StageKB, int Warps, int Pad>
 struct Ring {
-    static constexpr int kStageBytes = StageKB * 1024;
+    static constexpr int kTileBytes = StageKB * 1024;  // one aligned tile of every stream
+    static constexpr int kStageBytes = kTileBytes + Pad;
     static constexpr int kWarps = Warps;
     static constexpr int kThreads = 32 * Warps;
     static constexpr int kSmemBytes = Warps * (kStageBytes + 8);
-    static_assert(kSmemBytes <= 227 * 1024, "one CTA per SM");
+    static_assert(kSmemBytes <= 227 * 1024 && kStageBytes % 16 == 0, "one CTA per SM");
     // Elements per tile when `streams` tensors share one stage (multiple of 128).
     __host__ __device__ static constexpr int tile_elems(int streams) {
-        return (kStageBytes / (4 * streams)) / 128 * 128;
+        return (kTileBytes / (4 * streams)) / 128 * 128;
+    }
+    // Whether the shifted tiles (see issue_edge_tile) of `streams` tensors fit, too.
+    static constexpr bool shifted_fits(int streams) {
+        return streams * (4 * tile_elems(streams) + kShiftBytes) <= kStageBytes;
     }
 };
+template <typename R>
+constexpr bool shifted_fits_up_to(int streams) {
+    for (int ns = 1; ns <= streams; ++ns)
+        if (!R::shifted_fits(ns)) return false;
+    return true;
+}
 // Pass 1 streams K (+1, +2) tensors through 36 KB stages.
-using Ring1 = Ring<36, 6>;
-// Pass 1 when it also reads w (LARS, tula_layer_stats): five 45 KB stages.
-using Ring1W = Ring<45, 5>;
-template <bool RW>
-using Ring1Of = std::conditional_t<RW, Ring1W, Ring1>;
+// SH: with room for shifted tiles, in the kernels of launches that have any.
+template <bool SH>
+using Ring1 = Ring<36, 6, SH ? 256 : 0>;
+static_assert(shifted_fits_up_to<Ring1<true>>(TULA_MAX_K), "shifted tiles fit a stage");
+// Pass 1 when it also reads w (LARS, tula_layer_stats): five 45 KB stages.  No more padding than
+// the stream count needs: beside the CTA, an SM must have the 1 KB of shared memory left that any
+// other CTA takes, or the small kernels around it cannot be resident while it runs (a ResNet-50
+// LARS step with 256 bytes more a stage took 251 us instead of 236).
+template <int KT, bool SH>
+using Ring1W = Ring<45, 5, !SH ? 0 : KT == 0 ? 240 : (KT + 1) * kShiftBytes>;
+static_assert(shifted_fits_up_to<Ring1W<0, true>>(TULA_MAX_K + 1) &&
+                  Ring1W<1, true>::shifted_fits(2) && Ring1W<2, true>::shifted_fits(3) &&
+                  Ring1W<4, true>::shifted_fits(5) && Ring1W<8, true>::shifted_fits(9) &&
+                  Ring1W<16, true>::shifted_fits(17),
+              "shifted tiles fit a stage");
+template <int KT, bool RW, bool SH>
+using Ring1Of = std::conditional_t<RW, Ring1W<KT, SH>, Ring1<SH>>;
 // Pass 2: eight 24 KB stages.
-using Ring2 = Ring<24, 8>;
+template <bool SH>
+using Ring2 = Ring<24, 8, SH ? 256 : 0>;
+static_assert(shifted_fits_up_to<Ring2<true>>(4), "shifted tiles fit a stage");
 constexpr int kPend = 4;                // tiles whose warp reductions run together
 constexpr int kFinWarps = 4;            // k_finish: one warp per tensor, 4 per CTA
 constexpr int kParamBudget = 31 * 1024; // kernel parameter bytes per launch (limit 32764)
@@ -106,7 +134,8 @@ struct Table {
     int nc;     // tiles in this launch
     int chunk;  // elements per tile
     int first;  // 1 for the first launch of the pass (in issue order)
-    int pad[2];
+    int shifted;  // 1: some tensor has a stream off a 16-byte boundary
+    int pad;
     long long numel[kMaxT];
     int cstart[kMaxT + 1];  // first tile of each tensor, relative to c0; cstart[n] = nc
     unsigned short hint[kHints];  // tensor of tile min(i * kHintTiles, nc - 1)
@@ -146,6 +175,12 @@ __device__ __forceinline__ float4 lds4(uint32_t addr) {
     asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
                  : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
                  : "r"(addr));
+    return v;
+}
+
+__device__ __forceinline__ float lds1(uint32_t addr) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
     return v;
 }
 
@@ -537,6 +572,15 @@ __device__ __forceinline__ void bulk_g2s_hint(uint32_t dst, const void *src, uin
         "l"(src), "r"(bytes), "r"(smem_addr(bar)), "l"(policy)
         : "memory");
 }
+// One fp32 global -> shared, asynchronously, by this lane; cp_async_wait() waits for every such
+// copy of this lane.
+__device__ __forceinline__ void cp_async4(uint32_t dst, const float *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+__device__ __forceinline__ void fence_async_proxy() {
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+}
 // L2 policy: these lines are the first to go.
 __device__ __forceinline__ uint64_t policy_evict_first() {
     uint64_t p;
@@ -617,8 +661,8 @@ struct TensorCache {
     int t = -1;
     long long numel = 0;
     const float *mine = nullptr;
-    bool aligned = false;
-    int nv = 0;  // float4 moved by TMA for the last tile asked for
+    bool aligned = false;  // every stream at a 16-byte boundary
+    int nv = 0;            // whole float4 columns of the last tile asked for (0: a shifted tile)
     template <int NP>
     __device__ __forceinline__ TilePos at(const Table<NP> &tab, int c, int chunk, int role, int ns) {
         const int tn = walk.to(tab, c);
@@ -664,7 +708,56 @@ struct TensorCache {
 // last warp to finish puts both counters (ctr[0], ctr[1]) back to zero.  Where a tile is processed
 // never changes its result: each tile's partial sums are added exactly, in integers, into its
 // tensor's accumulators.
-template <typename R>
+//
+// Any 4-byte aligned tensor moves this way.  When some stream of a tensor lies off a 16-byte
+// boundary (views into a flat bucket, say), its tiles are shifted: stream i's part of the stage
+// starts at i * (4 * chunk + kShiftBytes) and holds the 16-byte granules that the tile touches and
+// that lie wholly inside the tensor, so element j of the tile sits addr & 12 bytes plus 4 j in,
+// whatever the streams' alignments are to one another.  (The first and last granule may bring
+// elements of the neighbouring tiles along, which another warp may be updating; nobody reads
+// them.)  The up to three elements at each end of a tensor outside those granules, and the last
+// n % 4 elements of an aligned tensor, come by 4-byte cp.async into the same places.  Only the
+// kernels for launches with such a tensor (SH) hold this code: in the others it cost 0.4 % (ResNet-50)
+// to 5 % (1024 small layers) of a step, and they load an aligned tensor's tail directly.  Before,
+// misaligned tensors were loaded one element at a time and squared in fp64: 17.3 M elements in 128
+// tensors, K = 4, the gradients packed, took 548 us a step; now 133 us, against 109 us aligned.
+
+// A shifted tile, or the last tile of an aligned tensor of n % 4 != 0 elements: this lane's stream
+// (mine; nullptr: none) of n elements from `begin` of a tensor with `rest` elements from there on.
+// part: the lane's part of the stage.  The bytes of all streams are armed by lane 0 when `arm`.
+// Out of line, so that the path of ordinary tiles stays short.
+__device__ __noinline__ void issue_edge_tile(uint32_t part, const float *mine, bool aligned,
+                                             long long begin, int n, long long rest, bool arm,
+                                             bool copy, uint64_t *bar, bool hint, uint64_t policy) {
+    // Elements [lo, hi) of this lane's stream, counted from the tile's first, come in bulk.
+    int lo = 0, hi = n & ~3;
+    if (!aligned) {
+        const int phi = (int)(reinterpret_cast<uintptr_t>(mine) & 15u) >> 2;
+        const long long inside = rest - ((phi + rest) & 3);
+        const int up = (4 - phi) & 3;
+        lo = begin == 0 ? up : -phi;
+        hi = (int)min((long long)(n + up), inside);
+        if (hi < lo) hi = lo;
+        part += (uint32_t)(4 * phi);
+    }
+    if (!mine) hi = lo;
+    const uint32_t bytes = 4u * (uint32_t)(hi - lo);
+    const uint32_t expect = __reduce_add_sync(kFull, bytes);
+    if (arm && (threadIdx.x & 31) == 0) mbar_arrive_tx(bar, expect);
+    __syncwarp();
+    if (!mine || !copy) return;
+    const float *src = mine + begin;
+    if (bytes) {
+        const uint32_t to = part + 4u * (uint32_t)lo;  // lo may be negative: modulo 2^32
+        if (hint) bulk_g2s_hint(to, src + lo, bytes, bar, policy);
+        else bulk_g2s(to, src + lo, bytes, bar);
+    }
+    const int head = bytes ? max(lo, 0) : n, tail = bytes ? min(hi, n) : n;
+    for (int e = 0; e < head; ++e) cp_async4(part + 4u * (uint32_t)e, src + e);
+    for (int e = tail; e < n; ++e) cp_async4(part + 4u * (uint32_t)e, src + e);
+}
+
+template <typename R, bool SH>
 struct Stream {
     uint32_t stage;  // shared-memory address of this warp's stage
     uint64_t *bar;   // its mbarrier: one arrival, which arms the bytes of all streams
@@ -676,6 +769,7 @@ struct Stream {
     uint64_t policy;
     bool hint;
     TensorCache tc;  // of the tile in the stage (or on its way there)
+    bool edges = false;  // SH: it came partly by cp.async
 
     // Barrier init; returns this warp's first tile (-1: none).  Called by the whole CTA.
     __device__ __forceinline__ int start(unsigned char *smem, int n_tiles, unsigned *counter,
@@ -716,14 +810,31 @@ struct Stream {
                                              int ns, int from = 0) {
         const int lane = threadIdx.x & 31;
         const TilePos q = tc.at(tab, c, chunk, role, ns);
+        if constexpr (SH) {
+            const int n = (int)(q.end - q.begin);
+            if (edges) fence_async_proxy();  // cp.async wrote the stage: before bulk copies do
+            edges = n > 0 && !(tc.aligned && (n & 3) == 0);
+            if (edges) {
+                edge(q, lane, lane >= from && lane < ns, lane < ns, chunk, true);
+                return q;
+            }
+        }
         if (lane == 0) mbar_arrive_tx(bar, 16u * (uint32_t)(tc.nv * ns));
         __syncwarp();
         if (lane >= from && lane < ns) copy(q, lane, chunk);
         return q;
     }
-    __device__ __forceinline__ void issue_below(const TilePos &q, int from, int chunk) {
+    __device__ __forceinline__ void issue_below(const TilePos &q, int from, int ns, int chunk) {
         const int lane = threadIdx.x & 31;
-        if (lane < from) copy(q, lane, chunk);
+        if (SH && edges) edge(q, lane, lane < from, lane < ns, chunk, false);
+        else if (lane < from) copy(q, lane, chunk);
+    }
+    __device__ __forceinline__ void edge(const TilePos &q, int lane, bool mine, bool stream,
+                                         int chunk, bool arm) {
+        const uint32_t part = (uint32_t)(4 * chunk + (tc.aligned ? 0 : kShiftBytes));
+        issue_edge_tile(stage + (uint32_t)lane * part, stream ? tc.mine : nullptr, tc.aligned,
+                        q.begin, (int)(q.end - q.begin), tc.numel - q.begin, arm, mine, bar, hint,
+                        policy);
     }
     __device__ __forceinline__ void copy(const TilePos &q, int lane, int chunk) {
         const uint32_t bytes = 16u * (uint32_t)tc.nv;
@@ -744,6 +855,10 @@ struct Stream {
             claims = false;
         }
         phase ^= 1u;
+        if (SH && edges) {  // each lane's cp.async copies, then every lane's are there
+            cp_async_wait();
+            __syncwarp();
+        }
         return ok;
     }
     // After the warp's last tile: the last warp of the launch re-arms the counters.
@@ -873,16 +988,110 @@ __device__ __noinline__ F3 tile_cols_scaled(uint32_t stage, int chunk, int nv, c
     return r;
 }
 
+// A tile of a tensor off a 16-byte boundary (see issue_edge_tile() for where its elements lie): lane l
+// takes elements l, l + 32, ..., four at a time, with conflict-free 4-byte loads from shared
+// memory and coalesced 4-byte stores of the mean.  The squares are float-float pairs in either
+// mode: the elements of such tensors used to be squared in fp64, and these sums keep that
+// precision (relative error ~1e-15 a lane) without GB300's slow FP64 pipe.  Returns the lane's
+// sums; out of line, so that the streaming loop of aligned tensors keeps its shape.
+template <int KT, bool WM, bool RW, bool SS>
+__device__ __noinline__ D3 tile_shifted(uint32_t stage, int chunk, const float *const *ptr,
+                                        long long begin, int n, const Scalars &sc) {
+    constexpr int KS = P1<KT>::KS;
+    const int lane = threadIdx.x & 31;
+    const int K = KT > 0 ? KT : sc.K;
+    const uint32_t part = (uint32_t)(4 * chunk + kShiftBytes);
+    auto at = [&](int stream, int role) {
+        return stage + (uint32_t)stream * part + ((uint32_t)reinterpret_cast<uintptr_t>(ptr[role]) & 12u);
+    };
+    uint32_t at_k[KT > 0 ? KT : 1];
+#pragma unroll
+    for (int k = 0; k < (KT > 0 ? KT : 1); ++k) at_k[k] = at(k, k);
+    const uint32_t at_w = RW ? at(K, KS) : 0u;
+    const uint32_t at_s = SS ? at(K + (RW ? 1 : 0), KS + 1) : 0u;
+    float *out = const_cast<float *>(ptr[0]) + begin;
+    Dw4 ag, as, aw;
+    dw_zero(ag);
+    dw_zero(as);
+    dw_zero(aw);
+    for (int j0 = lane; j0 < n; j0 += 128) {
+        uint32_t o[4];  // byte offsets; past the end, the last element's (taken as 0)
+        bool in[4];
+        float x0[4], s[4], wv[4], sv[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            in[u] = j0 + 32 * u < n;
+            o[u] = 4u * (uint32_t)min(j0 + 32 * u, n - 1);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) s[u] = x0[u] = lds1(at_k[0] + o[u]);
+        if constexpr (KT > 0) {
+#pragma unroll
+            for (int k = 1; k < KT; ++k)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) s[u] = __fadd_rn(s[u], lds1(at_k[k] + o[u]));
+        } else {
+            for (int k = 1; k < K; ++k) {
+                const uint32_t a = at(k, k);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) s[u] = __fadd_rn(s[u], lds1(a + o[u]));
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            wv[u] = RW ? lds1(at_w + o[u]) : 0.f;
+            sv[u] = SS ? lds1(at_s + o[u]) : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (K > 1) {
+                s[u] = mean1<KT>(s[u], sc);
+                if (WM && in[u]) out[j0 + 32 * u] = s[u];
+            }
+            dw_sq(ag.hi[u], ag.lo[u], in[u] ? s[u] : 0.f);
+            if (K > 1) dw_sq(as.hi[u], as.lo[u], in[u] ? x0[u] : 0.f);
+            if (SS) dw_sq(as.hi[u], as.lo[u], in[u] ? sv[u] : 0.f);
+            if (RW) dw_sq(aw.hi[u], aw.lo[u], in[u] ? wv[u] : 0.f);
+        }
+    }
+    __syncwarp();
+    const float2 pg = dw_pair(ag), ps = dw_pair(as), pw = dw_pair(aw);
+    const bool bad = lane < n && !(dw_lane_ok(pg) && (!(K > 1 || SS) || dw_lane_ok(ps)) &&
+                                   (!RW || dw_lane_ok(pw)));
+    D3 r = {ff_to_double(pg), ff_to_double(ps), ff_to_double(pw)};
+    if (__any_sync(kFull, bad)) {  // as tile_cols_fp64: again, every square exact in fp64
+        r = {0.0, 0.0, 0.0};
+        for (int j = lane; j < n; j += 32) {
+            const uint32_t o = 4u * (uint32_t)j;
+            const float x0 = lds1(at_k[0] + o);
+            float s = x0;
+            for (int k = 1; k < K; ++k) s = __fadd_rn(s, lds1(at(k, k) + o));
+            if (K > 1) s = mean1<KT>(s, sc);
+            r.g = __fma_rn((double)s, (double)s, r.g);
+            if (K > 1) r.s = __fma_rn((double)x0, (double)x0, r.s);
+            if (SS) {
+                const double y = (double)lds1(at_s + o);
+                r.s = __fma_rn(y, y, r.s);
+            }
+            if (RW) {
+                const double y = (double)lds1(at_w + o);
+                r.w = __fma_rn(y, y, r.w);
+            }
+        }
+        __syncwarp();
+    }
+    return r;
+}
+
 // Per-lane partial sums of one tile (not yet reduced across the warp).  Precise mode (PR):
 // accd holds the lane's fp64 sums.  Default mode: accf holds the lane's fp32 sums over the
-// tile's shared-memory columns, scaled by 2^(2 acce) (acce is the same in every lane), and accd
-// the lane's exact fp64 sums over the elements loaded directly (tail, misaligned tensor).
-template <int KT, bool WM, bool RW, bool SS, bool PR>
+// tile's float4 columns, scaled by 2^(2 acce) (acce is the same in every lane), and accd the
+// lane's fp64 sums over the elements taken one by one (tail, shifted tile).
+template <int KT, bool WM, bool RW, bool SS, bool PR, bool SH>
 __device__ __forceinline__ void reduce_tile(uint32_t stage, int chunk, const float *const *ptr,
-                                            const TilePos &q, int nv, const Scalars &sc,
-                                            double (&accd)[kAcc], float (&accf)[kAcc],
+                                            const TilePos &q, int nv, bool aligned,
+                                            const Scalars &sc, double (&accd)[kAcc], float (&accf)[kAcc],
                                             int (&acce)[kAcc], unsigned &ecode, bool &tail) {
-    constexpr int KS = P1<KT>::KS;
     const int lane = threadIdx.x & 31;
     const int K = KT > 0 ? KT : sc.K;
     const uint32_t sw_s = stage + (uint32_t)(K * chunk * 4);
@@ -892,14 +1101,25 @@ __device__ __forceinline__ void reduce_tile(uint32_t stage, int chunk, const flo
     dw_zero(ag);
     dw_zero(as);
     dw_zero(aw);
-    double rg = 0.0, rs = 0.0, rw = 0.0;  // exact fp64 sums of the elements loaded directly
-    const int ncols = nv;                 // the shared-memory columns (nv is reused below)
-    tail = false;                         // the tile has elements loaded one by one
+    double rg = 0.0, rs = 0.0, rw = 0.0;  // exact fp64 sums of the tail
+    const int ncols = nv;                 // the float4 columns (nv is reused below)
+    tail = false;                         // the tile has elements taken one by one
     ecode = 0u;                           // scale_code of acce[a] in bits 2a, 2a + 1
+    if (SH && !aligned) {
+        const D3 d = tile_shifted<KT, WM, RW, SS>(stage, chunk, ptr, q.begin,
+                                                         (int)(q.end - q.begin), sc);
+        accd[0] = d.g;
+        accd[1] = (K > 1 || SS) ? d.s : d.g;  // K = 1: replica 0 is the mean
+        accd[2] = d.w;
+        accf[0] = accf[1] = accf[2] = 0.f;
+        acce[0] = acce[1] = acce[2] = 0;
+        tail = true;
+        return;
+    }
     float fg = 0.f, fs = 0.f, fw = 0.f;   // fp32 sums (not PR)
 
     if constexpr (KT > 0) {
-        constexpr int CH = Ring1Of<RW>::tile_elems(KT + (RW ? 1 : 0) + (SS ? 1 : 0));
+        constexpr int CH = Ring1Of<KT, RW, SH>::tile_elems(KT + (RW ? 1 : 0) + (SS ? 1 : 0));
         constexpr int COLS = CH / 128;  // float4 columns per lane of a full tile
         if (nv == CH / 4) {
             // Full tile: every lane has COLS columns; all loads of a column issue together.
@@ -958,19 +1178,20 @@ __device__ __forceinline__ void reduce_tile(uint32_t stage, int chunk, const flo
                 if (RW) fw = __fadd_rn(fw, pw);
             }
         }
-        // Tail (< 4 elements) or a misaligned tensor: plain loads from global memory, exact
-        // squares in fp64 (this is where replica 0 is overwritten, so there is no second look).
+        // The last n % 4 elements, exact squares in fp64: from the stage (SH) or by plain loads.
         tail = q.begin + 4 * (long long)nv < q.end;  // the same in every lane
         for (long long j = q.begin + 4 * (long long)nv + lane; j < q.end; j += 32) {
-            const float x0 = __ldcs(ptr[0] + j);
+            const uint32_t o = 4u * (uint32_t)(j - q.begin);
+            const float x0 = SH ? lds1(stage + o) : __ldcs(ptr[0] + j);
             float s = x0;
-            for (int k = 1; k < K; ++k) s = __fadd_rn(s, __ldcs(ptr[k] + j));
+            for (int k = 1; k < K; ++k)
+                s = __fadd_rn(s, SH ? lds1(stage + (uint32_t)(4 * k * chunk) + o) : __ldcs(ptr[k] + j));
             if (K > 1) {
                 s = mean1<KT>(s, sc);
                 if (WM) const_cast<float *>(ptr[0])[j] = s;
             }
-            const float y_s = SS ? __ldcs(ptr[KS + 1] + j) : 0.f;
-            const float y_w = RW ? __ldcs(ptr[KS] + j) : 0.f;
+            const float y_s = !SS ? 0.f : SH ? lds1(ss_s + o) : __ldcs(ptr[P1<KT>::KS + 1] + j);
+            const float y_w = !RW ? 0.f : SH ? lds1(sw_s + o) : __ldcs(ptr[P1<KT>::KS] + j);
             if (K > 1) rs = __fma_rn((double)x0, (double)x0, rs);
             rg = __fma_rn((double)s, (double)s, rg);
             if (SS) rs = __fma_rn((double)y_s, (double)y_s, rs);
@@ -1044,7 +1265,7 @@ __device__ __forceinline__ unsigned long long *acc2_of(const Scalars &sc, int tg
     return sc.acc2 + ((size_t)tg * kTCopies + (blockIdx.x & (kTCopies - 1))) * kAccWords;
 }
 
-// A default-mode tile with elements loaded one by one (the last tile of a tensor whose size is
+// A default-mode tile with elements taken one by one (the last tile of a tensor whose size is
 // not a multiple of 4, or a misaligned tensor): its sums are reduced across the warp at once,
 // fp32 part and fp64 part, and lane 0 adds both into the tensor's accumulators.
 __device__ __noinline__ void add_tile_now(const Scalars &sc, int tg, const float (&accf)[kAcc],
@@ -1071,8 +1292,8 @@ __device__ __noinline__ void add_tile_now(const Scalars &sc, int tg, const float
     }
 }
 
-template <int KT, bool WM, bool RW, bool SS, bool PR>
-__global__ void __launch_bounds__(Ring1Of<RW>::kThreads, 1)
+template <int KT, bool WM, bool RW, bool SS, bool PR, bool SH>
+__global__ void __launch_bounds__(Ring1Of<KT, RW, SH>::kThreads, 1)
     k_reduce(const __grid_constant__ Table<P1<KT>::NP> tab, const __grid_constant__ Scalars sc) {
     constexpr int KS = P1<KT>::KS;
     extern __shared__ __align__(128) unsigned char smem[];
@@ -1092,7 +1313,7 @@ __global__ void __launch_bounds__(Ring1Of<RW>::kThreads, 1)
     // Stage streams: replicas 0 .. K - 1, then w (RW), then g_small (SS).
     const int ns = K + (RW ? 1 : 0) + (SS ? 1 : 0);
     const int role = lane < K ? lane : (RW && lane == K ? KS : KS + 1);
-    Stream<Ring1Of<RW>> st;
+    Stream<Ring1Of<KT, RW, SH>, SH> st;
     int c = st.start(smem, tab.nc, sc.tiles, sc.evict_first != 0);
     TilePos q = {};
     if (c >= 0) q = st.issue(tab, c, chunk, role, ns);
@@ -1110,7 +1331,7 @@ __global__ void __launch_bounds__(Ring1Of<RW>::kThreads, 1)
     while (c >= 0) {
         // PR: the lanes' fp64 sums.  Default: fp32 sums of the shared-memory columns, scaled by
         // 2^(2e) with e coded in two bits per value in `ecode` (same in every lane); a tile with
-        // elements loaded one by one (fp64, rare) is stored at once instead (add_tile_now).
+        // elements taken one by one is stored at once instead (add_tile_now).
         double pendd[PR ? kRS : 1];
         float pendf[PR ? 1 : kRS];
         unsigned ecode = 0u;
@@ -1136,8 +1357,8 @@ __global__ void __launch_bounds__(Ring1Of<RW>::kThreads, 1)
             int acce[kAcc];
             unsigned tcode;
             bool tile_tail;
-            reduce_tile<KT, WM, RW, SS, PR>(st.stage, chunk, ptr, q, st.tc.nv, sc, accd, accf, acce,
-                                            tcode, tile_tail);
+            reduce_tile<KT, WM, RW, SS, PR, SH>(st.stage, chunk, ptr, q, st.tc.nv, st.tc.aligned, sc,
+                                            accd, accf, acce, tcode, tile_tail);
             __syncwarp();
             const int tg = q.tg;
             c = st.next();
@@ -1452,7 +1673,7 @@ __device__ __noinline__ float w_cols_scaled(uint32_t w_stage, int nv, float f) {
     return a;
 }
 
-// A tile of the update with elements loaded one by one: its |w|^2 (fp32 part scaled by 2^(2e),
+// A tile of the update with elements taken one by one: its |w|^2 (fp32 part scaled by 2^(2e),
 // fp64 part) reduced across the warp at once and added into the accumulator A by lane 0.
 __device__ __noinline__ void add_w_tile_now(unsigned long long *A, float aw, int e, double awt) {
     float f[1] = {aw};
@@ -1465,8 +1686,63 @@ __device__ __noinline__ void add_w_tile_now(unsigned long long *A, float aw, int
     }
 }
 
+// A tile of a tensor off a 16-byte boundary, as tile_shifted() of pass 1: four elements per lane
+// and step.  Returns the lane's |w|^2 (float-float pairs, to fp64 once) when the statistics want it.
 template <bool HM, bool PE, bool SW>
-__global__ void __launch_bounds__(Ring2::kThreads, 1)
+__device__ __noinline__ double update_shifted(uint32_t stage, const float *const *ptr,
+                                              long long begin, int n, float ct, bool use_se,
+                                              const Scalars &sc) {
+    constexpr uint32_t part = (uint32_t)(4 * Ring2<false>::tile_elems(2 + (HM ? 1 : 0) + (PE ? 1 : 0)) +
+                                         kShiftBytes);
+    const int lane = threadIdx.x & 31;
+    auto at = [&](int stream, int role) {
+        return stage + (uint32_t)stream * part + ((uint32_t)reinterpret_cast<uintptr_t>(ptr[role]) & 12u);
+    };
+    const uint32_t at_g = at(0, 0), at_w = at(1, 1), at_m = HM ? at(2, 2) : 0u;
+    const uint32_t at_c = use_se ? at(HM ? 3 : 2, 3) : 0u;
+    float *wp = const_cast<float *>(ptr[1]) + begin;
+    float *mp = HM ? const_cast<float *>(ptr[2]) + begin : nullptr;
+    Dw4 aw;
+    dw_zero(aw);
+    for (int j0 = lane; j0 < n; j0 += 128) {
+        float g[4], w[4], m[4], c[4];
+        bool in[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            in[u] = j0 + 32 * u < n;
+            const uint32_t o = 4u * (uint32_t)min(j0 + 32 * u, n - 1);
+            g[u] = lds1(at_g + o);
+            w[u] = lds1(at_w + o);
+            m[u] = HM ? lds1(at_m + o) : 0.f;
+            c[u] = use_se ? lds1(at_c + o) : (PE ? 1.f : ct);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (SW) dw_sq(aw.hi[u], aw.lo[u], in[u] ? w[u] : 0.f);
+            sgd1(g[u], c[u], w[u], m[u], sc, HM);
+            if (in[u]) {
+                __stcs(wp + j0 + 32 * u, w[u]);
+                if (HM) __stcs(mp + j0 + 32 * u, m[u]);
+            }
+        }
+    }
+    __syncwarp();
+    if (!SW) return 0.0;
+    const float2 pw = dw_pair(aw);
+    double r = ff_to_double(pw);
+    if (__any_sync(kFull, lane < n && !dw_lane_ok(pw))) {
+        r = 0.0;
+        for (int j = lane; j < n; j += 32) {
+            const double y = (double)lds1(at_w + 4u * (uint32_t)j);
+            r = __fma_rn(y, y, r);
+        }
+        __syncwarp();
+    }
+    return r;
+}
+
+template <bool HM, bool PE, bool SW, bool SH>
+__global__ void __launch_bounds__(Ring2<SH>::kThreads, 1)
     k_update(const __grid_constant__ Table<kNP2> tab, const __grid_constant__ Scalars sc) {
     extern __shared__ __align__(128) unsigned char smem[];
     // The first launch of the pass issues w and m of its first tiles at once: it starts only when
@@ -1499,12 +1775,12 @@ __global__ void __launch_bounds__(Ring2::kThreads, 1)
     const bool use_se = PE && scaled;
     const int ns = 2 + (HM ? 1 : 0) + (use_se ? 1 : 0);
     const int role = !HM && lane == 2 ? 3 : (lane < 4 ? lane : 0);
-    constexpr int CH = Ring2::tile_elems(2 + (HM ? 1 : 0) + (PE ? 1 : 0));
+    constexpr int CH = Ring2<false>::tile_elems(2 + (HM ? 1 : 0) + (PE ? 1 : 0));
     constexpr int COLS = CH / 128;
     const uint32_t w_off = (uint32_t)(CH * 4);
     const uint32_t m_off = (uint32_t)(2 * CH * 4);
     const uint32_t se_off = (uint32_t)((HM ? 3 : 2) * CH * 4);
-    Stream<Ring2> st;
+    Stream<Ring2<SH>, SH> st;
     int c = st.start(smem, tab.nc, sc.tiles + 2, sc.evict_first != 0);
     TilePos q = {};
     if (c >= 0) q = st.issue(tab, c, chunk, role, ns, early ? 1 : 0);
@@ -1512,7 +1788,7 @@ __global__ void __launch_bounds__(Ring2::kThreads, 1)
     if (early) {
         grid_wait();
         grid_launch_dependents();
-        if (c >= 0) st.issue_below(q, 1, chunk);
+        if (c >= 0) st.issue_below(q, 1, ns, chunk);
         scaled = take_branch();
     }
     const uint32_t stage = st.stage;
@@ -1526,7 +1802,7 @@ __global__ void __launch_bounds__(Ring2::kThreads, 1)
     float ct = c_all;
     while (c >= 0) {
         // fp32 |w|^2 of the tiles' shared-memory columns, scaled by 2^(2e) (e coded in `ecode`);
-        // a tile with elements loaded one by one (fp64, rare) is stored at once instead.
+        // a tile with elements taken one by one is stored at once instead.
         float pend[kPend];
         unsigned ecode = 0u;
         int ptensor[kPend];  // global index of each pending tile's tensor, -1: none
@@ -1597,19 +1873,29 @@ __global__ void __launch_bounds__(Ring2::kThreads, 1)
                 ew = sq_range_exp(aw);
                 if (ew) aw = w_cols_scaled(stage + w_off, nv, pow2f(ew));
             }
-            __syncwarp();
+            if constexpr (SH) {
+                if (!st.tc.aligned)
+                    awt = update_shifted<HM, PE, SW>(stage, ptr, q.begin, (int)(q.end - q.begin), ct,
+                                                     use_se, sc);
+            }
             const long long n = q.end - q.begin;
             const bool tile_tail = 4 * (long long)nv < n;  // the same in every lane
-            for (long long jj = 4 * (long long)nv + lane; jj < n; jj += 32) {
-                const float g = __ldcs(ptr[0] + q.begin + jj);
-                float w = wp[jj];
-                float m = HM ? mp[jj] : 0.f;
-                const float cj = use_se ? __ldcs(ptr[3] + q.begin + jj) : (PE ? 1.f : ct);
-                if (SW) awt = __fma_rn((double)w, (double)w, awt);
-                sgd1(g, cj, w, m, sc, HM);
-                wp[jj] = w;
-                if (HM) mp[jj] = m;
+            if (!SH || st.tc.aligned) {
+                // The last n % 4 elements: from the stage (SH) or by plain loads.
+                for (long long jj = 4 * (long long)nv + lane; jj < n; jj += 32) {
+                    const uint32_t o = stage + 4u * (uint32_t)jj;
+                    const float g = SH ? lds1(o) : __ldcs(ptr[0] + q.begin + jj);
+                    float w = SH ? lds1(o + w_off) : wp[jj];
+                    float m = !HM ? 0.f : SH ? lds1(o + m_off) : mp[jj];
+                    const float cj = !use_se ? (PE ? 1.f : ct)
+                                     : SH    ? lds1(o + se_off) : __ldcs(ptr[3] + q.begin + jj);
+                    if (SW) awt = __fma_rn((double)w, (double)w, awt);
+                    sgd1(g, cj, w, m, sc, HM);
+                    wp[jj] = w;
+                    if (HM) mp[jj] = m;
+                }
             }
+            __syncwarp();
             const int tg = q.tg;
             c = st.next();
             if (c >= 0) q = st.issue(tab, c, chunk, role, ns);
@@ -1705,9 +1991,26 @@ __global__ void __launch_bounds__(kScaleThreads)
                                                      scale1(x[u].z, y[u].z, sc), scale1(x[u].w, y[u].w, sc)));
             }
         }
+        // The tail, or a tensor off a 16-byte boundary: eight rows of 32 elements per step, every
+        // load issued before the first store (the output may not be assumed distinct, so the
+        // compiler would keep them in turn).
         const long long n = q.end - q.begin;
-        for (long long j = 4 * (long long)nv + lane; j < n; j += 32)
-            o[j] = scale1(__ldcs(a + j), __ldcs(b + j), sc);
+        for (long long j0 = 4 * (long long)nv + lane; j0 < n; j0 += 8 * 32) {
+            float x[8], y[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const long long j = j0 + 32 * u;
+                if (j < n) {
+                    x[u] = __ldcs(a + j);
+                    y[u] = __ldcs(b + j);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const long long j = j0 + 32 * u;
+                if (j < n) o[j] = scale1(x[u], y[u], sc);
+            }
+        }
     }
 }
 
@@ -1727,11 +2030,11 @@ inline int replica_slot(int K) {
 // Tile sizes: the smallest a pass can use for K replicas sizes the workspace.
 inline int chunk1(int K, bool rw, bool ss) {
     const int streams = K + (rw ? 1 : 0) + (ss ? 1 : 0);
-    return rw ? Ring1W::tile_elems(streams) : Ring1::tile_elems(streams);
+    return rw ? Ring1W<0, false>::tile_elems(streams) : Ring1<false>::tile_elems(streams);
 }
-inline int chunk2(bool hm, bool pe) { return Ring2::tile_elems(2 + (hm ? 1 : 0) + (pe ? 1 : 0)); }
+inline int chunk2(bool hm, bool pe) { return Ring2<false>::tile_elems(2 + (hm ? 1 : 0) + (pe ? 1 : 0)); }
 // No pass-1 tile is smaller: K (+1 with g_small) streams in 36 KB, or K + 1 in 45 KB.
-inline int chunk1_min(int K) { return Ring1::tile_elems(K + 1 + (K == 1 ? 1 : 0)); }
+inline int chunk1_min(int K) { return Ring1<false>::tile_elems(K + 1 + (K == 1 ? 1 : 0)); }
 inline int chunk2_min() { return chunk2(true, true); }
 
 struct Plan {
@@ -1871,18 +2174,19 @@ struct TableCache {
 // launches `kernel` once per block.
 // fill(p, ptrs) writes tensor p's pointers.  With a cache, the blocks are taken from it, or
 // built once and kept there.
-template <int NP, typename Kernel, typename Fill>
-int launch_streaming(Kernel kernel, int n, const int64_t *numels, int chunk, int threads,
-                     int smem, const Scalars &sc, int grid_override, cudaStream_t stream,
+template <int NP>
+struct StreamKernel {
+    void (*fn)(Table<NP>, Scalars);
+    int smem;
+};
+// kernel: for launches whose tensors are all 16-byte aligned; shifted: for the others.
+template <int NP, typename Fill>
+int launch_streaming(StreamKernel<NP> kernel, StreamKernel<NP> shifted, int n,
+                     const int64_t *numels, int chunk, int threads, const Scalars &sc, int grid_override, cudaStream_t stream,
                      Fill fill, TableCache *cache = nullptr) {
     using T = Table<NP>;
-    const int grid_cap = resident_ctas((const void *)kernel, threads, smem);
-    if (grid_cap <= 0) {
-        g_last_cuda = (int)cudaGetLastError();
-        return TULA_ERR_CUDA;
-    }
     const std::vector<std::shared_ptr<const void>> *blocks =
-        cache ? cache->find((const void *)kernel, chunk) : nullptr;
+        cache ? cache->find((const void *)kernel.fn, chunk) : nullptr;
     std::vector<std::shared_ptr<const void>> built;
     if (!blocks) {
         try {
@@ -1900,6 +2204,9 @@ int launch_streaming(Kernel kernel, int n, const int64_t *numels, int chunk, int
                     tab->numel[cnt] = numels[p];
                     tab->cstart[cnt] = nc;
                     fill(p, tab->ptr[cnt]);
+                    if (numels[p] > 0)
+                        for (const float *q : tab->ptr[cnt])
+                            if (reinterpret_cast<uintptr_t>(q) & 15u) tab->shifted = 1;
                     nc += (int)tiles_of(numels[p], chunk);
                     ++cnt;
                     ++p;
@@ -1915,7 +2222,7 @@ int launch_streaming(Kernel kernel, int n, const int64_t *numels, int chunk, int
                 built.push_back(std::move(tab));
             }
             if (cache) {
-                cache->entries.push_back({(const void *)kernel, chunk, std::move(built)});
+                cache->entries.push_back({(const void *)kernel.fn, chunk, std::move(built)});
                 blocks = &cache->entries.back().blocks;
             }
         } catch (const std::bad_alloc &) {
@@ -1925,9 +2232,15 @@ int launch_streaming(Kernel kernel, int n, const int64_t *numels, int chunk, int
     }
     for (const auto &b : *blocks) {
         const T &tab = *static_cast<const T *>(b.get());
-        int grid = grid_override > 0 ? grid_override : grid_cap;
+        const StreamKernel<NP> &k = tab.shifted ? shifted : kernel;
+        int grid = resident_ctas((const void *)k.fn, threads, k.smem);
+        if (grid <= 0) {
+            g_last_cuda = (int)cudaGetLastError();
+            return TULA_ERR_CUDA;
+        }
+        if (grid_override > 0) grid = grid_override;
         grid = std::max(1, std::min(grid, tab.nc));
-        const int rc = launch_pdl(kernel, grid, threads, smem, stream, tab, sc);
+        const int rc = launch_pdl(k.fn, grid, threads, k.smem, stream, tab, sc);
         if (rc) return rc;
     }
     return TULA_OK;
@@ -1984,9 +2297,13 @@ template <int KT, bool WM, bool RW, bool SS, bool PR, typename Fill>
 int run_reduce_k(int K, int n, const int64_t *numels, const Scalars &sc, int grid, cudaStream_t s,
                  Fill fill, TableCache *cache) {
     const int chunk = chunk1(K, RW, SS);
-    return launch_streaming<P1<KT>::NP>(k_reduce<KT, WM, RW, SS, PR>, n, numels, chunk,
-                                       Ring1Of<RW>::kThreads, Ring1Of<RW>::kSmemBytes, sc, grid,
-                                       s, fill, cache);
+    constexpr int NP = P1<KT>::NP;
+    using R = Ring1Of<KT, RW, false>;
+    const StreamKernel<NP> kernel{k_reduce<KT, WM, RW, SS, PR, false>, R::kSmemBytes};
+    const StreamKernel<NP> shifted{k_reduce<KT, WM, RW, SS, PR, true>,
+                                   Ring1Of<KT, RW, true>::kSmemBytes};
+    return launch_streaming<NP>(kernel, shifted, n, numels, chunk, R::kThreads, sc, grid, s, fill,
+                                cache);
 }
 
 template <bool WM, bool RW, bool SS, bool PR, typename Fill>
@@ -2042,9 +2359,9 @@ int tula_ags_workspace_size(const int64_t *numels, int n_tensors, int K, size_t 
 
 int tula_ags_chunk_elems(int pass, int streams) {
     if (streams < 1 || streams > TULA_MAX_K + 2) return TULA_ERR_ARG;
-    if (pass == 1) return Ring1::tile_elems(streams);
-    if (pass == 2 && streams <= 4) return Ring2::tile_elems(streams);
-    if (pass == 3) return Ring1W::tile_elems(streams);
+    if (pass == 1) return Ring1<false>::tile_elems(streams);
+    if (pass == 2 && streams <= 4) return Ring2<false>::tile_elems(streams);
+    if (pass == 3) return Ring1W<0, false>::tile_elems(streams);
     return TULA_ERR_ARG;
 }
 
@@ -2218,9 +2535,10 @@ int run_step(float *const *param_ptrs, float *const *grad_ptrs, float *const *mo
     const bool hm = mom_ptrs != nullptr;
     const bool sw = hp->layer_stats != nullptr && !lars;  // the update takes |w|^2
     const int c2 = chunk2(hm, per_elem);
-#define TULA_UPD(HM, PE, SW)                                                                \
-    launch_streaming<kNP2>(k_update<HM, PE, SW>, n, numels, c2, Ring2::kThreads,             \
-                           Ring2::kSmemBytes, sc, hp->grid_ctas, s, fill2, cache)
+#define TULA_UPD(HM, PE, SW)                                                                       \
+    launch_streaming<kNP2>({k_update<HM, PE, SW, false>, Ring2<false>::kSmemBytes},                 \
+                           {k_update<HM, PE, SW, true>, Ring2<true>::kSmemBytes}, n, numels, c2,    \
+                           Ring2<false>::kThreads, sc, hp->grid_ctas, s, fill2, cache)
     if (hm) {
         if (per_elem) rc = sw ? TULA_UPD(true, true, true) : TULA_UPD(true, true, false);
         else rc = sw ? TULA_UPD(true, false, true) : TULA_UPD(true, false, false);
@@ -2414,9 +2732,8 @@ int tula_ags_update_scale(const float *const *g_small, const float *const *g_lar
             dst[1] = g_large[p];
             dst[2] = hp->scale_elem[p];
         };
-        return launch_streaming<kNP3>(k_scale_elem, n, numels, 4096, kScaleThreads, 0, sc,
-                                      hp->grid_ctas, s,
-                                      fill);
+        return launch_streaming<kNP3>({k_scale_elem, 0}, {k_scale_elem, 0}, n, numels, 4096,
+                                      kScaleThreads, sc, hp->grid_ctas, s, fill);
     }
     int rc = check_ws(hp->workspace, hp->workspace_bytes, n, pl);
     if (rc) return rc;

@@ -805,3 +805,53 @@ def test_branch_at_the_rounding_boundary_of_delta(delta):
     got = st.state.cpu().numpy()
     assert np.isinf(got[2]) and got[3] == 0.0
     assert st.error() == 0
+
+
+@pytest.mark.parametrize("K", [1, 3, 4, 8, 16])
+@pytest.mark.parametrize("rule,gran", [(T.TULA_RULE_AGS, T.TULA_SCALE_PER_TENSOR),
+                                       (T.TULA_RULE_LARS, T.TULA_SCALE_PER_TENSOR),
+                                       (T.TULA_RULE_AGS, T.TULA_SCALE_PER_ELEMENT)])
+def test_streams_at_different_alignments(K, rule, gran, monkeypatch):
+    """Tensors packed back to back, every role starting at its own offset within 16 bytes (the
+    weights, the momentum and each replica at others), with sizes around a granule, a row of lanes
+    and a tile: the mean bitwise, everything else as the oracle.  Such tiles keep float-float sums:
+    norms are within 75 * 2^-46 = 1.1e-12 of the oracle's (a lane and component adds at most
+    9216 / 128 = 72 squares and the two tree steps after them, below 2^-46 each)."""
+    sizes = [1, 2, 3, 4, 5, 6, 7, 8, 9, 31, 33, 127, 128, 129, 131, 1021]
+    for t in (T.tula_ags_chunk_elems(1, K), T.tula_ags_chunk_elems(2, 3),
+              T.tula_ags_chunk_elems(3, K + 1)):
+        sizes += [t - 3, t - 1, t, t + 1, t + 2, t + 3, 2 * t + 1, 3 * t - 2]
+    ps = W.ParamSet("packed")
+    for n in sizes:
+        ps.add((n,), W.KIND_NORMAL)
+    plain = W.allocate
+
+    def phased(*args, **kw):
+        buf = plain(*args, **kw)
+
+        def moved(flat, shift):
+            return torch.zeros(flat.numel() + 8, device=flat.device)[shift:shift + flat.numel()]
+        buf.w_flat, buf.m_flat = moved(buf.w_flat, 1), moved(buf.m_flat, 3)
+        buf.g_flats = [moved(f, (2 * k + k // 2) % 4) for k, f in enumerate(buf.g_flats)]
+        buf.w, buf.m, *g = [W._views(f, buf.offsets, ps.shapes, buf.numels)
+                            for f in (buf.w_flat, buf.m_flat, *buf.g_flats)]
+        buf.g = g
+        return buf
+
+    monkeypatch.setattr(W, "allocate", phased)
+    wl = W.workload("stress_k4", seed=211 + K, factor_range=(1e-3, 1e1), zero_patterns=False)
+    pair = Pair(wl, K=K, align=1, pset=ps, rule=rule, granularity=gran, lars_trust=0.01)
+    for i, (seed_step, mult) in enumerate(((1, 1.0), (1, 1.0), (1, 2.0))):
+        pair.step(seed_step, mult, refresh=(K > 1 and i == 0 and gran == T.TULA_SCALE_PER_TENSOR))
+    assert pair.flags == [0, 1, 0]
+    stats = torch.zeros(pair.n, T.TULA_STATS_LEN, dtype=torch.float64, device="cuda")
+    T.tula_layer_stats(pair.buf.w, pair.buf.g, stats, pair.gpu.workspace)
+    ref = O.layer_stats(W.to_numpy(pair.buf.w), [W.to_numpy(pair.buf.g[k]) for k in range(K)])
+    got = stats.cpu().numpy()
+    moved = np.array([any(t.data_ptr() % 16 for t in (pair.buf.w[p], *(g[p] for g in pair.buf.g)))
+                      for p in range(pair.n)])
+    assert moved.sum() > pair.n // 2
+    assert_stats_close(got, ref, "layer_stats")
+    for col in (T.TULA_STAT_W_SQ, T.TULA_STAT_G_SQ, T.TULA_STAT_G0_SQ):
+        assert_norm_close(got[moved, col], ref[moved, col], f"col {col}", rtol=75 * 2.0 ** -46)
+    assert pair.gpu.error() == 0
