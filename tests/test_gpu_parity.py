@@ -855,3 +855,30 @@ def test_streams_at_different_alignments(K, rule, gran, monkeypatch):
     for col in (T.TULA_STAT_W_SQ, T.TULA_STAT_G_SQ, T.TULA_STAT_G0_SQ):
         assert_norm_close(got[moved, col], ref[moved, col], f"col {col}", rtol=75 * 2.0 ** -46)
     assert pair.gpu.error() == 0
+
+
+@pytest.mark.parametrize("K", [3, 5, 6, 7, 9, 10, 11, 12, 13, 14, 15])
+def test_the_mean_of_every_significand(K):
+    """The division by a K that is no power of two, over every significand of one binade (it scales
+    with powers of two) and at the ends of fp32's range: replica 0 alone is not zero, so its mean is
+    its own quotient, which must be the correctly rounded one, bit for bit."""
+    m = torch.arange(1 << 23, 1 << 24, dtype=torch.float32, device="cuda")
+    ends = torch.tensor([0.0, -0.0, 1.0, -1.0, 2.0 ** -149, 2.0 ** -126, 2.0 ** -91, 2.0 ** -90,
+                         1.9 * 2.0 ** -91, 3.0e38, -3.4028234663852886e38, float("inf"),
+                         -float("inf"), float("nan"), 7.0 * 2.0 ** -149, 1e-30],
+                        dtype=torch.float32, device="cuda").repeat(256)
+    params = [torch.zeros_like(m), torch.zeros_like(ends)]
+    grads = [[m, ends]] + [[torch.zeros_like(p) for p in params] for _ in range(K - 1)]
+    want = [t.cpu().numpy() for t in (m, ends)]
+    step = T.AGSOptimizerStep(params, grads, stats=False)
+    step.step(0.0, 0.0, 0.0)
+    torch.cuda.synchronize()
+    with np.errstate(all="ignore"):
+        for t, w in zip(grads[0], want):
+            q = w.astype(np.float32) / np.float32(K)
+            got = t.cpu().numpy()
+            nan = np.isnan(q)
+            assert np.array_equal(np.isnan(got), nan)
+            # -0.0 + 0.0 (the other replicas) is +0.0
+            q = np.where(q == 0, np.float32(0), q)
+            assert np.array_equal(got[~nan].view(np.int32), q[~nan].view(np.int32))
