@@ -133,7 +133,7 @@ struct Table {
     int c0;     // global index of its first tile
     int nc;     // tiles in this launch
     int chunk;  // elements per tile
-    int first;  // 1 for the first launch of the pass (in issue order)
+    int seq;    // 0, 1, ... in the order of the pass's launches
     int shifted;  // 1: some tensor has a stream off a 16-byte boundary
     int pad;
     long long numel[kMaxT];
@@ -155,7 +155,7 @@ struct Scalars {
     unsigned long long *gacc;  // [kGCopies][kAccWords]: |G|^2 = every tensor's |gbar|^2
     unsigned long long *acc2;  // [tensor][kTCopies][kAccWords]: |w|^2, pass 2
     float *cand;               // [tensor]: c_p of a LARS step
-    unsigned *tiles;           // [2 * pass]: next tile to claim, [2 * pass + 1]: CTAs finished
+    unsigned *tiles;           // [4 * (seq & 1) + 2 * pass]: next tile to claim, warps finished
     const unsigned long long *g2ext;  // a sharded step's |G|^2: the ranks' shares summed (or NULL)
 };
 
@@ -805,6 +805,8 @@ struct Stream {
         ctr = counter;
         hint = evict_first;
         policy = policy_evict_first();
+        // cp.async reads through L1: nothing there from before this kernel.
+        if constexpr (SH) __threadfence();
         const unsigned v = (unsigned)warp * gridDim.x + blockIdx.x;
         return v < nc ? (int)v : -1;
     }
@@ -1233,16 +1235,16 @@ __device__ __forceinline__ void reduce_tile(uint32_t stage, int chunk, const flo
         tail = q.begin + 4 * (long long)nv < q.end;  // the same in every lane
         for (long long j = q.begin + 4 * (long long)nv + lane; j < q.end; j += 32) {
             const uint32_t o = 4u * (uint32_t)(j - q.begin);
-            const float x0 = SH ? lds1(stage + o) : __ldcs(ptr[0] + j);
+            const float x0 = SH ? lds1(stage + o) : __ldcg(ptr[0] + j);
             float s = x0;
             for (int k = 1; k < K; ++k)
-                s = __fadd_rn(s, SH ? lds1(stage + (uint32_t)(4 * k * chunk) + o) : __ldcs(ptr[k] + j));
+                s = __fadd_rn(s, SH ? lds1(stage + (uint32_t)(4 * k * chunk) + o) : __ldcg(ptr[k] + j));
             if (K > 1) {
                 s = mean1<KT>(s, sc);
                 if (WM) const_cast<float *>(ptr[0])[j] = s;
             }
-            const float y_s = !SS ? 0.f : SH ? lds1(ss_s + o) : __ldcs(ptr[P1<KT>::KS + 1] + j);
-            const float y_w = !RW ? 0.f : SH ? lds1(sw_s + o) : __ldcs(ptr[P1<KT>::KS] + j);
+            const float y_s = !SS ? 0.f : SH ? lds1(ss_s + o) : __ldcg(ptr[P1<KT>::KS + 1] + j);
+            const float y_w = !RW ? 0.f : SH ? lds1(sw_s + o) : __ldcg(ptr[P1<KT>::KS] + j);
             if (K > 1) rs = __fma_rn((double)x0, (double)x0, rs);
             rg = __fma_rn((double)s, (double)s, rg);
             if (SS) rs = __fma_rn((double)y_s, (double)y_s, rs);
@@ -1351,10 +1353,14 @@ __global__ void __launch_bounds__(Ring1Of<KT, RW, SH>::kThreads, 1)
     // The first launch of a step's pass that does not read w issues its first tiles at once: the
     // only kernel that lets it start early is the previous call's k_finish, once all before that
     // one had completed.  What it writes, the mean and the accumulators, waits for k_finish, which
-    // reads the accumulators.  Otherwise the whole CTA waits first.  The next kernel may start when
-    // that wait has passed.
-    const bool early = !RW && !SS && sc.mode == kModeStep && tab.first;
-    if (!early) {
+    // reads the accumulators.  A first launch that reads w waits whole.  The next kernel may start
+    // when that wait has passed; a later launch of the pass (more tensors than one parameter block
+    // holds) therefore finds all but its predecessor in the pass complete.  It shares no tensor
+    // with that one, and takes the other of two tile counters, so it only has to complete after it:
+    // its warps wait once their first tile is done.
+    const bool first = tab.seq == 0;
+    const bool early = !RW && !SS && sc.mode == kModeStep;
+    if (first && !early) {
         grid_wait();
         grid_launch_dependents();
     }
@@ -1365,14 +1371,15 @@ __global__ void __launch_bounds__(Ring1Of<KT, RW, SH>::kThreads, 1)
     const int ns = K + (RW ? 1 : 0) + (SS ? 1 : 0);
     const int role = lane < K ? lane : (RW && lane == K ? KS : KS + 1);
     Stream<Ring1Of<KT, RW, SH>, SH> st;
-    int c = st.start(smem, tab.nc, sc.tiles, sc.evict_first != 0);
+    int c = st.start(smem, tab.nc, sc.tiles + 4 * (tab.seq & 1), sc.evict_first != 0);
     TilePos q = {};
     if (c >= 0) q = st.issue(tab, c, chunk, role, ns);
     st.claim_first();
-    if (early) {
+    if (first && early) {
         grid_wait();
         grid_launch_dependents();
     }
+    bool to_wait = !first;
     const bool step_g2 = sc.mode == kModeStep;  // |gbar|^2 also goes into |G|^2
     // The partial sums of a batch of kPend tiles are reduced across the warp together
     // (reduce-scatter, kRS values with padding) and added into the accumulators by the lanes
@@ -1414,6 +1421,11 @@ __global__ void __launch_bounds__(Ring1Of<KT, RW, SH>::kThreads, 1)
             const int tg = q.tg;
             c = st.next();
             if (c >= 0) q = st.issue(tab, c, chunk, role, ns);
+            if (to_wait) {
+                grid_wait();
+                grid_launch_dependents();
+                to_wait = false;
+            }
             if (!PR && tile_tail) {
                 add_tile_now(sc, tg, accf, acce, accd);
                 continue;
@@ -1453,6 +1465,7 @@ __global__ void __launch_bounds__(Ring1Of<KT, RW, SH>::kThreads, 1)
             }
         }
     }
+    if (to_wait) grid_wait();
     st.finish();
 }
 
@@ -1607,7 +1620,8 @@ __device__ __forceinline__ double step_g2_of(const Scalars &sc, bool rearm) {
 }
 // The branch of this step for the update, by one warp, once the reduction has completed.
 __device__ __forceinline__ int step_branch(const Scalars &sc) {
-    const double g2_prev = sc.state[TULA_STATE_G2_PREV], steps = sc.state[TULA_STATE_STEPS];
+    const double g2_prev = __ldcg(sc.state + TULA_STATE_G2_PREV);
+    const double steps = __ldcg(sc.state + TULA_STATE_STEPS);
     return branch_from(sc, step_g2_of(sc, false), g2_prev, steps);
 }
 
@@ -1799,11 +1813,14 @@ __global__ void __launch_bounds__(Ring2<SH>::kThreads, 1)
     // The first launch of the pass issues w and m of its first tiles at once: it starts only when
     // this step's reduction (and k_lars) have started, which let it once every kernel before them
     // had completed, so both are final.  The mean follows when the kernel before has completed.
-    // The whole CTA waits per element (the stream count depends on the branch), in later launches
-    // of the pass (which share the tile counter with the launch before) and in a sharded step
-    // (whatever ran between its two calls).
-    const bool early = !PE && tab.first && sc.early_w;
-    if (!early) {
+    // The whole CTA waits per element (the stream count depends on the branch) and in a sharded
+    // step (whatever ran between its two calls).  The next kernel may start when that wait has
+    // passed: the next step's reduction reads the mean this step's has written.  A later launch of
+    // the pass only has to complete after the one before, as in k_reduce; what it reads was final
+    // when that one let it start, and it reads it through L2 (its own wait comes later).
+    const bool first = tab.seq == 0;
+    const bool early = !PE && first && sc.early_w;
+    if (first && !early) {
         grid_wait();
         grid_launch_dependents();
     }
@@ -1832,7 +1849,7 @@ __global__ void __launch_bounds__(Ring2<SH>::kThreads, 1)
     const uint32_t m_off = (uint32_t)(2 * CH * 4);
     const uint32_t se_off = (uint32_t)((HM ? 3 : 2) * CH * 4);
     Stream<Ring2<SH>, SH> st;
-    int c = st.start(smem, tab.nc, sc.tiles + 2, sc.evict_first != 0);
+    int c = st.start(smem, tab.nc, sc.tiles + 4 * (tab.seq & 1) + 2, sc.evict_first != 0);
     TilePos q = {};
     if (c >= 0) q = st.issue(tab, c, chunk, role, ns, early ? 1 : 0);
     st.claim_first();
@@ -1842,6 +1859,7 @@ __global__ void __launch_bounds__(Ring2<SH>::kThreads, 1)
         if (c >= 0) st.issue_below(q, 1, ns, chunk);
         scaled = take_branch();
     }
+    bool to_wait = !first;
     const uint32_t stage = st.stage;
     // Where a tensor's coefficient comes from (per tensor): the gradscale or s when scaled, LARS's
     // ratio, else 1.
@@ -1865,7 +1883,7 @@ __global__ void __launch_bounds__(Ring2<SH>::kThreads, 1)
 #pragma unroll 1
         for (int p = 0; p < kPend && c >= 0; ++p) {
             if (q.tg != cand_t) {  // c_p changes only with the tensor
-                if (cand_of) ct = cand_of[q.tg];
+                if (cand_of) ct = __ldcg(cand_of + q.tg);
                 cand_t = q.tg;
             }
             if (!st.arrived(sc)) {
@@ -1935,11 +1953,11 @@ __global__ void __launch_bounds__(Ring2<SH>::kThreads, 1)
                 // The last n % 4 elements: from the stage (SH) or by plain loads.
                 for (long long jj = 4 * (long long)nv + lane; jj < n; jj += 32) {
                     const uint32_t o = stage + 4u * (uint32_t)jj;
-                    const float g = SH ? lds1(o) : __ldcs(ptr[0] + q.begin + jj);
-                    float w = SH ? lds1(o + w_off) : wp[jj];
-                    float m = !HM ? 0.f : SH ? lds1(o + m_off) : mp[jj];
+                    const float g = SH ? lds1(o) : __ldcg(ptr[0] + q.begin + jj);
+                    float w = SH ? lds1(o + w_off) : __ldcg(wp + jj);
+                    float m = !HM ? 0.f : SH ? lds1(o + m_off) : __ldcg(mp + jj);
                     const float cj = !use_se ? (PE ? 1.f : ct)
-                                     : SH    ? lds1(o + se_off) : __ldcs(ptr[3] + q.begin + jj);
+                                     : SH    ? lds1(o + se_off) : __ldcg(ptr[3] + q.begin + jj);
                     if (SW) awt = __fma_rn((double)w, (double)w, awt);
                     sgd1(g, cj, w, m, sc, HM);
                     wp[jj] = w;
@@ -1950,6 +1968,11 @@ __global__ void __launch_bounds__(Ring2<SH>::kThreads, 1)
             const int tg = q.tg;
             c = st.next();
             if (c >= 0) q = st.issue(tab, c, chunk, role, ns);
+            if (to_wait) {
+                grid_wait();
+                grid_launch_dependents();
+                to_wait = false;
+            }
             if (SW) {
                 if (tile_tail) {
                     add_w_tile_now(acc2_of(sc, tg), aw, ew, awt);
@@ -1977,6 +2000,7 @@ __global__ void __launch_bounds__(Ring2<SH>::kThreads, 1)
             }
         }
     }
+    if (to_wait) grid_wait();
     st.finish();
 }
 
@@ -2111,7 +2135,7 @@ WsLayout ws_layout(int n_tensors, const Plan &) {
     WsLayout L;
     L.flags = take(sizeof(int) * 4);
     L.err = take(sizeof(unsigned) * 4);
-    L.tiles = take(sizeof(unsigned) * 4);
+    L.tiles = take(sizeof(unsigned) * 8);
     L.acc1 = take(acc * kAcc * kTCopies * (size_t)n_tensors);
     L.gacc = take(acc * kGCopies);
     L.acc2 = take(acc * kTCopies * (size_t)n_tensors);
@@ -2249,7 +2273,7 @@ int launch_streaming(StreamKernel<NP> kernel, StreamKernel<NP> shifted, int n,
                 tab->t0 = p;
                 tab->c0 = (int)c_global;
                 tab->chunk = chunk;
-                tab->first = p == 0 ? 1 : 0;
+                tab->seq = (int)built.size();
                 int cnt = 0, nc = 0;
                 while (p < n && cnt < T::kMaxT) {
                     tab->numel[cnt] = numels[p];
