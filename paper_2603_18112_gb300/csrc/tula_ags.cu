@@ -1318,31 +1318,24 @@ __device__ __forceinline__ unsigned long long *acc2_of(const Scalars &sc, int tg
     return sc.acc2 + ((size_t)tg * kTCopies + (blockIdx.x & (kTCopies - 1))) * kAccWords;
 }
 
-// A default-mode tile with elements taken one by one (the last tile of a tensor whose size is
-// not a multiple of 4, or a misaligned tensor): its sums are reduced across the warp at once,
-// fp32 part and fp64 part, and lane 0 adds both into the tensor's accumulators.
-__device__ __noinline__ void add_tile_now(const Scalars &sc, int tg, const float (&accf)[kAcc],
-                                          const int (&acce)[kAcc], const double (&accd)[kAcc]) {
-    float f[kAcc];
+// The fp64 squares of a default-mode tile's tail: the up to three lanes that hold an element each
+// add it themselves, exactly, so that no warp-wide fp64 tree is needed.
+__device__ __forceinline__ void add_tail(const Scalars &sc, int tg, const double (&accd)[kAcc]) {
+    if (accd[0] == 0.0 && accd[1] == 0.0 && accd[2] == 0.0) return;  // (a NaN goes on)
+#pragma unroll 1
+    for (int a = 0; a < kAcc; ++a) {
+        const double d = a == 0 ? accd[0] : a == 1 ? accd[1] : accd[2];
+        acc_add_f64(acc1_of(sc, tg, a), d);
+        if (a == 0 && sc.mode == kModeStep) acc_add_f64(gacc_of(sc), d);
+    }
+}
+// The fp64 sums of a shifted tile, reduced across the warp and added by lane 0.
+__device__ __noinline__ void add_shifted(const Scalars &sc, int tg, const double (&accd)[kAcc]) {
     double d[kAcc];
 #pragma unroll
-    for (int a = 0; a < kAcc; ++a) {
-        f[a] = accf[a];
-        d[a] = accd[a];
-    }
-    warp_sums<kAcc>(f);
+    for (int a = 0; a < kAcc; ++a) d[a] = accd[a];
     warp_sums<kAcc>(d);
-    if ((threadIdx.x & 31) == 0) {
-#pragma unroll
-        for (int a = 0; a < kAcc; ++a) {
-            acc_add_f32(acc1_of(sc, tg, a), f[a], -2 * acce[a]);
-            acc_add_f64(acc1_of(sc, tg, a), d[a]);
-        }
-        if (sc.mode == kModeStep) {
-            acc_add_f32(gacc_of(sc), f[0], -2 * acce[0]);
-            acc_add_f64(gacc_of(sc), d[0]);
-        }
-    }
+    if ((threadIdx.x & 31) == 0) add_tail(sc, tg, d);
 }
 
 template <int KT, bool WM, bool RW, bool SS, bool PR, bool SH>
@@ -1388,8 +1381,8 @@ __global__ void __launch_bounds__(Ring1Of<KT, RW, SH>::kThreads, 1)
     static_assert(kPend * kAcc <= kRS, "one reduce-scatter per batch");
     while (c >= 0) {
         // PR: the lanes' fp64 sums.  Default: fp32 sums of the shared-memory columns, scaled by
-        // 2^(2e) with e coded in two bits per value in `ecode` (same in every lane); a tile with
-        // elements taken one by one is stored at once instead (add_tile_now).
+        // 2^(2e) with e coded in two bits per value in `ecode` (same in every lane); a tail's fp64
+        // squares, and a shifted tile's sums, are added at once instead.
         double pendd[PR ? kRS : 1];
         float pendf[PR ? 1 : kRS];
         unsigned ecode = 0u;
@@ -1419,6 +1412,7 @@ __global__ void __launch_bounds__(Ring1Of<KT, RW, SH>::kThreads, 1)
                                             accd, accf, acce, tcode, tile_tail);
             __syncwarp();
             const int tg = q.tg;
+            const bool shifted = SH && !st.tc.aligned;
             c = st.next();
             if (c >= 0) q = st.issue(tab, c, chunk, role, ns);
             if (to_wait) {
@@ -1426,9 +1420,14 @@ __global__ void __launch_bounds__(Ring1Of<KT, RW, SH>::kThreads, 1)
                 grid_launch_dependents();
                 to_wait = false;
             }
-            if (!PR && tile_tail) {
-                add_tile_now(sc, tg, accf, acce, accd);
-                continue;
+            if constexpr (!PR) {
+                if (tile_tail) {
+                    if (SH && shifted) {
+                        add_shifted(sc, tg, accd);
+                        continue;
+                    }
+                    add_tail(sc, tg, accd);
+                }
             }
 #pragma unroll
             for (int i = 0; i < kPend; ++i) {
@@ -1738,19 +1737,6 @@ __device__ __noinline__ float w_cols_scaled(uint32_t w_stage, int nv, float f) {
     return a;
 }
 
-// A tile of the update with elements taken one by one: its |w|^2 (fp32 part scaled by 2^(2e),
-// fp64 part) reduced across the warp at once and added into the accumulator A by lane 0.
-__device__ __noinline__ void add_w_tile_now(unsigned long long *A, float aw, int e, double awt) {
-    float f[1] = {aw};
-    double d[1] = {awt};
-    warp_sums<1>(f);
-    warp_sums<1>(d);
-    if ((threadIdx.x & 31) == 0) {
-        acc_add_f32(A, f[0], -2 * e);
-        acc_add_f64(A, d[0]);
-    }
-}
-
 // A tile of a tensor off a 16-byte boundary, as tile_shifted() of pass 1: four elements per lane
 // and step.  Returns the lane's |w|^2 (float-float pairs, to fp64 once) when the statistics want it.
 template <bool HM, bool PE, bool SW>
@@ -1871,7 +1857,7 @@ __global__ void __launch_bounds__(Ring2<SH>::kThreads, 1)
     float ct = c_all;
     while (c >= 0) {
         // fp32 |w|^2 of the tiles' shared-memory columns, scaled by 2^(2e) (e coded in `ecode`);
-        // a tile with elements taken one by one is stored at once instead.
+        // a tail's fp64 squares, and a shifted tile's sum, are added at once instead.
         float pend[kPend];
         unsigned ecode = 0u;
         int ptensor[kPend];  // global index of each pending tile's tensor, -1: none
@@ -1966,6 +1952,7 @@ __global__ void __launch_bounds__(Ring2<SH>::kThreads, 1)
             }
             __syncwarp();
             const int tg = q.tg;
+            const bool shifted = SH && !st.tc.aligned;
             c = st.next();
             if (c >= 0) q = st.issue(tab, c, chunk, role, ns);
             if (to_wait) {
@@ -1974,18 +1961,21 @@ __global__ void __launch_bounds__(Ring2<SH>::kThreads, 1)
                 to_wait = false;
             }
             if (SW) {
-                if (tile_tail) {
-                    add_w_tile_now(acc2_of(sc, tg), aw, ew, awt);
-                } else {
-#pragma unroll
-                    for (int i = 0; i < kPend; ++i) {
-                        if (p == i) {
-                            ptensor[i] = tg;
-                            pend[i] = aw;
-                        }
-                    }
-                    if (ew) ecode |= scale_code(ew) << (2 * p);
+                if (SH && shifted) {
+                    double d[1] = {awt};
+                    warp_sums<1>(d);
+                    if (lane == 0) acc_add_f64(acc2_of(sc, tg), d[0]);
+                    continue;
                 }
+                if (tile_tail && lane < 3) acc_add_f64(acc2_of(sc, tg), awt);  // as add_tail
+#pragma unroll
+                for (int i = 0; i < kPend; ++i) {
+                    if (p == i) {
+                        ptensor[i] = tg;
+                        pend[i] = aw;
+                    }
+                }
+                if (ew) ecode |= scale_code(ew) << (2 * p);
             }
         }
         if (SW) {
