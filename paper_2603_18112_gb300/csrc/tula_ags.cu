@@ -125,9 +125,9 @@ enum Mode { kModeStep = 0, kModeStats = 1, kModeScale = 2 };
 // ----------------------------------------------------------------------------
 
 constexpr int kHints = 160, kHintTiles = 8;  // covers the first tiles of 152 SMs' 8 warps
-template <int NP>
+template <int NP, int MaxT>
 struct Table {
-    static constexpr int kMaxT = (kParamBudget - 64 - 2 * kHints) / (NP * 8 + 12);
+    static constexpr int kMaxT = MaxT;
     int n;      // tensors in this launch
     int t0;     // global index of its first tensor
     int c0;     // global index of its first tile
@@ -141,6 +141,14 @@ struct Table {
     unsigned short hint[kHints];  // tensor of tile min(i * kHintTiles, nc - 1)
     const float *ptr[kMaxT][NP];
 };
+// A launch of few tensors passes a smaller block: three launches with 31 KB each cost the host
+// 8.0 us, with 8 KB 5.6 us, and a call that waits for them 17.0 and 13.2 us.
+template <int NP>
+constexpr int kFullT = (kParamBudget - 64 - 2 * kHints) / (NP * 8 + 12);
+template <int NP>
+constexpr int kSmallT = NP <= 10 ? 168 : kFullT<NP>;  // 7.7 KB for the update, 16 KB for K = 8
+template <int NP, bool Small>
+using TableOf = Table<NP, Small ? kSmallT<NP> : kFullT<NP>>;
 
 struct Scalars {
     int K, rule, gran, force, refresh, mode, n_total, read_w;
@@ -627,8 +635,8 @@ __device__ __forceinline__ int find_tensor(const int *cstart, int lo, int hi, in
 // first, then a search over the rest.
 struct Walker {
     int t = -1;
-    template <int NP>
-    __device__ __forceinline__ int to(const Table<NP> &tab, int c) {
+    template <typename Tab>
+    __device__ __forceinline__ int to(const Tab &tab, int c) {
         if (t < 0) {
             // The warp's first tile: the table is not in the constant cache yet, and the eight
             // or so steps of a search, each a miss, took 2 us.  Two with the hint.
@@ -650,8 +658,8 @@ struct TilePos {
     long long begin, end;
 };
 
-template <int NP>
-__device__ __forceinline__ TilePos locate(const Table<NP> &tab, int c, int t, int chunk) {
+template <typename Tab>
+__device__ __forceinline__ TilePos locate(const Tab &tab, int c, int t, int chunk) {
     TilePos q;
     q.t = t;
     q.tg = tab.t0 + t;
@@ -680,8 +688,8 @@ struct TensorCache {
     const float *mine = nullptr;
     bool aligned = false;  // every stream at a 16-byte boundary
     int nv = 0;            // whole float4 columns of the last tile asked for (0: a shifted tile)
-    template <int NP>
-    __device__ __forceinline__ TilePos at(const Table<NP> &tab, int c, int chunk, int role, int ns) {
+    template <typename Tab>
+    __device__ __forceinline__ TilePos at(const Tab &tab, int c, int chunk, int role, int ns) {
         const int tn = walk.to(tab, c);
         if (tn != t) {
             t = tn;
@@ -824,8 +832,8 @@ struct Stream {
     }
     // Issues tile c, or of it only streams `from` .. ns - 1, the rest left to issue_below();
     // every lane has read what the stage held (a __syncwarp ago).
-    template <int NP>
-    __device__ __forceinline__ TilePos issue(const Table<NP> &tab, int c, int chunk, int role,
+    template <typename Tab>
+    __device__ __forceinline__ TilePos issue(const Tab &tab, int c, int chunk, int role,
                                              int ns, int from = 0) {
         const int lane = threadIdx.x & 31;
         const TilePos q = tc.at(tab, c, chunk, role, ns);
@@ -1338,9 +1346,9 @@ __device__ __noinline__ void add_shifted(const Scalars &sc, int tg, const double
     if ((threadIdx.x & 31) == 0) add_tail(sc, tg, d);
 }
 
-template <int KT, bool WM, bool RW, bool SS, bool PR, bool SH>
+template <int KT, bool WM, bool RW, bool SS, bool PR, bool SH, bool Small>
 __global__ void __launch_bounds__(Ring1Of<KT, RW, SH>::kThreads, 1)
-    k_reduce(const __grid_constant__ Table<P1<KT>::NP> tab, const __grid_constant__ Scalars sc) {
+    k_reduce(const __grid_constant__ TableOf<P1<KT>::NP, Small> tab, const __grid_constant__ Scalars sc) {
     constexpr int KS = P1<KT>::KS;
     extern __shared__ __align__(128) unsigned char smem[];
     // The first launch of a step's pass that does not read w issues its first tiles at once: the
@@ -1792,9 +1800,9 @@ __device__ __noinline__ double update_shifted(uint32_t stage, const float *const
     return r;
 }
 
-template <bool HM, bool PE, bool SW, bool SH>
+template <bool HM, bool PE, bool SW, bool SH, bool Small>
 __global__ void __launch_bounds__(Ring2<SH>::kThreads, 1)
-    k_update(const __grid_constant__ Table<kNP2> tab, const __grid_constant__ Scalars sc) {
+    k_update(const __grid_constant__ TableOf<kNP2, Small> tab, const __grid_constant__ Scalars sc) {
     extern __shared__ __align__(128) unsigned char smem[];
     // The first launch of the pass issues w and m of its first tiles at once: it starts only when
     // this step's reduction (and k_lars) have started, which let it once every kernel before them
@@ -2022,8 +2030,9 @@ __global__ void __launch_bounds__(32) k_wait_check(unsigned *err) {
 
 constexpr int kScaleThreads = 128;
 
+template <bool Small>
 __global__ void __launch_bounds__(kScaleThreads)
-    k_scale_elem(const __grid_constant__ Table<kNP3> tab, const __grid_constant__ Scalars sc) {
+    k_scale_elem(const __grid_constant__ TableOf<kNP3, Small> tab, const __grid_constant__ Scalars sc) {
     grid_wait();  // no early start for the successor: it may overwrite what this kernel reads
     const int lane = threadIdx.x & 31;
     const int warp = (int)((blockIdx.x * (unsigned)kScaleThreads + threadIdx.x) >> 5);
@@ -2151,6 +2160,13 @@ bool valid_numels(const int64_t *numels, int n, int K, Plan *pl) {
     return true;
 }
 
+// Whether some pointer of a tensor's table row lies off a 16-byte boundary.
+template <int NP>
+inline bool off_16(const float *const (&ptr)[NP]) {
+    for (const float *q : ptr)
+        if (reinterpret_cast<uintptr_t>(q) & 15u) return true;
+    return false;
+}
 inline bool aligned4(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 3u) == 0; }
 
 // One wave of resident CTAs of `kernel` on the current device (cached); sets
@@ -2221,73 +2237,104 @@ int launch_pdl(void (*kernel)(KArgs...), int grid, int threads, int smem, cudaSt
 // The launch tables of a plan (tula_ags_plan_create): for each kernel instantiation and tile
 // size, its parameter blocks, built by the first call that launches them and reused by every
 // later one (they hold only sizes and pointers, which a plan fixes).
+struct Blocks {
+    bool small = false;  // TableOf<NP, true>: one launch of few, aligned tensors
+    std::vector<std::shared_ptr<const void>> tabs;
+};
 struct TableCache {
     struct Entry {
-        const void *kernel;
+        const void *kernel;  // its instantiation for full blocks
         int chunk;
-        std::vector<std::shared_ptr<const void>> blocks;
+        Blocks blocks;
     };
     std::vector<Entry> entries;
-    const std::vector<std::shared_ptr<const void>> *find(const void *kernel, int chunk) const {
+    const Blocks *find(const void *kernel, int chunk) const {
         for (const Entry &e : entries)
             if (e.kernel == kernel && e.chunk == chunk) return &e.blocks;
         return nullptr;
     }
 };
 
-// Splits tensors [0, n) into parameter blocks of tiles of `chunk` elements and
-// launches `kernel` once per block.
-// fill(p, ptrs) writes tensor p's pointers.  With a cache, the blocks are taken from it, or
-// built once and kept there.
+// Splits tensors [0, n) into parameter blocks of type Tab of tiles of `chunk` elements.
+// fill(p, ptrs) writes tensor p's pointers.
+template <typename Tab, typename Fill>
+void build_blocks(int n, const int64_t *numels, int chunk, Fill fill,
+                  std::vector<std::shared_ptr<const void>> &tabs) {
+    long long c_global = 0;
+    int p = 0;
+    while (p < n) {
+        std::shared_ptr<Tab> tab = std::make_shared<Tab>();
+        std::memset(tab.get(), 0, sizeof(Tab));
+        tab->t0 = p;
+        tab->c0 = (int)c_global;
+        tab->chunk = chunk;
+        tab->seq = (int)tabs.size();
+        int cnt = 0, nc = 0;
+        while (p < n && cnt < Tab::kMaxT) {
+            tab->numel[cnt] = numels[p];
+            tab->cstart[cnt] = nc;
+            fill(p, tab->ptr[cnt]);
+            if (numels[p] > 0 && off_16(tab->ptr[cnt])) tab->shifted = 1;
+            nc += (int)tiles_of(numels[p], chunk);
+            ++cnt;
+            ++p;
+        }
+        tab->n = cnt;
+        tab->nc = nc;
+        tab->cstart[cnt] = nc;
+        for (int i = 0, t = 0; i < kHints; ++i) {
+            while (t + 1 < cnt && i * kHintTiles >= tab->cstart[t + 1]) ++t;
+            tab->hint[i] = (unsigned short)t;
+        }
+        c_global += nc;
+        tabs.push_back(std::move(tab));
+    }
+}
+
+// The instantiations of a streaming kernel: for launches whose tensors are all 16-byte aligned,
+// with a small parameter block and with a full one, and for the others.
 template <int NP>
-struct StreamKernel {
-    void (*fn)(Table<NP>, Scalars);
-    int smem;
+struct StreamKernels {
+    void (*small)(TableOf<NP, true>, Scalars);
+    void (*full)(TableOf<NP, false>, Scalars);
+    void (*shifted)(TableOf<NP, false>, Scalars);
+    int smem, smem_shifted;
 };
-// kernel: for launches whose tensors are all 16-byte aligned; shifted: for the others.
+template <typename Tab>
+int launch_block(void (*fn)(Tab, Scalars), const void *block, int threads, int smem,
+                 const Scalars &sc, int grid_override, cudaStream_t stream) {
+    const Tab &tab = *static_cast<const Tab *>(block);
+    int grid = resident_ctas((const void *)fn, threads, smem);
+    if (grid <= 0) {
+        g_last_cuda = (int)cudaGetLastError();
+        return TULA_ERR_CUDA;
+    }
+    if (grid_override > 0) grid = grid_override;
+    grid = std::max(1, std::min(grid, tab.nc));
+    return launch_pdl(fn, grid, threads, smem, stream, tab, sc);
+}
+// Launches a streaming kernel once per parameter block.  With a cache, the blocks are taken from
+// it, or built once and kept there.
 template <int NP, typename Fill>
-int launch_streaming(StreamKernel<NP> kernel, StreamKernel<NP> shifted, int n,
-                     const int64_t *numels, int chunk, int threads, const Scalars &sc, int grid_override, cudaStream_t stream,
+int launch_streaming(const StreamKernels<NP> &k, int n, const int64_t *numels, int chunk,
+                     int threads, const Scalars &sc, int grid_override, cudaStream_t stream,
                      Fill fill, TableCache *cache = nullptr) {
-    using T = Table<NP>;
-    const std::vector<std::shared_ptr<const void>> *blocks =
-        cache ? cache->find((const void *)kernel.fn, chunk) : nullptr;
-    std::vector<std::shared_ptr<const void>> built;
+    using SmallTab = TableOf<NP, true>;
+    using FullTab = TableOf<NP, false>;
+    const Blocks *blocks = cache ? cache->find((const void *)k.full, chunk) : nullptr;
+    Blocks built;
     if (!blocks) {
+        built.small = n <= SmallTab::kMaxT && SmallTab::kMaxT < FullTab::kMaxT;
+        for (int p = 0; p < n && built.small; ++p) {
+            const float *ptr[NP] = {};
+            if (numels[p] > 0) fill(p, ptr);
+            if (off_16(ptr)) built.small = false;
+        }
         try {
-            long long c_global = 0;
-            int p = 0;
-            while (p < n) {
-                std::shared_ptr<T> tab = std::make_shared<T>();
-                std::memset(tab.get(), 0, sizeof(T));
-                tab->t0 = p;
-                tab->c0 = (int)c_global;
-                tab->chunk = chunk;
-                tab->seq = (int)built.size();
-                int cnt = 0, nc = 0;
-                while (p < n && cnt < T::kMaxT) {
-                    tab->numel[cnt] = numels[p];
-                    tab->cstart[cnt] = nc;
-                    fill(p, tab->ptr[cnt]);
-                    if (numels[p] > 0)
-                        for (const float *q : tab->ptr[cnt])
-                            if (reinterpret_cast<uintptr_t>(q) & 15u) tab->shifted = 1;
-                    nc += (int)tiles_of(numels[p], chunk);
-                    ++cnt;
-                    ++p;
-                }
-                tab->n = cnt;
-                tab->nc = nc;
-                tab->cstart[cnt] = nc;
-                for (int i = 0, t = 0; i < kHints; ++i) {
-                    while (t + 1 < cnt && i * kHintTiles >= tab->cstart[t + 1]) ++t;
-                    tab->hint[i] = (unsigned short)t;
-                }
-                c_global += nc;
-                built.push_back(std::move(tab));
-            }
+            if (built.small) build_blocks<SmallTab>(n, numels, chunk, fill, built.tabs);
+            else build_blocks<FullTab>(n, numels, chunk, fill, built.tabs);
             if (cache) {
-                cache->entries.push_back({(const void *)kernel.fn, chunk, std::move(built)});
+                cache->entries.push_back({(const void *)k.full, chunk, std::move(built)});
                 blocks = &cache->entries.back().blocks;
             }
         } catch (const std::bad_alloc &) {
@@ -2295,17 +2342,14 @@ int launch_streaming(StreamKernel<NP> kernel, StreamKernel<NP> shifted, int n,
         }
         if (!blocks) blocks = &built;
     }
-    for (const auto &b : *blocks) {
-        const T &tab = *static_cast<const T *>(b.get());
-        const StreamKernel<NP> &k = tab.shifted ? shifted : kernel;
-        int grid = resident_ctas((const void *)k.fn, threads, k.smem);
-        if (grid <= 0) {
-            g_last_cuda = (int)cudaGetLastError();
-            return TULA_ERR_CUDA;
-        }
-        if (grid_override > 0) grid = grid_override;
-        grid = std::max(1, std::min(grid, tab.nc));
-        const int rc = launch_pdl(k.fn, grid, threads, k.smem, stream, tab, sc);
+    for (const auto &b : blocks->tabs) {
+        int rc;
+        if (blocks->small)
+            rc = launch_block(k.small, b.get(), threads, k.smem, sc, grid_override, stream);
+        else if (static_cast<const FullTab *>(b.get())->shifted)
+            rc = launch_block(k.shifted, b.get(), threads, k.smem_shifted, sc, grid_override, stream);
+        else
+            rc = launch_block(k.full, b.get(), threads, k.smem, sc, grid_override, stream);
         if (rc) return rc;
     }
     return TULA_OK;
@@ -2364,11 +2408,12 @@ int run_reduce_k(int K, int n, const int64_t *numels, const Scalars &sc, int gri
     const int chunk = chunk1(K, RW, SS);
     constexpr int NP = P1<KT>::NP;
     using R = Ring1Of<KT, RW, false>;
-    const StreamKernel<NP> kernel{k_reduce<KT, WM, RW, SS, PR, false>, R::kSmemBytes};
-    const StreamKernel<NP> shifted{k_reduce<KT, WM, RW, SS, PR, true>,
-                                   Ring1Of<KT, RW, true>::kSmemBytes};
-    return launch_streaming<NP>(kernel, shifted, n, numels, chunk, R::kThreads, sc, grid, s, fill,
-                                cache);
+    constexpr bool kSmall = kSmallT<NP> < kFullT<NP>;  // else both blocks are the same type
+    const StreamKernels<NP> k{k_reduce<KT, WM, RW, SS, PR, false, kSmall>,
+                              k_reduce<KT, WM, RW, SS, PR, false, false>,
+                              k_reduce<KT, WM, RW, SS, PR, true, false>, R::kSmemBytes,
+                              Ring1Of<KT, RW, true>::kSmemBytes};
+    return launch_streaming<NP>(k, n, numels, chunk, R::kThreads, sc, grid, s, fill, cache);
 }
 
 template <bool WM, bool RW, bool SS, bool PR, typename Fill>
@@ -2601,9 +2646,10 @@ int run_step(float *const *param_ptrs, float *const *grad_ptrs, float *const *mo
     const bool sw = hp->layer_stats != nullptr && !lars;  // the update takes |w|^2
     const int c2 = chunk2(hm, per_elem);
 #define TULA_UPD(HM, PE, SW)                                                                       \
-    launch_streaming<kNP2>({k_update<HM, PE, SW, false>, Ring2<false>::kSmemBytes},                 \
-                           {k_update<HM, PE, SW, true>, Ring2<true>::kSmemBytes}, n, numels, c2,    \
-                           Ring2<false>::kThreads, sc, hp->grid_ctas, s, fill2, cache)
+    launch_streaming<kNP2>({k_update<HM, PE, SW, false, true>, k_update<HM, PE, SW, false, false>,  \
+                            k_update<HM, PE, SW, true, false>, Ring2<false>::kSmemBytes,             \
+                            Ring2<true>::kSmemBytes},                                                \
+                           n, numels, c2, Ring2<false>::kThreads, sc, hp->grid_ctas, s, fill2, cache)
     if (hm) {
         if (per_elem) rc = sw ? TULA_UPD(true, true, true) : TULA_UPD(true, true, false);
         else rc = sw ? TULA_UPD(true, false, true) : TULA_UPD(true, false, false);
@@ -2797,8 +2843,8 @@ int tula_ags_update_scale(const float *const *g_small, const float *const *g_lar
             dst[1] = g_large[p];
             dst[2] = hp->scale_elem[p];
         };
-        return launch_streaming<kNP3>({k_scale_elem, 0}, {k_scale_elem, 0}, n, numels, 4096,
-                                      kScaleThreads, sc, hp->grid_ctas, s, fill);
+        return launch_streaming<kNP3>({k_scale_elem<true>, k_scale_elem<false>, k_scale_elem<false>, 0, 0},
+                                      n, numels, 4096, kScaleThreads, sc, hp->grid_ctas, s, fill);
     }
     int rc = check_ws(hp->workspace, hp->workspace_bytes, n, pl);
     if (rc) return rc;
