@@ -10,6 +10,9 @@ from __future__ import annotations
 import ctypes
 import math
 import re
+from array import array
+from itertools import chain
+from operator import attrgetter
 from pathlib import Path
 
 import torch
@@ -121,32 +124,51 @@ def header_functions() -> list[str]:
 # marshalling helpers
 # ---------------------------------------------------------------------------
 
-def _ptr_array(ptrs):
-    arr = (c_void_p * max(1, len(ptrs)))()
-    for i, p in enumerate(ptrs):
-        arr[i] = p or None
-    return arr
+_is_contiguous, _data_ptr, _numel = (torch.Tensor.is_contiguous, torch.Tensor.data_ptr,
+                                     torch.Tensor.numel)
+_dtype = attrgetter("dtype")
+_FLOAT32 = {torch.float32}
+
+
+def _host_array(ctype, code, values):
+    """A ctypes array over values; it keeps them alive."""
+    a = array(code, values)
+    if not a:
+        a.append(0)
+    return (ctype * len(a)).from_buffer(a)
 
 
 def _tensor_ptrs(tensors):
-    out = []
+    """The tensors' addresses (NULL for None), after checking each.  The loops run in C, about
+    0.17 us a tensor instead of 0.29: tula_layer_stats over 161 tensors and K = 8 passes 1449."""
+    try:
+        if not all(map(_is_contiguous, tensors)) or not set(map(_dtype, tensors)) <= _FLOAT32:
+            raise ValueError
+        return _host_array(c_void_p, "Q", map(_data_ptr, tensors))
+    except (TypeError, ValueError):
+        pass
+    ptrs = []  # something that is no contiguous float32 tensor: None, or an error
     for t in tensors:
         if t is None:
-            out.append(None)
+            ptrs.append(0)
             continue
         if t.dtype != torch.float32 or not t.is_contiguous():
             raise TypeError("tensors must be contiguous float32")
-        out.append(t.data_ptr())
-    return _ptr_array(out)
+        ptrs.append(t.data_ptr())
+    return _host_array(c_void_p, "Q", ptrs)
 
 
 def _numels(tensors):
-    return (ctypes.c_int64 * max(1, len(tensors)))(*[t.numel() for t in tensors])
+    try:
+        return _host_array(ctypes.c_int64, "q", map(_numel, tensors))
+    except TypeError:
+        return _host_array(ctypes.c_int64, "q", [t.numel() for t in tensors])
 
 
 def _stream_ptr(stream):
     if stream is None:
-        stream = torch.cuda.current_stream()
+        # torch.cuda.current_stream().cuda_stream without building the Stream object (2.8 us)
+        return c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
     return c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
 
 
@@ -167,7 +189,7 @@ def _replica_list(params, grads, hp, where, moms=None):
     for k, r in enumerate(grads):
         if len(r) != n:
             raise ValueError(f"{where}: replica {k} has {len(r)} tensors, params has {n}")
-    return [grads[k][p] for k in range(len(grads)) for p in range(n)]
+    return list(chain.from_iterable(grads))
 
 
 # ---------------------------------------------------------------------------
