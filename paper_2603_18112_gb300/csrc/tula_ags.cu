@@ -124,31 +124,64 @@ enum Mode { kModeStep = 0, kModeStats = 1, kModeScale = 2 };
 // Launch tables (kernel parameters)
 // ----------------------------------------------------------------------------
 
+// One launch's tensors: sizes, first tiles and pointers, in a parameter block of Bytes bytes.  The
+// arrays lie one after the other in `raw`, `np` pointers per tensor: a pointer is its role's base
+// plus a 32-bit offset in fp32 elements (a 16 GB window), with 16 more bits when some role's
+// tensors lie farther apart (`wide`).  8 to 12 bytes per tensor and 8 per pointer, as the table was
+// before, took 4096 tensors with K = 16 through 21 launches of pass 1 instead of 10, and left more
+// of the block to miss the constant cache on.
 constexpr int kHints = 160, kHintTiles = 8;  // covers the first tiles of 152 SMs' 8 warps
-template <int NP, int MaxT>
-struct Table {
-    static constexpr int kMaxT = MaxT;
-    int n;      // tensors in this launch
-    int t0;     // global index of its first tensor
-    int c0;     // global index of its first tile
-    int nc;     // tiles in this launch
-    int chunk;  // elements per tile
-    int seq;    // 0, 1, ... in the order of the pass's launches
+constexpr int kMaxRoles = TULA_MAX_K + 1;
+struct TableHead {
+    int n;        // tensors in this launch
+    int t0;       // global index of its first tensor
+    int nc;       // tiles in this launch
+    int chunk;    // elements per tile
+    int seq;      // 0, 1, ... in the order of the pass's launches
     int shifted;  // 1: some tensor has a stream off a 16-byte boundary
+    int np, wide;
+    int o_last, o_lo, o_hi;  // byte offsets in raw
     int pad;
-    long long numel[kMaxT];
-    int cstart[kMaxT + 1];  // first tile of each tensor, relative to c0; cstart[n] = nc
+    unsigned long long base[kMaxRoles];
     unsigned short hint[kHints];  // tensor of tile min(i * kHintTiles, nc - 1)
-    const float *ptr[kMaxT][NP];
+};
+template <int Bytes>
+struct Table : TableHead {
+    static constexpr int kRaw = Bytes - (int)sizeof(TableHead);
+    alignas(8) unsigned char raw[kRaw];  // cstart[n + 1], last[n], lo[n][np] [, hi[n][np]]
+    static constexpr int bytes_for(int n, int np, bool wide) {
+        return 4 * (n + 1) + (2 * n + 3) / 4 * 4 + 4 * n * np + (wide ? 2 * n * np : 0);
+    }
+    // First tile of tensor t (t = n: nc).
+    __host__ __device__ int cstart(int t) const { return reinterpret_cast<const int *>(raw)[t]; }
+    // Elements of its last tile.
+    __host__ __device__ int last(int t) const {
+        return reinterpret_cast<const unsigned short *>(raw + o_last)[t];
+    }
+    __host__ __device__ long long numel(int t) const {
+        return (long long)(cstart(t + 1) - cstart(t) - 1) * chunk + last(t);
+    }
+    __host__ __device__ float *ptr(int t, int role) const { return ptr(t, role, base[role]); }
+    __host__ __device__ float *ptr(int t, int role, unsigned long long base_of_role) const {
+        const int i = t * np + role;
+        unsigned long long e = reinterpret_cast<const unsigned *>(raw + o_lo)[i];
+        if (wide)
+            e |= (unsigned long long)reinterpret_cast<const unsigned short *>(raw + o_hi)[i] << 32;
+        return reinterpret_cast<float *>(base_of_role + 4ull * e);
+    }
+};
+// A tensor's pointers by role.
+template <typename Tab>
+struct Row {
+    const Tab &tab;
+    int t;
+    __host__ __device__ float *operator[](int role) const { return tab.ptr(t, role); }
 };
 // A launch of few tensors passes a smaller block: three launches with 31 KB each cost the host
 // 8.0 us, with 8 KB 5.6 us, and a call that waits for them 17.0 and 13.2 us.
-template <int NP>
-constexpr int kFullT = (kParamBudget - 64 - 2 * kHints) / (NP * 8 + 12);
-template <int NP>
-constexpr int kSmallT = NP <= 10 ? 168 : kFullT<NP>;  // 7.7 KB for the update, 16 KB for K = 8
-template <int NP, bool Small>
-using TableOf = Table<NP, Small ? kSmallT<NP> : kFullT<NP>>;
+template <bool Small>
+using TableOf = Table<Small ? 8 * 1024 : kParamBudget>;
+static_assert(sizeof(TableOf<true>) == 8 * 1024 && sizeof(TableOf<false>) == kParamBudget, "as sized");
 
 struct Scalars {
     int K, rule, gran, force, refresh, mode, n_total, read_w;
@@ -622,11 +655,12 @@ __device__ __forceinline__ void report_timeout(const Scalars &sc) {
 // Tile table lookups
 // ----------------------------------------------------------------------------
 
-__device__ __forceinline__ int find_tensor(const int *cstart, int lo, int hi, int c) {
-    // cstart[lo] <= c < cstart[hi]
+template <typename Tab>
+__device__ __forceinline__ int find_tensor(const Tab &tab, int lo, int hi, int c) {
+    // cstart(lo) <= c < cstart(hi)
     while (hi - lo > 1) {
         int mid = (lo + hi) >> 1;
-        if (cstart[mid] <= c) lo = mid; else hi = mid;
+        if (tab.cstart(mid) <= c) lo = mid; else hi = mid;
     }
     return lo;
 }
@@ -640,15 +674,15 @@ struct Walker {
         if (t < 0) {
             // The warp's first tile: the table is not in the constant cache yet, and the eight
             // or so steps of a search, each a miss, took 2 us.  Two with the hint.
-            if (c >= kHints * kHintTiles) return t = find_tensor(tab.cstart, 0, tab.n, c);
+            if (c >= kHints * kHintTiles) return t = find_tensor(tab, 0, tab.n, c);
             t = tab.hint[c / kHintTiles];
-            while (c >= tab.cstart[t + 1]) ++t;  // at most kHintTiles - 1 steps
+            while (c >= tab.cstart(t + 1)) ++t;  // at most kHintTiles - 1 steps
             return t;
         }
-        if (c < tab.cstart[t + 1]) return t;
+        if (c < tab.cstart(t + 1)) return t;
         ++t;
-        if (c < tab.cstart[t + 1]) return t;
-        return t = find_tensor(tab.cstart, t + 1, tab.n, c);
+        if (c < tab.cstart(t + 1)) return t;
+        return t = find_tensor(tab, t + 1, tab.n, c);
     }
 };
 
@@ -663,9 +697,9 @@ __device__ __forceinline__ TilePos locate(const Tab &tab, int c, int t, int chun
     TilePos q;
     q.t = t;
     q.tg = tab.t0 + t;
-    q.c_in_t = c - tab.cstart[t];
+    q.c_in_t = c - tab.cstart(t);
     q.begin = (long long)q.c_in_t * chunk;
-    q.end = min(q.begin + (long long)chunk, tab.numel[t]);
+    q.end = min(q.begin + (long long)chunk, tab.numel(t));
     return q;
 }
 
@@ -681,32 +715,42 @@ __device__ __forceinline__ int tile_vecs(const float *mine, int ns, const TilePo
 // The tensor of the previous tile, kept while the next tile stays in it: its
 // index, its streams' alignment and the lane's stream pointer, so a tile in
 // the same tensor needs no table look-up.
+template <bool SH>
 struct TensorCache {
     Walker walk;
     int t = -1;
     long long numel = 0;
     const float *mine = nullptr;
-    bool aligned = false;  // every stream at a 16-byte boundary
+    unsigned long long base = 0;  // of the lane's role
+    bool aligned = !SH;    // every stream at a 16-byte boundary
     int nv = 0;            // whole float4 columns of the last tile asked for (0: a shifted tile)
     template <typename Tab>
     __device__ __forceinline__ TilePos at(const Tab &tab, int c, int chunk, int role, int ns) {
         const int tn = walk.to(tab, c);
         if (tn != t) {
             t = tn;
-            numel = tab.numel[t];
-            mine = (threadIdx.x & 31) < ns ? tab.ptr[t][role] : nullptr;
-            const unsigned low =
-                (threadIdx.x & 31) < ns ? (unsigned)(reinterpret_cast<uintptr_t>(mine) & 15u) : 0u;
-            aligned = __reduce_or_sync(kFull, low) == 0u;
+            numel = tab.numel(t);
+            if (base == 0ull) base = tab.base[role];
+            mine = (threadIdx.x & 31) < ns ? tab.ptr(t, role, base) : nullptr;
+            if constexpr (SH) {
+                const unsigned low =
+                    (threadIdx.x & 31) < ns ? (unsigned)(reinterpret_cast<uintptr_t>(mine) & 15u) : 0u;
+                aligned = __reduce_or_sync(kFull, low) == 0u;
+            }
         }
         TilePos q;
         q.t = t;
         q.tg = tab.t0 + t;
-        q.c_in_t = c - tab.cstart[t];
+        q.c_in_t = c - tab.cstart(t);
         q.begin = (long long)q.c_in_t * chunk;
         q.end = min(q.begin + (long long)chunk, numel);
         nv = (aligned && q.end > q.begin) ? (int)((q.end - q.begin) >> 2) : 0;
         return q;
+    }
+    // Stream i's pointer, from the lane that holds it (the table may miss the constant cache).
+    __device__ __forceinline__ float *stream(int i) const {
+        return reinterpret_cast<float *>(
+            __shfl_sync(kFull, (unsigned long long)reinterpret_cast<uintptr_t>(mine), i));
     }
 };
 
@@ -793,7 +837,7 @@ struct Stream {
     unsigned pend = 0;  // lane 0: the claim in flight
     uint64_t policy;
     bool hint;
-    TensorCache tc;  // of the tile in the stage (or on its way there)
+    TensorCache<SH> tc;  // of the tile in the stage (or on its way there)
     bool edges = false;  // SH: it came partly by cp.async
 
     // Barrier init; returns this warp's first tile (-1: none).  Called by the whole CTA.
@@ -920,14 +964,8 @@ struct Stream {
 // it valid over the whole fp32 range: a tile whose fp32 sums would overflow or
 // lose precision to underflow is summed again from shared memory with its
 // elements scaled by an exact power of two, and the scaling is undone in fp64.
-// Pointer roles per tensor: [0, K) replicas, KS = w, KS + 1 = g_small.
+// Pointer roles per tensor: [0, K) replicas, K = w (RW) or g_small (SS).
 // Stage streams: replicas 0..K-1, then w (RW), then g_small (SS).
-
-template <int KT>
-struct P1 {
-    static constexpr int KS = KT > 0 ? KT : TULA_MAX_K;
-    static constexpr int NP = KS + 2;
-};
 
 // One float4 column of a tile: mean, squares.  x0 = replica 0, s = sum.
 template <int KT, bool WM, bool RW, bool SS, bool PR>
@@ -1021,22 +1059,23 @@ __device__ __noinline__ F3 tile_cols_scaled(uint32_t stage, int chunk, int nv, c
 // mode: the elements of such tensors used to be squared in fp64, and these sums keep that
 // precision (relative error ~1e-15 a lane) without GB300's slow FP64 pipe.  Returns the lane's
 // sums; out of line, so that the streaming loop of aligned tensors keeps its shape.
-template <int KT, bool WM, bool RW, bool SS>
-__device__ __noinline__ D3 tile_shifted(uint32_t stage, int chunk, const float *const *ptr,
+template <int KT, bool WM, bool RW, bool SS, typename Tab>
+__device__ __noinline__ D3 tile_shifted(uint32_t stage, int chunk, const Tab &tab, int t,
                                         long long begin, int n, const Scalars &sc) {
-    constexpr int KS = P1<KT>::KS;
+    const Row<Tab> ptr{tab, t};
     const int lane = threadIdx.x & 31;
     const int K = KT > 0 ? KT : sc.K;
     const uint32_t part = (uint32_t)(4 * chunk + kShiftBytes);
-    auto at = [&](int stream, int role) {
-        return stage + (uint32_t)stream * part + ((uint32_t)reinterpret_cast<uintptr_t>(ptr[role]) & 12u);
+    auto at = [&](int role) {  // roles and streams are the same here
+        return stage + (uint32_t)role * part + ((uint32_t)reinterpret_cast<uintptr_t>(ptr[role]) & 12u);
     };
     uint32_t at_k[KT > 0 ? KT : 1];
 #pragma unroll
-    for (int k = 0; k < (KT > 0 ? KT : 1); ++k) at_k[k] = at(k, k);
-    const uint32_t at_w = RW ? at(K, KS) : 0u;
-    const uint32_t at_s = SS ? at(K + (RW ? 1 : 0), KS + 1) : 0u;
-    float *out = const_cast<float *>(ptr[0]) + begin;
+    for (int k = 0; k < (KT > 0 ? KT : 1); ++k) at_k[k] = at(k);
+    static_assert(!(RW && SS), "one of them is role K");
+    const uint32_t at_w = RW ? at(K) : 0u;
+    const uint32_t at_s = SS ? at(K) : 0u;
+    float *out = ptr[0] + begin;
     Dw4 ag, as, aw;
     dw_zero(ag);
     dw_zero(as);
@@ -1059,7 +1098,7 @@ __device__ __noinline__ D3 tile_shifted(uint32_t stage, int chunk, const float *
                 for (int u = 0; u < 4; ++u) s[u] = __fadd_rn(s[u], lds1(at_k[k] + o[u]));
         } else {
             for (int k = 1; k < K; ++k) {
-                const uint32_t a = at(k, k);
+                const uint32_t a = at(k);
 #pragma unroll
                 for (int u = 0; u < 4; ++u) s[u] = __fadd_rn(s[u], lds1(a + o[u]));
             }
@@ -1092,7 +1131,7 @@ __device__ __noinline__ D3 tile_shifted(uint32_t stage, int chunk, const float *
             const uint32_t o = 4u * (uint32_t)j;
             const float x0 = lds1(at_k[0] + o);
             float s = x0;
-            for (int k = 1; k < K; ++k) s = __fadd_rn(s, lds1(at(k, k) + o));
+            for (int k = 1; k < K; ++k) s = __fadd_rn(s, lds1(at(k) + o));
             if (K > 1) s = mean1<KT>(s, sc);
             r.g = __fma_rn((double)s, (double)s, r.g);
             if (K > 1) r.s = __fma_rn((double)x0, (double)x0, r.s);
@@ -1114,16 +1153,16 @@ __device__ __noinline__ D3 tile_shifted(uint32_t stage, int chunk, const float *
 // accd holds the lane's fp64 sums.  Default mode: accf holds the lane's fp32 sums over the
 // tile's float4 columns, scaled by 2^(2 acce) (acce is the same in every lane), and accd the
 // lane's fp64 sums over the elements taken one by one (tail, shifted tile).
-template <int KT, bool WM, bool RW, bool SS, bool PR, bool SH>
-__device__ __forceinline__ void reduce_tile(uint32_t stage, int chunk, const float *const *ptr,
-                                            const TilePos &q, int nv, bool aligned,
+template <int KT, bool WM, bool RW, bool SS, bool PR, bool SH, typename Tab>
+__device__ __forceinline__ void reduce_tile(uint32_t stage, int chunk, const Row<Tab> ptr,
+                                            float *out0, const TilePos &q, int nv, bool aligned,
                                             const Scalars &sc, double (&accd)[kAcc], float (&accf)[kAcc],
                                             int (&acce)[kAcc], unsigned &ecode, bool &tail) {
     const int lane = threadIdx.x & 31;
     const int K = KT > 0 ? KT : sc.K;
     const uint32_t sw_s = stage + (uint32_t)(K * chunk * 4);
     const uint32_t ss_s = stage + (uint32_t)((K + (RW ? 1 : 0)) * chunk * 4);
-    float *out = const_cast<float *>(ptr[0]) + q.begin;
+    float *out = out0 + q.begin;
     Dw4 ag, as, aw;                       // precise (PR) sums of the shared-memory columns
     dw_zero(ag);
     dw_zero(as);
@@ -1133,7 +1172,7 @@ __device__ __forceinline__ void reduce_tile(uint32_t stage, int chunk, const flo
     tail = false;                         // the tile has elements taken one by one
     ecode = 0u;                           // scale_code of acce[a] in bits 2a, 2a + 1
     if (SH && !aligned) {
-        const D3 d = tile_shifted<KT, WM, RW, SS>(stage, chunk, ptr, q.begin,
+        const D3 d = tile_shifted<KT, WM, RW, SS>(stage, chunk, ptr.tab, ptr.t, q.begin,
                                                          (int)(q.end - q.begin), sc);
         accd[0] = d.g;
         accd[1] = (K > 1 || SS) ? d.s : d.g;  // K = 1: replica 0 is the mean
@@ -1249,10 +1288,10 @@ __device__ __forceinline__ void reduce_tile(uint32_t stage, int chunk, const flo
                 s = __fadd_rn(s, SH ? lds1(stage + (uint32_t)(4 * k * chunk) + o) : __ldcg(ptr[k] + j));
             if (K > 1) {
                 s = mean1<KT>(s, sc);
-                if (WM) const_cast<float *>(ptr[0])[j] = s;
+                if (WM) out0[j] = s;
             }
-            const float y_s = !SS ? 0.f : SH ? lds1(ss_s + o) : __ldcg(ptr[P1<KT>::KS + 1] + j);
-            const float y_w = !RW ? 0.f : SH ? lds1(sw_s + o) : __ldcg(ptr[P1<KT>::KS] + j);
+            const float y_s = !SS ? 0.f : SH ? lds1(ss_s + o) : __ldcg(ptr[K] + j);
+            const float y_w = !RW ? 0.f : SH ? lds1(sw_s + o) : __ldcg(ptr[K] + j);
             if (K > 1) rs = __fma_rn((double)x0, (double)x0, rs);
             rg = __fma_rn((double)s, (double)s, rg);
             if (SS) rs = __fma_rn((double)y_s, (double)y_s, rs);
@@ -1348,8 +1387,7 @@ __device__ __noinline__ void add_shifted(const Scalars &sc, int tg, const double
 
 template <int KT, bool WM, bool RW, bool SS, bool PR, bool SH, bool Small>
 __global__ void __launch_bounds__(Ring1Of<KT, RW, SH>::kThreads, 1)
-    k_reduce(const __grid_constant__ TableOf<P1<KT>::NP, Small> tab, const __grid_constant__ Scalars sc) {
-    constexpr int KS = P1<KT>::KS;
+    k_reduce(const __grid_constant__ TableOf<Small> tab, const __grid_constant__ Scalars sc) {
     extern __shared__ __align__(128) unsigned char smem[];
     // The first launch of a step's pass that does not read w issues its first tiles at once: the
     // only kernel that lets it start early is the previous call's k_finish, once all before that
@@ -1370,7 +1408,7 @@ __global__ void __launch_bounds__(Ring1Of<KT, RW, SH>::kThreads, 1)
     const int chunk = tab.chunk;
     // Stage streams: replicas 0 .. K - 1, then w (RW), then g_small (SS).
     const int ns = K + (RW ? 1 : 0) + (SS ? 1 : 0);
-    const int role = lane < K ? lane : (RW && lane == K ? KS : KS + 1);
+    const int role = lane < ns ? lane : 0;
     Stream<Ring1Of<KT, RW, SH>, SH> st;
     int c = st.start(smem, tab.nc, sc.tiles + 4 * (tab.seq & 1), sc.evict_first != 0);
     TilePos q = {};
@@ -1410,13 +1448,13 @@ __global__ void __launch_bounds__(Ring1Of<KT, RW, SH>::kThreads, 1)
                 c = -1;
                 break;
             }
-            const float *const *ptr = tab.ptr[q.t];
+            const Row<TableOf<Small>> ptr{tab, q.t};
             double accd[kAcc];
             float accf[kAcc];
             int acce[kAcc];
             unsigned tcode;
             bool tile_tail;
-            reduce_tile<KT, WM, RW, SS, PR, SH>(st.stage, chunk, ptr, q, st.tc.nv, st.tc.aligned, sc,
+            reduce_tile<KT, WM, RW, SS, PR, SH>(st.stage, chunk, ptr, st.tc.stream(0), q, st.tc.nv, st.tc.aligned, sc,
                                             accd, accf, acce, tcode, tile_tail);
             __syncwarp();
             const int tg = q.tg;
@@ -1705,10 +1743,8 @@ __global__ void __launch_bounds__(32 * kFinWarps) k_finish(const __grid_constant
 // ----------------------------------------------------------------------------
 // Pass 2: scaled momentum-SGD + weight-decay update (Eq. 7b, Algorithm 1)
 // ----------------------------------------------------------------------------
-// Pointer roles: 0 = gbar, 1 = w, 2 = m, 3 = per-element gradscale.
+// Pointer roles: 0 = gbar, 1 = w, then m (HM), then the per-element gradscale (PE).
 // Stage streams: gbar, w, then m (HM), then the per-element scale (PE, scaled).
-
-constexpr int kNP2 = 4;
 
 __device__ __forceinline__ void sgd1(float g, float c, float &w, float &m, const Scalars &sc,
                                      bool has_m) {
@@ -1747,20 +1783,20 @@ __device__ __noinline__ float w_cols_scaled(uint32_t w_stage, int nv, float f) {
 
 // A tile of a tensor off a 16-byte boundary, as tile_shifted() of pass 1: four elements per lane
 // and step.  Returns the lane's |w|^2 (float-float pairs, to fp64 once) when the statistics want it.
-template <bool HM, bool PE, bool SW>
-__device__ __noinline__ double update_shifted(uint32_t stage, const float *const *ptr,
-                                              long long begin, int n, float ct, bool use_se,
+template <bool HM, bool PE, bool SW, typename Tab>
+__device__ __noinline__ double update_shifted(uint32_t stage, const Tab &tab, int t, long long begin, int n, float ct, bool use_se,
                                               const Scalars &sc) {
     constexpr uint32_t part = (uint32_t)(4 * Ring2<false>::tile_elems(2 + (HM ? 1 : 0) + (PE ? 1 : 0)) +
                                          kShiftBytes);
     const int lane = threadIdx.x & 31;
-    auto at = [&](int stream, int role) {
-        return stage + (uint32_t)stream * part + ((uint32_t)reinterpret_cast<uintptr_t>(ptr[role]) & 12u);
+    const Row<Tab> ptr{tab, t};
+    auto at = [&](int role) {
+        return stage + (uint32_t)role * part + ((uint32_t)reinterpret_cast<uintptr_t>(ptr[role]) & 12u);
     };
-    const uint32_t at_g = at(0, 0), at_w = at(1, 1), at_m = HM ? at(2, 2) : 0u;
-    const uint32_t at_c = use_se ? at(HM ? 3 : 2, 3) : 0u;
-    float *wp = const_cast<float *>(ptr[1]) + begin;
-    float *mp = HM ? const_cast<float *>(ptr[2]) + begin : nullptr;
+    const uint32_t at_g = at(0), at_w = at(1), at_m = HM ? at(2) : 0u;
+    const uint32_t at_c = use_se ? at(HM ? 3 : 2) : 0u;
+    float *wp = ptr[1] + begin;
+    float *mp = HM ? ptr[2] + begin : nullptr;
     Dw4 aw;
     dw_zero(aw);
     for (int j0 = lane; j0 < n; j0 += 128) {
@@ -1802,7 +1838,7 @@ __device__ __noinline__ double update_shifted(uint32_t stage, const float *const
 
 template <bool HM, bool PE, bool SW, bool SH, bool Small>
 __global__ void __launch_bounds__(Ring2<SH>::kThreads, 1)
-    k_update(const __grid_constant__ TableOf<kNP2, Small> tab, const __grid_constant__ Scalars sc) {
+    k_update(const __grid_constant__ TableOf<Small> tab, const __grid_constant__ Scalars sc) {
     extern __shared__ __align__(128) unsigned char smem[];
     // The first launch of the pass issues w and m of its first tiles at once: it starts only when
     // this step's reduction (and k_lars) have started, which let it once every kernel before them
@@ -1836,7 +1872,7 @@ __global__ void __launch_bounds__(Ring2<SH>::kThreads, 1)
     const int chunk = tab.chunk;
     const bool use_se = PE && scaled;
     const int ns = 2 + (HM ? 1 : 0) + (use_se ? 1 : 0);
-    const int role = !HM && lane == 2 ? 3 : (lane < 4 ? lane : 0);
+    const int role = lane < ns ? lane : 0;
     constexpr int CH = Ring2<false>::tile_elems(2 + (HM ? 1 : 0) + (PE ? 1 : 0));
     constexpr int COLS = CH / 128;
     const uint32_t w_off = (uint32_t)(CH * 4);
@@ -1884,13 +1920,13 @@ __global__ void __launch_bounds__(Ring2<SH>::kThreads, 1)
                 c = -1;
                 break;
             }
-            const float *const *ptr = tab.ptr[q.t];
+            const Row<TableOf<Small>> ptr{tab, q.t};
             const int nv = st.tc.nv;
             if (sc.stats && q.c_in_t == 0 && lane == 0)
                 sc.stats[(size_t)q.tg * TULA_STATS_LEN + TULA_STAT_COEF] =
                     PE ? (scaled ? (double)NAN : 1.0) : (double)ct;
-            float *wp = const_cast<float *>(ptr[1]) + q.begin;
-            float *mp = HM ? const_cast<float *>(ptr[2]) + q.begin : nullptr;
+            float *wp = st.tc.stream(1) + q.begin;
+            float *mp = HM ? st.tc.stream(2) + q.begin : nullptr;
             const float4 cdef = PE ? make_float4(1.f, 1.f, 1.f, 1.f) : make_float4(ct, ct, ct, ct);
             float aw = 0.f;    // fp32 |w|^2 of the tile's columns (statistics only)
             double awt = 0.0;  // exact fp64 |w|^2 of its tail
@@ -1938,7 +1974,7 @@ __global__ void __launch_bounds__(Ring2<SH>::kThreads, 1)
             }
             if constexpr (SH) {
                 if (!st.tc.aligned)
-                    awt = update_shifted<HM, PE, SW>(stage, ptr, q.begin, (int)(q.end - q.begin), ct,
+                    awt = update_shifted<HM, PE, SW>(stage, tab, q.t, q.begin, (int)(q.end - q.begin), ct,
                                                      use_se, sc);
             }
             const long long n = q.end - q.begin;
@@ -1951,7 +1987,7 @@ __global__ void __launch_bounds__(Ring2<SH>::kThreads, 1)
                     float w = SH ? lds1(o + w_off) : __ldcg(wp + jj);
                     float m = !HM ? 0.f : SH ? lds1(o + m_off) : __ldcg(mp + jj);
                     const float cj = !use_se ? (PE ? 1.f : ct)
-                                     : SH    ? lds1(o + se_off) : __ldcg(ptr[3] + q.begin + jj);
+                                     : SH    ? lds1(o + se_off) : __ldcg(ptr[HM ? 3 : 2] + q.begin + jj);
                     if (SW) awt = __fma_rn((double)w, (double)w, awt);
                     sgd1(g, cj, w, m, sc, HM);
                     wp[jj] = w;
@@ -2008,8 +2044,6 @@ __global__ void __launch_bounds__(Ring2<SH>::kThreads, 1)
 // A once-per-epoch call: plain 128-bit loads, one warp per tile.
 // Pointer roles: 0 = g_small, 1 = g_large, 2 = s_out.
 
-constexpr int kNP3 = 3;
-
 __device__ __forceinline__ float scale1(float gs, float gl, const Scalars &sc) {
     return fminf(fabsf(__fdiv_rn(gs, __fadd_rn(gl, sc.eps))), sc.s_max);
 }
@@ -2032,7 +2066,7 @@ constexpr int kScaleThreads = 128;
 
 template <bool Small>
 __global__ void __launch_bounds__(kScaleThreads)
-    k_scale_elem(const __grid_constant__ TableOf<kNP3, Small> tab, const __grid_constant__ Scalars sc) {
+    k_scale_elem(const __grid_constant__ TableOf<Small> tab, const __grid_constant__ Scalars sc) {
     grid_wait();  // no early start for the successor: it may overwrite what this kernel reads
     const int lane = threadIdx.x & 31;
     const int warp = (int)((blockIdx.x * (unsigned)kScaleThreads + threadIdx.x) >> 5);
@@ -2040,11 +2074,11 @@ __global__ void __launch_bounds__(kScaleThreads)
     Walker walk;
     for (int c = warp; c < tab.nc; c += nwarps) {
         const TilePos q = locate(tab, c, walk.to(tab, c), tab.chunk);
-        const float *const *ptr = tab.ptr[q.t];
+        const Row<TableOf<Small>> ptr{tab, q.t};
         const int nv = tile_vecs(lane < 3 ? ptr[lane] : nullptr, 3, q);
         const float *a = ptr[0] + q.begin;
         const float *b = ptr[1] + q.begin;
-        float *o = const_cast<float *>(ptr[2]) + q.begin;
+        float *o = ptr[2] + q.begin;
         // Four float4 columns of each input per lane per step: eight 16-byte loads in flight
         // per lane, which a plain-load streaming kernel needs to cover HBM latency.
         for (int v0 = lane; v0 < nv; v0 += 4 * 32) {
@@ -2096,10 +2130,6 @@ std::atomic<uint64_t> g_launches{0};
 thread_local int g_last_cuda = 0;
 
 inline long long tiles_of(int64_t n, int chunk) { return n <= 0 ? 1 : (n + chunk - 1) / chunk; }
-
-inline int replica_slot(int K) {
-    return (K == 1 || K == 2 || K == 4 || K == 8 || K == 16) ? K : TULA_MAX_K;
-}
 
 // Tile sizes: the smallest a pass can use for K replicas sizes the workspace.
 inline int chunk1(int K, bool rw, bool ss) {
@@ -2160,13 +2190,6 @@ bool valid_numels(const int64_t *numels, int n, int K, Plan *pl) {
     return true;
 }
 
-// Whether some pointer of a tensor's table row lies off a 16-byte boundary.
-template <int NP>
-inline bool off_16(const float *const (&ptr)[NP]) {
-    for (const float *q : ptr)
-        if (reinterpret_cast<uintptr_t>(q) & 15u) return true;
-    return false;
-}
 inline bool aligned4(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 3u) == 0; }
 
 // One wave of resident CTAs of `kernel` on the current device (cached); sets
@@ -2238,7 +2261,7 @@ int launch_pdl(void (*kernel)(KArgs...), int grid, int threads, int smem, cudaSt
 // size, its parameter blocks, built by the first call that launches them and reused by every
 // later one (they hold only sizes and pointers, which a plan fixes).
 struct Blocks {
-    bool small = false;  // TableOf<NP, true>: one launch of few, aligned tensors
+    bool small = false;  // TableOf<true>: one launch of few, aligned tensors
     std::vector<std::shared_ptr<const void>> tabs;
 };
 struct TableCache {
@@ -2255,49 +2278,96 @@ struct TableCache {
     }
 };
 
+// The pointers of a pass's launches: fill(p, ptrs) writes tensor p's np pointers.
+// What the tables of tensors [0, n) need: whether every role's pointers lie within 16 GB of its
+// lowest, and whether some non-empty tensor has a pointer off a 16-byte boundary.
+struct Pointers {
+    unsigned long long base[kMaxRoles] = {};
+    bool wide = false, shifted = false;
+};
+template <typename Fill>
+Pointers scan_pointers(int n, const int64_t *numels, int np, Fill fill) {
+    Pointers r;
+    unsigned long long low[kMaxRoles], high[kMaxRoles];
+    for (int i = 0; i < np; ++i) {
+        low[i] = ~0ull;
+        high[i] = 0ull;
+    }
+    const float *ptr[kMaxRoles];
+    for (int p = 0; p < n; ++p) {
+        if (numels[p] <= 0) continue;
+        fill(p, ptr);
+        for (int i = 0; i < np; ++i) {
+            const unsigned long long a = reinterpret_cast<uintptr_t>(ptr[i]);
+            low[i] = std::min(low[i], a);
+            high[i] = std::max(high[i], a);
+            if (a & 15u) r.shifted = true;
+        }
+    }
+    for (int i = 0; i < np; ++i) {
+        if (low[i] > high[i]) continue;  // no non-empty tensor
+        r.base[i] = low[i];
+        if ((high[i] - low[i]) / 4 > 0xffffffffull) r.wide = true;
+    }
+    return r;
+}
+
 // Splits tensors [0, n) into parameter blocks of type Tab of tiles of `chunk` elements.
-// fill(p, ptrs) writes tensor p's pointers.
 template <typename Tab, typename Fill>
-void build_blocks(int n, const int64_t *numels, int chunk, Fill fill,
+void build_blocks(int n, const int64_t *numels, int chunk, int np, const Pointers &pts, Fill fill,
                   std::vector<std::shared_ptr<const void>> &tabs) {
-    long long c_global = 0;
-    int p = 0;
-    while (p < n) {
+    const float *ptr[kMaxRoles];
+    for (int p = 0; p < n;) {
+        int cnt = 1;
+        while (p + cnt < n && Tab::bytes_for(cnt + 1, np, pts.wide) <= Tab::kRaw) ++cnt;
         std::shared_ptr<Tab> tab = std::make_shared<Tab>();
         std::memset(tab.get(), 0, sizeof(Tab));
         tab->t0 = p;
-        tab->c0 = (int)c_global;
+        tab->n = cnt;
         tab->chunk = chunk;
         tab->seq = (int)tabs.size();
-        int cnt = 0, nc = 0;
-        while (p < n && cnt < Tab::kMaxT) {
-            tab->numel[cnt] = numels[p];
-            tab->cstart[cnt] = nc;
-            fill(p, tab->ptr[cnt]);
-            if (numels[p] > 0 && off_16(tab->ptr[cnt])) tab->shifted = 1;
-            nc += (int)tiles_of(numels[p], chunk);
-            ++cnt;
-            ++p;
+        tab->np = np;
+        tab->wide = pts.wide ? 1 : 0;
+        tab->o_last = 4 * (cnt + 1);
+        tab->o_lo = tab->o_last + (2 * cnt + 3) / 4 * 4;
+        tab->o_hi = tab->o_lo + 4 * cnt * np;
+        std::memcpy(tab->base, pts.base, sizeof(tab->base));
+        int *cstart = reinterpret_cast<int *>(tab->raw);
+        unsigned short *last = reinterpret_cast<unsigned short *>(tab->raw + tab->o_last);
+        unsigned *lo = reinterpret_cast<unsigned *>(tab->raw + tab->o_lo);
+        unsigned short *hi = reinterpret_cast<unsigned short *>(tab->raw + tab->o_hi);
+        int nc = 0;
+        for (int t = 0; t < cnt; ++t, ++p) {
+            const long long tiles = tiles_of(numels[p], chunk);
+            cstart[t] = nc;
+            last[t] = (unsigned short)(numels[p] - (tiles - 1) * chunk);
+            nc += (int)tiles;
+            if (numels[p] <= 0) continue;  // its pointers may be NULL; nothing reads them
+            fill(p, ptr);
+            for (int i = 0; i < np; ++i) {
+                const unsigned long long a = reinterpret_cast<uintptr_t>(ptr[i]);
+                if (a & 15u) tab->shifted = 1;
+                const unsigned long long e = (a - pts.base[i]) / 4;
+                lo[t * np + i] = (unsigned)e;
+                if (pts.wide) hi[t * np + i] = (unsigned short)(e >> 32);
+            }
         }
-        tab->n = cnt;
+        cstart[cnt] = nc;
         tab->nc = nc;
-        tab->cstart[cnt] = nc;
         for (int i = 0, t = 0; i < kHints; ++i) {
-            while (t + 1 < cnt && i * kHintTiles >= tab->cstart[t + 1]) ++t;
+            while (t + 1 < cnt && i * kHintTiles >= cstart[t + 1]) ++t;
             tab->hint[i] = (unsigned short)t;
         }
-        c_global += nc;
         tabs.push_back(std::move(tab));
     }
 }
 
 // The instantiations of a streaming kernel: for launches whose tensors are all 16-byte aligned,
 // with a small parameter block and with a full one, and for the others.
-template <int NP>
 struct StreamKernels {
-    void (*small)(TableOf<NP, true>, Scalars);
-    void (*full)(TableOf<NP, false>, Scalars);
-    void (*shifted)(TableOf<NP, false>, Scalars);
+    void (*small)(TableOf<true>, Scalars);
+    void (*full)(TableOf<false>, Scalars);
+    void (*shifted)(TableOf<false>, Scalars);
     int smem, smem_shifted;
 };
 template <typename Tab>
@@ -2315,24 +2385,20 @@ int launch_block(void (*fn)(Tab, Scalars), const void *block, int threads, int s
 }
 // Launches a streaming kernel once per parameter block.  With a cache, the blocks are taken from
 // it, or built once and kept there.
-template <int NP, typename Fill>
-int launch_streaming(const StreamKernels<NP> &k, int n, const int64_t *numels, int chunk,
+template <typename Fill>
+int launch_streaming(const StreamKernels &k, int n, const int64_t *numels, int chunk, int np,
                      int threads, const Scalars &sc, int grid_override, cudaStream_t stream,
                      Fill fill, TableCache *cache = nullptr) {
-    using SmallTab = TableOf<NP, true>;
-    using FullTab = TableOf<NP, false>;
+    using SmallTab = TableOf<true>;
+    using FullTab = TableOf<false>;
     const Blocks *blocks = cache ? cache->find((const void *)k.full, chunk) : nullptr;
     Blocks built;
     if (!blocks) {
-        built.small = n <= SmallTab::kMaxT && SmallTab::kMaxT < FullTab::kMaxT;
-        for (int p = 0; p < n && built.small; ++p) {
-            const float *ptr[NP] = {};
-            if (numels[p] > 0) fill(p, ptr);
-            if (off_16(ptr)) built.small = false;
-        }
+        const Pointers pts = scan_pointers(n, numels, np, fill);
+        built.small = !pts.shifted && SmallTab::bytes_for(n, np, pts.wide) <= SmallTab::kRaw;
         try {
-            if (built.small) build_blocks<SmallTab>(n, numels, chunk, fill, built.tabs);
-            else build_blocks<FullTab>(n, numels, chunk, fill, built.tabs);
+            if (built.small) build_blocks<SmallTab>(n, numels, chunk, np, pts, fill, built.tabs);
+            else build_blocks<FullTab>(n, numels, chunk, np, pts, fill, built.tabs);
             if (cache) {
                 cache->entries.push_back({(const void *)k.full, chunk, std::move(built)});
                 blocks = &cache->entries.back().blocks;
@@ -2406,14 +2472,13 @@ template <int KT, bool WM, bool RW, bool SS, bool PR, typename Fill>
 int run_reduce_k(int K, int n, const int64_t *numels, const Scalars &sc, int grid, cudaStream_t s,
                  Fill fill, TableCache *cache) {
     const int chunk = chunk1(K, RW, SS);
-    constexpr int NP = P1<KT>::NP;
     using R = Ring1Of<KT, RW, false>;
-    constexpr bool kSmall = kSmallT<NP> < kFullT<NP>;  // else both blocks are the same type
-    const StreamKernels<NP> k{k_reduce<KT, WM, RW, SS, PR, false, kSmall>,
-                              k_reduce<KT, WM, RW, SS, PR, false, false>,
-                              k_reduce<KT, WM, RW, SS, PR, true, false>, R::kSmemBytes,
-                              Ring1Of<KT, RW, true>::kSmemBytes};
-    return launch_streaming<NP>(k, n, numels, chunk, R::kThreads, sc, grid, s, fill, cache);
+    const StreamKernels k{k_reduce<KT, WM, RW, SS, PR, false, true>,
+                          k_reduce<KT, WM, RW, SS, PR, false, false>,
+                          k_reduce<KT, WM, RW, SS, PR, true, false>, R::kSmemBytes,
+                          Ring1Of<KT, RW, true>::kSmemBytes};
+    return launch_streaming(k, n, numels, chunk, K + (RW || SS ? 1 : 0), R::kThreads, sc, grid, s,
+                            fill, cache);
 }
 
 template <bool WM, bool RW, bool SS, bool PR, typename Fill>
@@ -2609,11 +2674,9 @@ int run_step(float *const *param_ptrs, float *const *grad_ptrs, float *const *mo
     sc.wd = weight_decay;
     sc.early_w = part == kPartWhole ? 1 : 0;
 
-    const int KS = replica_slot(K);
     auto fill1 = [&](int p, const float **dst) {
         for (int k = 0; k < K; ++k) dst[k] = grad_ptrs[(size_t)k * n + p];
-        dst[KS] = param_ptrs[p];
-        dst[KS + 1] = nullptr;
+        dst[K] = param_ptrs[p];  // used by a pass that reads w
     };
     record(hp->trace_events[0], s);
     if (part == kPartUpdate) {
@@ -2639,17 +2702,18 @@ int run_step(float *const *param_ptrs, float *const *grad_ptrs, float *const *mo
     auto fill2 = [&](int p, const float **dst) {
         dst[0] = grad_ptrs[p];
         dst[1] = param_ptrs[p];
-        dst[2] = mom_ptrs ? mom_ptrs[p] : nullptr;
-        dst[3] = per_elem ? hp->scale_elem[p] : nullptr;
+        if (mom_ptrs) dst[2] = mom_ptrs[p];
+        if (per_elem) dst[mom_ptrs ? 3 : 2] = hp->scale_elem[p];
     };
     const bool hm = mom_ptrs != nullptr;
     const bool sw = hp->layer_stats != nullptr && !lars;  // the update takes |w|^2
     const int c2 = chunk2(hm, per_elem);
 #define TULA_UPD(HM, PE, SW)                                                                       \
-    launch_streaming<kNP2>({k_update<HM, PE, SW, false, true>, k_update<HM, PE, SW, false, false>,  \
+    launch_streaming({k_update<HM, PE, SW, false, true>, k_update<HM, PE, SW, false, false>,  \
                             k_update<HM, PE, SW, true, false>, Ring2<false>::kSmemBytes,             \
                             Ring2<true>::kSmemBytes},                                                \
-                           n, numels, c2, Ring2<false>::kThreads, sc, hp->grid_ctas, s, fill2, cache)
+                     n, numels, c2, 2 + (HM) + (PE), Ring2<false>::kThreads, sc, hp->grid_ctas, s,  \
+                     fill2, cache)
     if (hm) {
         if (per_elem) rc = sw ? TULA_UPD(true, true, true) : TULA_UPD(true, true, false);
         else rc = sw ? TULA_UPD(true, false, true) : TULA_UPD(true, false, false);
@@ -2805,11 +2869,9 @@ int tula_layer_stats(const float *const *param_ptrs, const float *const *grad_pt
     Scalars sc = make_scalars(nullptr, K, n, workspace, L, kModeStats);
     sc.stats = stats_out;
     sc.read_w = 1;
-    const int KS = replica_slot(K);
     auto fill = [&](int p, const float **dst) {
         for (int k = 0; k < K; ++k) dst[k] = grad_ptrs[(size_t)k * n + p];
-        dst[KS] = param_ptrs[p];
-        dst[KS + 1] = nullptr;
+        dst[K] = param_ptrs[p];
     };
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     rc = run_reduce<false, true, false, false>(K, n, numels, sc, 0, s, fill);
@@ -2843,8 +2905,8 @@ int tula_ags_update_scale(const float *const *g_small, const float *const *g_lar
             dst[1] = g_large[p];
             dst[2] = hp->scale_elem[p];
         };
-        return launch_streaming<kNP3>({k_scale_elem<true>, k_scale_elem<false>, k_scale_elem<false>, 0, 0},
-                                      n, numels, 4096, kScaleThreads, sc, hp->grid_ctas, s, fill);
+        return launch_streaming({k_scale_elem<true>, k_scale_elem<false>, k_scale_elem<false>, 0, 0}, n,
+                                numels, 4096, 3, kScaleThreads, sc, hp->grid_ctas, s, fill);
     }
     int rc = check_ws(hp->workspace, hp->workspace_bytes, n, pl);
     if (rc) return rc;
@@ -2852,8 +2914,7 @@ int tula_ags_update_scale(const float *const *g_small, const float *const *g_lar
     Scalars sc = make_scalars(hp, 1, n, hp->workspace, L, kModeScale);
     auto fill = [&](int p, const float **dst) {
         dst[0] = g_large[p];
-        dst[1] = nullptr;
-        dst[2] = g_small[p];
+        dst[1] = g_small[p];
     };
     rc = run_reduce_k<1, false, false, true, true>(1, n, numels, sc, hp->grid_ctas, s, fill, nullptr);
     return rc ? rc : launch_finish(n, sc, s);

@@ -882,3 +882,41 @@ def test_the_mean_of_every_significand(K):
             # -0.0 + 0.0 (the other replicas) is +0.0
             q = np.where(q == 0, np.float32(0), q)
             assert np.array_equal(got[~nan].view(np.int32), q[~nan].view(np.int32))
+
+
+@pytest.mark.parametrize("K", [1, 6])
+def test_tensors_farther_apart_than_a_32_bit_offset(K, monkeypatch):
+    """The weights at both ends of an 18 GB buffer (a launch's table holds 32-bit offsets, in fp32
+    elements, within 16 GB, and 48 bits beyond): as the oracle, for pass 1 with and without w."""
+    ps = W.ParamSet("far")
+    for n in (1000, 4097, 3, 20000):
+        ps.add((n,), W.KIND_NORMAL)
+    plain = W.allocate
+    far = torch.empty((18 << 30) // 4, dtype=torch.float32, device="cuda")
+
+    def spread(*args, **kw):
+        buf = plain(*args, **kw)
+        near = buf.w_flat
+        buf.w = []
+        for p, n in enumerate(ps.numels):
+            o = buf.offsets[p] + (far.numel() - 65536 if p % 2 else 0)
+            buf.w.append(far[o:o + n])
+        assert abs(buf.w[1].data_ptr() - buf.w[0].data_ptr()) > 17 << 30
+        fill = W.fill_state
+
+        def fill_far(b, wl):
+            fill(b, wl)
+            for p, n in enumerate(ps.numels):
+                b.w[p].copy_(near[b.offsets[p]:b.offsets[p] + n])
+        monkeypatch.setattr(W, "fill_state", fill_far)
+        return buf
+
+    monkeypatch.setattr(W, "allocate", spread)
+    wl = W.workload("stress_k4", seed=231 + K, factor_range=(1e-3, 1e1), zero_patterns=False)
+    for rule in (T.TULA_RULE_AGS, T.TULA_RULE_LARS):
+        monkeypatch.undo()
+        monkeypatch.setattr(W, "allocate", spread)
+        pair = Pair(wl, K=K, pset=ps, rule=rule, lars_trust=0.01)
+        pair.step(1, 1.0)
+        pair.step(1, 1.0)
+        assert pair.flags == [0, 1]
