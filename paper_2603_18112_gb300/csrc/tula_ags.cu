@@ -130,7 +130,7 @@ enum Mode { kModeStep = 0, kModeStats = 1, kModeScale = 2 };
 // tensors lie farther apart (`wide`).  8 to 12 bytes per tensor and 8 per pointer, as the table was
 // before, took 4096 tensors with K = 16 through 21 launches of pass 1 instead of 10, and left more
 // of the block to miss the constant cache on.
-constexpr int kHints = 160, kHintTiles = 8;  // covers the first tiles of 152 SMs' 8 warps
+constexpr int kHints = 160;
 constexpr int kMaxRoles = TULA_MAX_K + 1;
 struct TableHead {
     int n;        // tensors in this launch
@@ -141,9 +141,9 @@ struct TableHead {
     int shifted;  // 1: some tensor has a stream off a 16-byte boundary
     int np, wide;
     int o_last, o_lo, o_hi;  // byte offsets in raw
-    int pad;
+    int hint_shift;
     unsigned long long base[kMaxRoles];
-    unsigned short hint[kHints];  // tensor of tile min(i * kHintTiles, nc - 1)
+    unsigned short hint[kHints + 2];  // tensor of tile min(i << hint_shift, nc - 1)
 };
 template <int Bytes>
 struct Table : TableHead {
@@ -665,24 +665,16 @@ __device__ __forceinline__ int find_tensor(const Tab &tab, int lo, int hi, int c
     return lo;
 }
 
-// Follows the tensor index along one warp's tiles, which ascend: the next two tensors are tried
-// first, then a search over the rest.
+// Follows the tensor index along one warp's tiles, which ascend.  A kernel finds the table outside
+// the constant cache, and each step of a search through it is a miss (a search from scratch took
+// 2 us before a warp's first copy), so the hints narrow it to the tensors of a few tiles.
 struct Walker {
     int t = -1;
     template <typename Tab>
     __device__ __forceinline__ int to(const Tab &tab, int c) {
-        if (t < 0) {
-            // The warp's first tile: the table is not in the constant cache yet, and the eight
-            // or so steps of a search, each a miss, took 2 us.  Two with the hint.
-            if (c >= kHints * kHintTiles) return t = find_tensor(tab, 0, tab.n, c);
-            t = tab.hint[c / kHintTiles];
-            while (c >= tab.cstart(t + 1)) ++t;  // at most kHintTiles - 1 steps
-            return t;
-        }
-        if (c < tab.cstart(t + 1)) return t;
-        ++t;
-        if (c < tab.cstart(t + 1)) return t;
-        return t = find_tensor(tab, t + 1, tab.n, c);
+        if (t >= 0 && c < tab.cstart(t + 1)) return t;
+        const int h = c >> tab.hint_shift;
+        return t = find_tensor(tab, tab.hint[h], tab.hint[h + 1] + 1, c);
     }
 };
 
@@ -1227,6 +1219,15 @@ __device__ __forceinline__ void reduce_tile(uint32_t stage, int chunk, const Row
         // replica, so that U loads are always in flight: one column at a time, every load waited
         // for the one before, and K = 6 took 234 us a ResNet-50 step, 213 with this.
         constexpr int U = PR ? 2 : 4;
+        // The tail's loads go first (not SH, K known: one lane per element), to land meanwhile.
+        constexpr bool kTailFirst = !SH && KT > 0;
+        constexpr int kTailRoles = kTailFirst ? KT + (RW || SS ? 1 : 0) : 1;
+        const long long tail_at = q.begin + 4 * (long long)nv;
+        float xt[kTailRoles] = {};
+        if (kTailFirst && tail_at + lane < q.end) {
+#pragma unroll
+            for (int k = 0; k < kTailRoles; ++k) xt[k] = __ldcg(ptr[k] + tail_at + lane);
+        }
         for (int v0 = lane; v0 < nv; v0 += 32 * 4) {
             float pg = 0.f, ps = 0.f, pw = 0.f;
             if constexpr (KT > 0) {
@@ -1279,23 +1280,32 @@ __device__ __forceinline__ void reduce_tile(uint32_t stage, int chunk, const Row
             }
         }
         // The last n % 4 elements, exact squares in fp64: from the stage (SH) or by plain loads.
-        tail = q.begin + 4 * (long long)nv < q.end;  // the same in every lane
-        for (long long j = q.begin + 4 * (long long)nv + lane; j < q.end; j += 32) {
+        tail = tail_at < q.end;  // the same in every lane
+        if (tail_at + lane < q.end) {
+            const long long j = tail_at + lane;
             const uint32_t o = 4u * (uint32_t)(j - q.begin);
-            const float x0 = SH ? lds1(stage + o) : __ldcg(ptr[0] + j);
+            const float x0 = SH ? lds1(stage + o) : kTailFirst ? xt[0] : __ldcg(ptr[0] + j);
             float s = x0;
-            for (int k = 1; k < K; ++k)
-                s = __fadd_rn(s, SH ? lds1(stage + (uint32_t)(4 * k * chunk) + o) : __ldcg(ptr[k] + j));
+            if constexpr (kTailFirst) {
+#pragma unroll
+                for (int k = 1; k < KT; ++k) s = __fadd_rn(s, xt[k]);
+            } else {
+                for (int k = 1; k < K; ++k)
+                    s = __fadd_rn(s, SH ? lds1(stage + (uint32_t)(4 * k * chunk) + o)
+                                        : __ldcg(ptr[k] + j));
+            }
             if (K > 1) {
                 s = mean1<KT>(s, sc);
                 if (WM) out0[j] = s;
             }
-            const float y_s = !SS ? 0.f : SH ? lds1(ss_s + o) : __ldcg(ptr[K] + j);
-            const float y_w = !RW ? 0.f : SH ? lds1(sw_s + o) : __ldcg(ptr[K] + j);
             if (K > 1) rs = __fma_rn((double)x0, (double)x0, rs);
             rg = __fma_rn((double)s, (double)s, rg);
-            if (SS) rs = __fma_rn((double)y_s, (double)y_s, rs);
-            if (RW) rw = __fma_rn((double)y_w, (double)y_w, rw);
+            if (RW || SS) {  // role K
+                const float y = SH ? lds1((RW ? sw_s : ss_s) + o)
+                                   : kTailFirst ? xt[kTailRoles - 1] : __ldcg(ptr[K] + j);
+                double &r = RW ? rw : rs;
+                r = __fma_rn((double)y, (double)y, r);
+            }
         }
     }
     if (PR) {
@@ -1840,9 +1850,11 @@ template <bool HM, bool PE, bool SW, bool SH, bool Small>
 __global__ void __launch_bounds__(Ring2<SH>::kThreads, 1)
     k_update(const __grid_constant__ TableOf<Small> tab, const __grid_constant__ Scalars sc) {
     extern __shared__ __align__(128) unsigned char smem[];
-    // The first launch of the pass issues w and m of its first tiles at once: it starts only when
-    // this step's reduction (and k_lars) have started, which let it once every kernel before them
-    // had completed, so both are final.  The mean follows when the kernel before has completed.
+    // The first launch of the pass issues m (w when there is no m, w and m of shifted tiles) of its
+    // first tiles at once: it starts only when this step's reduction (and k_lars) have started,
+    // which let it once every kernel before them had completed, so both are final.  The rest
+    // follows when the kernel before has completed.  (w and m together: ResNet-18 73.9 us instead
+    // of 73.3, as the branch's reads queue behind them; neither: 74.5.)
     // The whole CTA waits per element (the stream count depends on the branch) and in a sharded
     // step (whatever ran between its two calls).  The next kernel may start when that wait has
     // passed: the next step's reduction reads the mean this step's has written.  A later launch of
@@ -1878,15 +1890,16 @@ __global__ void __launch_bounds__(Ring2<SH>::kThreads, 1)
     const uint32_t w_off = (uint32_t)(CH * 4);
     const uint32_t m_off = (uint32_t)(2 * CH * 4);
     const uint32_t se_off = (uint32_t)((HM ? 3 : 2) * CH * 4);
+    constexpr int kEarlyFrom = HM && !SH ? 2 : 1;  // streams from here on are issued early
     Stream<Ring2<SH>, SH> st;
     int c = st.start(smem, tab.nc, sc.tiles + 4 * (tab.seq & 1) + 2, sc.evict_first != 0);
     TilePos q = {};
-    if (c >= 0) q = st.issue(tab, c, chunk, role, ns, early ? 1 : 0);
+    if (c >= 0) q = st.issue(tab, c, chunk, role, ns, early ? kEarlyFrom : 0);
     st.claim_first();
     if (early) {
         grid_wait();
         grid_launch_dependents();
-        if (c >= 0) st.issue_below(q, 1, ns, chunk);
+        if (c >= 0) st.issue_below(q, kEarlyFrom, ns, chunk);
         scaled = take_branch();
     }
     bool to_wait = !first;
@@ -1930,6 +1943,18 @@ __global__ void __launch_bounds__(Ring2<SH>::kThreads, 1)
             const float4 cdef = PE ? make_float4(1.f, 1.f, 1.f, 1.f) : make_float4(ct, ct, ct, ct);
             float aw = 0.f;    // fp32 |w|^2 of the tile's columns (statistics only)
             double awt = 0.0;  // exact fp64 |w|^2 of its tail
+            // The last n % 4 elements, one per lane: their loads go first, to land meanwhile (SH:
+            // they are in the stage).
+            const long long n = q.end - q.begin;
+            const long long jj = 4 * (long long)nv + lane;
+            const bool in_tail = jj < n && (!SH || st.tc.aligned);
+            float g_t = 0.f, w_t = 0.f, m_t = 0.f, c_t = PE ? 1.f : ct;
+            if (!SH && in_tail) {
+                g_t = __ldcg(ptr[0] + q.begin + jj);
+                w_t = __ldcg(wp + jj);
+                if (HM) m_t = __ldcg(mp + jj);
+                if (use_se) c_t = __ldcg(ptr[HM ? 3 : 2] + q.begin + jj);
+            }
             if (nv == CH / 4) {
                 // Two columns per step of a rolled loop (unrolled over the tile, the body
                 // outgrew the instruction cache: 82.5 -> 75.5 us per ResNet-50 update pass).
@@ -1977,22 +2002,19 @@ __global__ void __launch_bounds__(Ring2<SH>::kThreads, 1)
                     awt = update_shifted<HM, PE, SW>(stage, tab, q.t, q.begin, (int)(q.end - q.begin), ct,
                                                      use_se, sc);
             }
-            const long long n = q.end - q.begin;
             const bool tile_tail = 4 * (long long)nv < n;  // the same in every lane
-            if (!SH || st.tc.aligned) {
-                // The last n % 4 elements: from the stage (SH) or by plain loads.
-                for (long long jj = 4 * (long long)nv + lane; jj < n; jj += 32) {
+            if (in_tail) {
+                if (SH) {
                     const uint32_t o = stage + 4u * (uint32_t)jj;
-                    const float g = SH ? lds1(o) : __ldcg(ptr[0] + q.begin + jj);
-                    float w = SH ? lds1(o + w_off) : __ldcg(wp + jj);
-                    float m = !HM ? 0.f : SH ? lds1(o + m_off) : __ldcg(mp + jj);
-                    const float cj = !use_se ? (PE ? 1.f : ct)
-                                     : SH    ? lds1(o + se_off) : __ldcg(ptr[HM ? 3 : 2] + q.begin + jj);
-                    if (SW) awt = __fma_rn((double)w, (double)w, awt);
-                    sgd1(g, cj, w, m, sc, HM);
-                    wp[jj] = w;
-                    if (HM) mp[jj] = m;
+                    g_t = lds1(o);
+                    w_t = lds1(o + w_off);
+                    if (HM) m_t = lds1(o + m_off);
+                    if (use_se) c_t = lds1(o + se_off);
                 }
+                if (SW) awt = __fma_rn((double)w_t, (double)w_t, awt);
+                sgd1(g_t, c_t, w_t, m_t, sc, HM);
+                wp[jj] = w_t;
+                if (HM) mp[jj] = m_t;
             }
             __syncwarp();
             const int tg = q.tg;
@@ -2354,8 +2376,9 @@ void build_blocks(int n, const int64_t *numels, int chunk, int np, const Pointer
         }
         cstart[cnt] = nc;
         tab->nc = nc;
-        for (int i = 0, t = 0; i < kHints; ++i) {
-            while (t + 1 < cnt && i * kHintTiles >= cstart[t + 1]) ++t;
+        while (((nc - 1) >> tab->hint_shift) >= kHints) ++tab->hint_shift;
+        for (int i = 0, t = 0; i < kHints + 2; ++i) {
+            while (t + 1 < cnt && ((long long)i << tab->hint_shift) >= cstart[t + 1]) ++t;
             tab->hint[i] = (unsigned short)t;
         }
         tabs.push_back(std::move(tab));
