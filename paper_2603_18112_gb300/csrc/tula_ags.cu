@@ -274,32 +274,6 @@ __device__ __forceinline__ float4 mean4(float4 s, const Scalars &sc) {
 }
 
 
-// Fixed-tree warp sum of R values at once (lane 0 gets the sums); the R chains
-// are independent, so their shuffle and fp64 add latencies overlap.
-template <int R>
-__device__ __forceinline__ void warp_sums(double (&v)[R]) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        double t[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) t[r] = __shfl_down_sync(kFull, v[r], o);
-#pragma unroll
-        for (int r = 0; r < R; ++r) v[r] = __dadd_rn(v[r], t[r]);
-    }
-}
-
-template <int R>
-__device__ __forceinline__ void warp_sums(float (&v)[R]) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        float t[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) t[r] = __shfl_down_sync(kFull, v[r], o);
-#pragma unroll
-        for (int r = 0; r < R; ++r) v[r] = __fadd_rn(v[r], t[r]);
-    }
-}
-
 // Warp reduce-scatter of R values per lane (R a power of two, <= 32): each of log2(R) halving
 // steps sends half of a lane's values to the lane `off` away and keeps the sums of the other
 // half; the remaining steps add the one value left across the lanes still sharing it.
@@ -854,17 +828,17 @@ struct Stream {
         const unsigned v = (unsigned)warp * gridDim.x + blockIdx.x;
         return v < nc ? (int)v : -1;
     }
-    // The first claim, once the first tile has been issued.
-    __device__ __forceinline__ void claim_first() {
+    // Claims the tile after the one just issued: after, because the warp may stop for the
+    // atomic's round trip here (its tile is on its way meanwhile; claimed before the copies, it
+    // kept every stage empty for about 1500 of a tile's 10,500 cycles).
+    __device__ __forceinline__ void claim() {
         if (claims && (threadIdx.x & 31) == 0) pend = atomicAdd(ctr, 1u);
     }
-    // The tile after the last one taken (-1: none left).
+    // The tile claimed last (-1: none left).
     __device__ __forceinline__ int next() {
         if (!claims) return -1;
         const unsigned c = __shfl_sync(kFull, pend, 0) + V;
-        if (c >= nc) return -1;
-        if ((threadIdx.x & 31) == 0) pend = atomicAdd(ctr, 1u);
-        return (int)c;
+        return c < nc ? (int)c : -1;
     }
     // Issues tile c, or of it only streams `from` .. ns - 1, the rest left to issue_below();
     // every lane has read what the stage held (a __syncwarp ago).
@@ -1046,7 +1020,7 @@ __device__ __noinline__ F3 tile_cols_scaled(uint32_t stage, int chunk, int nv, c
 }
 
 // A tile of a tensor off a 16-byte boundary (see issue_edge_tile() for where its elements lie): lane l
-// takes elements l, l + 32, ..., four at a time, with conflict-free 4-byte loads from shared
+// takes elements l, l + 32, ..., U at a time, with conflict-free 4-byte loads from shared
 // memory and coalesced 4-byte stores of the mean.  The squares are float-float pairs in either
 // mode: the elements of such tensors used to be squared in fp64, and these sums keep that
 // precision (relative error ~1e-15 a lane) without GB300's slow FP64 pipe.  Returns the lane's
@@ -1068,52 +1042,73 @@ __device__ __noinline__ D3 tile_shifted(uint32_t stage, int chunk, const Tab &ta
     const uint32_t at_w = RW ? at(K) : 0u;
     const uint32_t at_s = SS ? at(K) : 0u;
     float *out = ptr[0] + begin;
-    Dw4 ag, as, aw;
-    dw_zero(ag);
-    dw_zero(as);
-    dw_zero(aw);
-    for (int j0 = lane; j0 < n; j0 += 128) {
-        uint32_t o[4];  // byte offsets; past the end, the last element's (taken as 0)
-        bool in[4];
-        float x0[4], s[4], wv[4], sv[4];
+    // U elements per lane and step: their U independent chains hide one another's latency.
+    constexpr int U = KT >= 1 && KT <= 0 ? 8 : 4;
+    Dw4 ag[U / 4], as[U / 4], aw[U / 4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            in[u] = j0 + 32 * u < n;
-            o[u] = 4u * (uint32_t)min(j0 + 32 * u, n - 1);
+    for (int g = 0; g < U / 4; ++g) {
+        dw_zero(ag[g]);
+        dw_zero(as[g]);
+        dw_zero(aw[g]);
+    }
+    // One step from element j0 on; the elements past the end count as 0.
+    auto step = [&](int j0, auto whole) {
+        constexpr bool kWhole = decltype(whole)::value;
+        uint32_t o[U];  // byte offsets; past the end, the last element's
+        bool in[U];
+        float x0[U], s[U], y[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            in[u] = kWhole || j0 + 32 * u < n;
+            o[u] = 4u * (uint32_t)(kWhole ? j0 + 32 * u : min(j0 + 32 * u, n - 1));
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) s[u] = x0[u] = lds1(at_k[0] + o[u]);
+        for (int u = 0; u < U; ++u) s[u] = x0[u] = lds1(at_k[0] + o[u]);
         if constexpr (KT > 0) {
 #pragma unroll
             for (int k = 1; k < KT; ++k)
 #pragma unroll
-                for (int u = 0; u < 4; ++u) s[u] = __fadd_rn(s[u], lds1(at_k[k] + o[u]));
+                for (int u = 0; u < U; ++u) s[u] = __fadd_rn(s[u], lds1(at_k[k] + o[u]));
         } else {
             for (int k = 1; k < K; ++k) {
                 const uint32_t a = at(k);
 #pragma unroll
-                for (int u = 0; u < 4; ++u) s[u] = __fadd_rn(s[u], lds1(a + o[u]));
+                for (int u = 0; u < U; ++u) s[u] = __fadd_rn(s[u], lds1(a + o[u]));
             }
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            wv[u] = RW ? lds1(at_w + o[u]) : 0.f;
-            sv[u] = SS ? lds1(at_s + o[u]) : 0.f;
-        }
+        for (int u = 0; u < U; ++u) y[u] = RW || SS ? lds1((RW ? at_w : at_s) + o[u]) : 0.f;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u4 = 0; u4 < U; u4 += 4) {
             if (K > 1) {
-                s[u] = mean1<KT>(s[u], sc);
-                if (WM && in[u]) out[j0 + 32 * u] = s[u];
+                const float4 m = mean4<KT>(make_float4(s[u4], s[u4 + 1], s[u4 + 2], s[u4 + 3]), sc);
+                s[u4] = m.x;
+                s[u4 + 1] = m.y;
+                s[u4 + 2] = m.z;
+                s[u4 + 3] = m.w;
             }
-            dw_sq(ag.hi[u], ag.lo[u], in[u] ? s[u] : 0.f);
-            if (K > 1) dw_sq(as.hi[u], as.lo[u], in[u] ? x0[u] : 0.f);
-            if (SS) dw_sq(as.hi[u], as.lo[u], in[u] ? sv[u] : 0.f);
-            if (RW) dw_sq(aw.hi[u], aw.lo[u], in[u] ? wv[u] : 0.f);
         }
-    }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int g = u / 4, c = u % 4;
+            if (K > 1 && WM && in[u]) out[j0 + 32 * u] = s[u];
+            dw_sq(ag[g].hi[c], ag[g].lo[c], in[u] ? s[u] : 0.f);
+            if (K > 1) dw_sq(as[g].hi[c], as[g].lo[c], in[u] ? x0[u] : 0.f);
+            if (SS) dw_sq(as[g].hi[c], as[g].lo[c], in[u] ? y[u] : 0.f);
+            if (RW) dw_sq(aw[g].hi[c], aw[g].lo[c], in[u] ? y[u] : 0.f);
+        }
+    };
+    int j = lane;
+#pragma unroll 1
+    for (; j - lane + 32 * U <= n; j += 32 * U) step(j, std::true_type{});
+    if (j - lane < n) step(j, std::false_type{});
     __syncwarp();
-    const float2 pg = dw_pair(ag), ps = dw_pair(as), pw = dw_pair(aw);
+    float2 pg = dw_pair(ag[0]), ps = dw_pair(as[0]), pw = dw_pair(aw[0]);
+    if constexpr (U == 8) {
+        pg = ff_add(pg, dw_pair(ag[1]));
+        ps = ff_add(ps, dw_pair(as[1]));
+        pw = ff_add(pw, dw_pair(aw[1]));
+    }
     const bool bad = lane < n && !(dw_lane_ok(pg) && (!(K > 1 || SS) || dw_lane_ok(ps)) &&
                                    (!RW || dw_lane_ok(pw)));
     D3 r = {ff_to_double(pg), ff_to_double(ps), ff_to_double(pw)};
@@ -1386,13 +1381,53 @@ __device__ __forceinline__ void add_tail(const Scalars &sc, int tg, const double
         if (a == 0 && sc.mode == kModeStep) acc_add_f64(gacc_of(sc), d);
     }
 }
-// The fp64 sums of a shifted tile, reduced across the warp and added by lane 0.
-__device__ __noinline__ void add_shifted(const Scalars &sc, int tg, const double (&accd)[kAcc]) {
-    double d[kAcc];
+// The lanes' fp64 sums d[0 .. R) (>= 0, finite or not) of a shifted tile into R accumulators, and
+// the first one into `also` as well (unless NULL).  An fp64 tree across the warp took 4000 cycles of
+// a tile's 13,000 on GB300's slow FP64 pipe, so the lanes are added as integers: relative to the
+// warp's largest exponent a sum is a fixed-point number of 79 bits, limbs of 26, 26 and 27, and
+// each limb's warp total (below 2^32) takes one instruction.  What lies below 2^-78 of the largest
+// sum is cut off, less than an fp64 addition's own rounding.  The totals are exact integers and go
+// to the accumulators by a lane each (the lowest limb is zero where its weight lies below the
+// accumulators' 2^-352: squares of fp32 numbers are multiples of 2^-298).
+template <int R>
+__device__ __noinline__ void add_shifted(const double (&d)[R], unsigned long long *const (&A)[R],
+                                         unsigned long long *also) {
+    const int lane = threadIdx.x & 31;
+    unsigned sum = 0u;  // lane 3 r + i: limb i of sum r; lanes 3 R + i: of sum 0, for `also`
+    int ex = 0;
+    unsigned long long *to = nullptr;
 #pragma unroll
-    for (int a = 0; a < kAcc; ++a) d[a] = accd[a];
-    warp_sums<kAcc>(d);
-    if ((threadIdx.x & 31) == 0) add_tail(sc, tg, d);
+    for (int r = 0; r < R; ++r) {
+        const unsigned long long u = (unsigned long long)__double_as_longlong(d[r]);
+        const int e = (int)(u >> 52) & 0x7ff;
+        const int top = __reduce_max_sync(kFull, e);
+        if (top == 0x7ff) {  // an inf or a NaN: its lanes flag it, and nothing else counts
+            if (e == 0x7ff) {
+                acc_add_f64(A[r], d[r]);
+                if (r == 0 && also) acc_add_f64(also, d[r]);
+            }
+            continue;
+        }
+        // e == 0: zero (a square of an fp32 number is far above fp64's subnormal range)
+        const unsigned long long m = e ? (u & 0xfffffffffffffull) | (1ull << 52) : 0ull;
+        const int shift = top - e;
+        // Bits 78 .. 26: m >> shift; bits 25 .. 0: the first 26 of those that cuts off.
+        const unsigned long long hi = shift < 64 ? m >> shift : 0ull;
+        const unsigned long long cut = shift == 0 ? 0ull
+                                       : shift < 64 ? m << (64 - shift) : shift < 128 ? m >> (shift - 64) : 0ull;
+        const unsigned low = (unsigned)(cut >> 38);
+        const unsigned l0 = __reduce_add_sync(kFull, low);
+        const unsigned l1 = __reduce_add_sync(kFull, (unsigned)(hi & 0x3ffffffull));
+        const unsigned l2 = __reduce_add_sync(kFull, (unsigned)(hi >> 26));
+        const int i = lane - 3 * r, j = lane - 3 * R;
+        if ((i >= 0 && i < 3) || (r == 0 && also && j >= 0 && j < 3)) {
+            const int limb = i >= 0 && i < 3 ? i : j;
+            sum = limb == 0 ? l0 : limb == 1 ? l1 : l2;
+            ex = top - 1075 - 26 + 26 * limb;
+            to = i >= 0 && i < 3 ? A[r] : also;
+        }
+    }
+    if (to) acc_add(to, sum, ex);
 }
 
 template <int KT, bool WM, bool RW, bool SS, bool PR, bool SH, bool Small>
@@ -1423,7 +1458,7 @@ __global__ void __launch_bounds__(Ring1Of<KT, RW, SH>::kThreads, 1)
     int c = st.start(smem, tab.nc, sc.tiles + 4 * (tab.seq & 1), sc.evict_first != 0);
     TilePos q = {};
     if (c >= 0) q = st.issue(tab, c, chunk, role, ns);
-    st.claim_first();
+    st.claim();
     if (first && early) {
         grid_wait();
         grid_launch_dependents();
@@ -1470,7 +1505,10 @@ __global__ void __launch_bounds__(Ring1Of<KT, RW, SH>::kThreads, 1)
             const int tg = q.tg;
             const bool shifted = SH && !st.tc.aligned;
             c = st.next();
-            if (c >= 0) q = st.issue(tab, c, chunk, role, ns);
+            if (c >= 0) {
+                q = st.issue(tab, c, chunk, role, ns);
+                st.claim();
+            }
             if (to_wait) {
                 grid_wait();
                 grid_launch_dependents();
@@ -1479,7 +1517,9 @@ __global__ void __launch_bounds__(Ring1Of<KT, RW, SH>::kThreads, 1)
             if constexpr (!PR) {
                 if (tile_tail) {
                     if (SH && shifted) {
-                        add_shifted(sc, tg, accd);
+                        unsigned long long *const A[kAcc] = {acc1_of(sc, tg, 0), acc1_of(sc, tg, 1),
+                                                             acc1_of(sc, tg, 2)};
+                        add_shifted<kAcc>(accd, A, step_g2 ? gacc_of(sc) : nullptr);
                         continue;
                     }
                     add_tail(sc, tg, accd);
@@ -1809,13 +1849,15 @@ __device__ __noinline__ double update_shifted(uint32_t stage, const Tab &tab, in
     float *mp = HM ? ptr[2] + begin : nullptr;
     Dw4 aw;
     dw_zero(aw);
-    for (int j0 = lane; j0 < n; j0 += 128) {
+    // One step from element j0 on; the elements past the end count as 0.
+    auto step = [&](int j0, auto whole) {
+        constexpr bool kWhole = decltype(whole)::value;
         float g[4], w[4], m[4], c[4];
         bool in[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            in[u] = j0 + 32 * u < n;
-            const uint32_t o = 4u * (uint32_t)min(j0 + 32 * u, n - 1);
+            in[u] = kWhole || j0 + 32 * u < n;
+            const uint32_t o = 4u * (uint32_t)(kWhole ? j0 + 32 * u : min(j0 + 32 * u, n - 1));
             g[u] = lds1(at_g + o);
             w[u] = lds1(at_w + o);
             m[u] = HM ? lds1(at_m + o) : 0.f;
@@ -1830,7 +1872,11 @@ __device__ __noinline__ double update_shifted(uint32_t stage, const Tab &tab, in
                 if (HM) __stcs(mp + j0 + 32 * u, m[u]);
             }
         }
-    }
+    };
+    int j0 = lane;
+#pragma unroll 1
+    for (; j0 - lane + 128 <= n; j0 += 128) step(j0, std::true_type{});
+    if (j0 - lane < n) step(j0, std::false_type{});
     __syncwarp();
     if (!SW) return 0.0;
     const float2 pw = dw_pair(aw);
@@ -1895,7 +1941,7 @@ __global__ void __launch_bounds__(Ring2<SH>::kThreads, 1)
     int c = st.start(smem, tab.nc, sc.tiles + 4 * (tab.seq & 1) + 2, sc.evict_first != 0);
     TilePos q = {};
     if (c >= 0) q = st.issue(tab, c, chunk, role, ns, early ? kEarlyFrom : 0);
-    st.claim_first();
+    st.claim();
     if (early) {
         grid_wait();
         grid_launch_dependents();
@@ -2020,7 +2066,10 @@ __global__ void __launch_bounds__(Ring2<SH>::kThreads, 1)
             const int tg = q.tg;
             const bool shifted = SH && !st.tc.aligned;
             c = st.next();
-            if (c >= 0) q = st.issue(tab, c, chunk, role, ns);
+            if (c >= 0) {
+                q = st.issue(tab, c, chunk, role, ns);
+                st.claim();
+            }
             if (to_wait) {
                 grid_wait();
                 grid_launch_dependents();
@@ -2028,9 +2077,9 @@ __global__ void __launch_bounds__(Ring2<SH>::kThreads, 1)
             }
             if (SW) {
                 if (SH && shifted) {
-                    double d[1] = {awt};
-                    warp_sums<1>(d);
-                    if (lane == 0) acc_add_f64(acc2_of(sc, tg), d[0]);
+                    const double d[1] = {awt};
+                    unsigned long long *const A[1] = {acc2_of(sc, tg)};
+                    add_shifted<1>(d, A, nullptr);
                     continue;
                 }
                 if (tile_tail && lane < 3) acc_add_f64(acc2_of(sc, tg), awt);  // as add_tail
