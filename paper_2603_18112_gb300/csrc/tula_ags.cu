@@ -196,7 +196,8 @@ struct Scalars {
     unsigned long long *gacc;  // [kGCopies][kAccWords]: |G|^2 = every tensor's |gbar|^2
     unsigned long long *acc2;  // [tensor][kTCopies][kAccWords]: |w|^2, pass 2
     float *cand;               // [tensor]: c_p of a LARS step
-    unsigned *tiles;           // [4 * (seq & 1) + 2 * pass]: next tile to claim, warps finished
+    unsigned *tiles;           // [2 * (seq & 1) + pass]: claims made
+    unsigned claim_base;       // of them, by the pass's launches before this one on this counter
     const unsigned long long *g2ext;  // a sharded step's |G|^2: the ranks' shares summed (or NULL)
 };
 
@@ -739,10 +740,13 @@ struct TensorCache {
 // when there are more tiles than warps, tiles claimed one at a time from a global counter
 // (ctr[0]), the claim made a whole tile ahead so that its round trip is never waited for.  SMs
 // stream at unequal rates; with 36 KB tiles claims run at 7.19-7.25 TB/s where a fixed deal runs
-// at 6.95.  (Tiles under ~18 KB would be bound by the counter: one atomic every 1.5-2.8 ns.)  The
-// last warp to finish puts both counters (ctr[0], ctr[1]) back to zero.  Where a tile is processed
-// never changes its result: each tile's partial sums are added exactly, in integers, into its
-// tensor's accumulators.
+// at 6.95.  (Tiles under ~18 KB would be bound by the counter: one atomic every 1.5-2.8 ns.)  A
+// launch of nc tiles that claims makes exactly nc claims (nc - V tiles and one past the end for
+// each warp), so the host knows where the next launch on the counter begins, and nobody waits at
+// the end of a launch to re-arm it: the update does that for pass 1, k_finish for pass 2.  (A fence
+// and a ticket per warp for it took about 1 us at the end of each pass.)  Where a tile is
+// processed never changes its result: each tile's partial sums are added exactly, in integers,
+// into its tensor's accumulators.
 //
 // Any 4-byte aligned tensor moves this way.  When some stream of a tensor lies off a 16-byte
 // boundary (views into a flat bucket, say), its tiles are shifted: stream i's part of the stage
@@ -797,7 +801,7 @@ struct Stream {
     uint32_t stage;  // shared-memory address of this warp's stage
     uint64_t *bar;   // its mbarrier: one arrival, which arms the bytes of all streams
     uint32_t phase = 0;
-    unsigned nc, V;
+    unsigned nc, V, base;
     bool claims;
     unsigned *ctr;
     unsigned pend = 0;  // lane 0: the claim in flight
@@ -808,7 +812,7 @@ struct Stream {
 
     // Barrier init; returns this warp's first tile (-1: none).  Called by the whole CTA.
     __device__ __forceinline__ int start(unsigned char *smem, int n_tiles, unsigned *counter,
-                                         bool evict_first) {
+                                         const Scalars &sc) {
         const int warp = threadIdx.x >> 5;
         stage = smem_addr(smem) + (uint32_t)warp * R::kStageBytes;
         bar = reinterpret_cast<uint64_t *>(smem + R::kWarps * R::kStageBytes) + warp;
@@ -821,7 +825,8 @@ struct Stream {
         V = gridDim.x * (unsigned)R::kWarps;
         claims = nc > V;
         ctr = counter;
-        hint = evict_first;
+        base = sc.claim_base;
+        hint = sc.evict_first != 0;
         policy = policy_evict_first();
         // cp.async reads through L1: nothing there from before this kernel.
         if constexpr (SH) __threadfence();
@@ -837,7 +842,7 @@ struct Stream {
     // The tile claimed last (-1: none left).
     __device__ __forceinline__ int next() {
         if (!claims) return -1;
-        const unsigned c = __shfl_sync(kFull, pend, 0) + V;
+        const unsigned c = __shfl_sync(kFull, pend, 0) - base + V;
         return c < nc ? (int)c : -1;
     }
     // Issues tile c, or of it only streams `from` .. ns - 1, the rest left to issue_below();
@@ -897,16 +902,6 @@ struct Stream {
             __syncwarp();
         }
         return ok;
-    }
-    // After the warp's last tile: the last warp of the launch re-arms the counters.
-    __device__ __forceinline__ void finish() {
-        if (claims && (threadIdx.x & 31) == 0) {
-            __threadfence();
-            if (atomicAdd(ctr + 1, 1u) == V - 1u) {
-                atomicExch(ctr, 0u);
-                atomicExch(ctr + 1, 0u);
-            }
-        }
     }
 };
 
@@ -1455,7 +1450,7 @@ __global__ void __launch_bounds__(Ring1Of<KT, RW, SH>::kThreads, 1)
     const int ns = K + (RW ? 1 : 0) + (SS ? 1 : 0);
     const int role = lane < ns ? lane : 0;
     Stream<Ring1Of<KT, RW, SH>, SH> st;
-    int c = st.start(smem, tab.nc, sc.tiles + 4 * (tab.seq & 1), sc.evict_first != 0);
+    int c = st.start(smem, tab.nc, sc.tiles + 2 * (tab.seq & 1), sc);
     TilePos q = {};
     if (c >= 0) q = st.issue(tab, c, chunk, role, ns);
     st.claim();
@@ -1561,7 +1556,6 @@ __global__ void __launch_bounds__(Ring1Of<KT, RW, SH>::kThreads, 1)
         }
     }
     if (to_wait) grid_wait();
-    st.finish();
 }
 
 // ----------------------------------------------------------------------------
@@ -1745,9 +1739,14 @@ __global__ void __launch_bounds__(32 * kFinWarps) k_finish(const __grid_constant
     const int n = sc.n_total;
     const bool step = sc.mode == kModeStep;
     grid_wait();
-    // The next call's reduction may start now: it only reads replicas until this kernel has
-    // completed.
-    grid_launch_dependents();
+    // After a step, the next call's reduction may start now: it only reads replicas, and claims
+    // tiles, until this kernel has completed.  (After the other calls it would find their pass's
+    // counters not re-armed yet.)
+    if (step) grid_launch_dependents();
+    if (t == 0 && lane == 0) {
+        const int pass = step ? 1 : 0;
+        sc.tiles[pass] = sc.tiles[2 + pass] = 0u;
+    }
     if (t > n || (t == n && !step)) return;
     if (t == n) {  // the step record
         const double g2_prev = sc.state[TULA_STATE_G2_PREV], steps = sc.state[TULA_STATE_STEPS];
@@ -1912,6 +1911,11 @@ __global__ void __launch_bounds__(Ring2<SH>::kThreads, 1)
         grid_wait();
         grid_launch_dependents();
     }
+    // The reduction has completed: its tile counters for the next call.
+    auto rearm_pass1 = [&]() {
+        if (blockIdx.x == 0 && threadIdx.x == 0) sc.tiles[0] = sc.tiles[2] = 0u;
+    };
+    if (first && !early) rearm_pass1();
     __shared__ int branch;
     const bool gated = sc.rule == TULA_RULE_AGS || sc.rule == TULA_RULE_STATIC;
     // Called by the whole CTA after its wait: every CTA forms the branch from the accumulator for
@@ -1938,7 +1942,7 @@ __global__ void __launch_bounds__(Ring2<SH>::kThreads, 1)
     const uint32_t se_off = (uint32_t)((HM ? 3 : 2) * CH * 4);
     constexpr int kEarlyFrom = HM && !SH ? 2 : 1;  // streams from here on are issued early
     Stream<Ring2<SH>, SH> st;
-    int c = st.start(smem, tab.nc, sc.tiles + 4 * (tab.seq & 1) + 2, sc.evict_first != 0);
+    int c = st.start(smem, tab.nc, sc.tiles + 2 * (tab.seq & 1) + 1, sc);
     TilePos q = {};
     if (c >= 0) q = st.issue(tab, c, chunk, role, ns, early ? kEarlyFrom : 0);
     st.claim();
@@ -1946,6 +1950,7 @@ __global__ void __launch_bounds__(Ring2<SH>::kThreads, 1)
         grid_wait();
         grid_launch_dependents();
         if (c >= 0) st.issue_below(q, kEarlyFrom, ns, chunk);
+        rearm_pass1();
         scaled = take_branch();
     }
     bool to_wait = !first;
@@ -2106,7 +2111,6 @@ __global__ void __launch_bounds__(Ring2<SH>::kThreads, 1)
         }
     }
     if (to_wait) grid_wait();
-    st.finish();
 }
 
 // ----------------------------------------------------------------------------
@@ -2442,9 +2446,10 @@ struct StreamKernels {
     void (*shifted)(TableOf<false>, Scalars);
     int smem, smem_shifted;
 };
+// base: claims made so far on the launch's tile counter.
 template <typename Tab>
 int launch_block(void (*fn)(Tab, Scalars), const void *block, int threads, int smem,
-                 const Scalars &sc, int grid_override, cudaStream_t stream) {
+                 const Scalars &call, int grid_override, cudaStream_t stream, unsigned (&base)[2]) {
     const Tab &tab = *static_cast<const Tab *>(block);
     int grid = resident_ctas((const void *)fn, threads, smem);
     if (grid <= 0) {
@@ -2453,6 +2458,9 @@ int launch_block(void (*fn)(Tab, Scalars), const void *block, int threads, int s
     }
     if (grid_override > 0) grid = grid_override;
     grid = std::max(1, std::min(grid, tab.nc));
+    Scalars sc = call;
+    sc.claim_base = base[tab.seq & 1];
+    if ((long long)tab.nc > (long long)grid * (threads / 32)) base[tab.seq & 1] += (unsigned)tab.nc;
     return launch_pdl(fn, grid, threads, smem, stream, tab, sc);
 }
 // Launches a streaming kernel once per parameter block.  With a cache, the blocks are taken from
@@ -2480,14 +2488,15 @@ int launch_streaming(const StreamKernels &k, int n, const int64_t *numels, int c
         }
         if (!blocks) blocks = &built;
     }
+    unsigned base[2] = {0u, 0u};
     for (const auto &b : blocks->tabs) {
         int rc;
         if (blocks->small)
-            rc = launch_block(k.small, b.get(), threads, k.smem, sc, grid_override, stream);
+            rc = launch_block(k.small, b.get(), threads, k.smem, sc, grid_override, stream, base);
         else if (static_cast<const FullTab *>(b.get())->shifted)
-            rc = launch_block(k.shifted, b.get(), threads, k.smem_shifted, sc, grid_override, stream);
+            rc = launch_block(k.shifted, b.get(), threads, k.smem_shifted, sc, grid_override, stream, base);
         else
-            rc = launch_block(k.full, b.get(), threads, k.smem, sc, grid_override, stream);
+            rc = launch_block(k.full, b.get(), threads, k.smem, sc, grid_override, stream, base);
         if (rc) return rc;
     }
     return TULA_OK;
