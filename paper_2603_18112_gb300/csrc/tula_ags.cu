@@ -241,9 +241,15 @@ __device__ __forceinline__ float4 add4(float4 a, float4 b) {
                        __fadd_rn(a.w, b.w));
 }
 
-// Eq. 1c: divide the k-ascending sum by K (exact reciprocal when K is a power of 2)
+// Eq. 1c: divide the k-ascending sum by K (exact reciprocal when K is a power of 2).  K by value,
+// for the same reason as Sgd.
+struct MeanK {
+    int pow2K;
+    float invK, Kf;
+};
+__device__ __forceinline__ MeanK mean_k(const Scalars &sc) { return {sc.pow2K, sc.invK, sc.Kf}; }
 template <int KT>
-__device__ __forceinline__ float mean1(float s, const Scalars &sc) {
+__device__ __forceinline__ float mean1(float s, const MeanK &sc) {
     if constexpr (KT > 0 && (KT & (KT - 1)) == 0) {
         return __fmul_rn(s, 1.0f / (float)KT);
     } else if constexpr (KT > 0) {
@@ -261,12 +267,12 @@ __device__ __forceinline__ bool mean_in_range(float s) {
     return __float_as_uint(fabsf(s)) - __float_as_uint(0x1p-90f) <
            0x7f800000u - __float_as_uint(0x1p-90f);
 }
-__device__ __forceinline__ float mean_fast(float s, const Scalars &sc) {
+__device__ __forceinline__ float mean_fast(float s, const MeanK &sc) {
     const float q = __fmul_rn(s, sc.invK);
     return __fmaf_rn(__fmaf_rn(-sc.Kf, q, s), sc.invK, q);
 }
 template <int KT>
-__device__ __forceinline__ float4 mean4(float4 s, const Scalars &sc) {
+__device__ __forceinline__ float4 mean4(float4 s, const MeanK &sc) {
     if (KT == 0 && mean_in_range(s.x) && mean_in_range(s.y) && mean_in_range(s.z) &&
         mean_in_range(s.w))  // (K a power of two as well: its remainders are 0)
         return make_float4(mean_fast(s.x, sc), mean_fast(s.y, sc), mean_fast(s.z, sc),
@@ -929,23 +935,29 @@ struct Stream {
 // Pointer roles per tensor: [0, K) replicas, K = w (RW) or g_small (SS).
 // Stage streams: replicas 0..K-1, then w (RW), then g_small (SS).
 
+// Whether there is more than one replica: K = 1 has a kernel of its own, so that this is known at
+// compile time for a K that is not.  (Tested at run time, it kept the four elements' chains of a
+// step apart: a shifted tile with K = 3 took 21,000 cycles, and @@ so.)
+template <int KT>
+constexpr bool kMulti = KT != 1;
+
 // One float4 column of a tile: mean, squares.  x0 = replica 0, s = sum.
 template <int KT, bool WM, bool RW, bool SS, bool PR>
 __device__ __forceinline__ void column1(float4 x0, float4 s, float4 wv, float4 sv, float *out,
                                         const Scalars &sc, int K, Dw4 &ag, Dw4 &as, Dw4 &aw,
                                         float &pg, float &ps, float &pw) {
-    if (K > 1) {
-        s = mean4<KT>(s, sc);
+    if (kMulti<KT>) {
+        s = mean4<KT>(s, mean_k(sc));
         if (WM) st_keep(out, s);
     }
     if (PR) {
         dw_sq4(ag, s);
-        if (K > 1) dw_sq4(as, x0);
+        if (kMulti<KT>) dw_sq4(as, x0);
         if (SS) dw_sq4(as, sv);
         if (RW) dw_sq4(aw, wv);
     } else {
         pg = sq4(pg, s);
-        if (K > 1) ps = sq4(ps, x0);
+        if (kMulti<KT>) ps = sq4(ps, x0);
         if (SS) ps = sq4(ps, sv);
         if (RW) pw = sq4(pw, wv);
     }
@@ -969,7 +981,7 @@ __device__ __noinline__ D3 tile_cols_fp64(uint32_t stage, int chunk, int nv, con
         const float4 x0 = lds4(stage + (uint32_t)(16 * v));
         float4 s = x0;
         for (int k = 1; k < K; ++k) s = add4(s, lds4(stage + (uint32_t)((k * chunk + 4 * v) * 4)));
-        if (K > 1) s = mean4<KT>(s, sc);
+        if (kMulti<KT>) s = mean4<KT>(s, mean_k(sc));
         const float gs[4] = {s.x, s.y, s.z, s.w};
         const float g0[4] = {x0.x, x0.y, x0.z, x0.w};
         float4 wv = make_float4(0.f, 0.f, 0.f, 0.f), sv = wv;
@@ -979,7 +991,7 @@ __device__ __noinline__ D3 tile_cols_fp64(uint32_t stage, int chunk, int nv, con
         const float ss[4] = {sv.x, sv.y, sv.z, sv.w};
         for (int c = 0; c < 4; ++c) {
             r.g = __fma_rn((double)gs[c], (double)gs[c], r.g);
-            if (K > 1) r.s = __fma_rn((double)g0[c], (double)g0[c], r.s);
+            if (kMulti<KT>) r.s = __fma_rn((double)g0[c], (double)g0[c], r.s);
             if (SS) r.s = __fma_rn((double)ss[c], (double)ss[c], r.s);
             if (RW) r.w = __fma_rn((double)ws[c], (double)ws[c], r.w);
         }
@@ -1006,9 +1018,9 @@ __device__ __noinline__ F3 tile_cols_scaled(uint32_t stage, int chunk, int nv, c
         const float4 x0 = lds4(stage + (uint32_t)(16 * v));
         float4 s = x0;
         for (int k = 1; k < K; ++k) s = add4(s, lds4(stage + (uint32_t)((k * chunk + 4 * v) * 4)));
-        if (K > 1) s = mean4<KT>(s, sc);
+        if (kMulti<KT>) s = mean4<KT>(s, mean_k(sc));
         r.g = sq4(r.g, mul4(s, fg));
-        if (K > 1) r.s = sq4(r.s, mul4(x0, fs));
+        if (kMulti<KT>) r.s = sq4(r.s, mul4(x0, fs));
         if (SS) r.s = sq4(r.s, mul4(lds4(ss_s + (uint32_t)(16 * v)), fs));
         if (RW) r.w = sq4(r.w, mul4(lds4(sw_s + (uint32_t)(16 * v)), fw));
     }
@@ -1025,11 +1037,18 @@ template <int KT, bool WM, bool RW, bool SS, typename Tab>
 __device__ __noinline__ D3 tile_shifted(uint32_t stage, int chunk, const Tab &tab, int t,
                                         long long begin, int n, const Scalars &sc) {
     const Row<Tab> ptr{tab, t};
+    const MeanK mk = mean_k(sc);
     const int lane = threadIdx.x & 31;
     const int K = KT > 0 ? KT : sc.K;
     const uint32_t part = (uint32_t)(4 * chunk + kShiftBytes);
-    auto at = [&](int role) {  // roles and streams are the same here
-        return stage + (uint32_t)role * part + ((uint32_t)reinterpret_cast<uintptr_t>(ptr[role]) & 12u);
+    // The streams' places within 16 bytes, two bits each (roles and streams are the same here): a
+    // look-up in the table for every load costs more than the load.
+    constexpr bool kExtra = RW || SS;
+    unsigned long long phases = 0ull;
+    for (int i = 0; i < K + (kExtra ? 1 : 0); ++i)
+        phases |= (unsigned long long)((reinterpret_cast<uintptr_t>(ptr[i]) >> 2) & 3u) << (2 * i);
+    auto at = [&](int i) {
+        return stage + (uint32_t)i * part + ((uint32_t)(phases >> (2 * i)) & 3u) * 4u;
     };
     uint32_t at_k[KT > 0 ? KT : 1];
 #pragma unroll
@@ -1076,8 +1095,8 @@ __device__ __noinline__ D3 tile_shifted(uint32_t stage, int chunk, const Tab &ta
         for (int u = 0; u < U; ++u) y[u] = RW || SS ? lds1((RW ? at_w : at_s) + o[u]) : 0.f;
 #pragma unroll
         for (int u4 = 0; u4 < U; u4 += 4) {
-            if (K > 1) {
-                const float4 m = mean4<KT>(make_float4(s[u4], s[u4 + 1], s[u4 + 2], s[u4 + 3]), sc);
+            if (kMulti<KT>) {
+                const float4 m = mean4<KT>(make_float4(s[u4], s[u4 + 1], s[u4 + 2], s[u4 + 3]), mk);
                 s[u4] = m.x;
                 s[u4 + 1] = m.y;
                 s[u4 + 2] = m.z;
@@ -1087,9 +1106,9 @@ __device__ __noinline__ D3 tile_shifted(uint32_t stage, int chunk, const Tab &ta
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int g = u / 4, c = u % 4;
-            if (K > 1 && WM && in[u]) out[j0 + 32 * u] = s[u];
+            if (kMulti<KT> && WM && in[u]) out[j0 + 32 * u] = s[u];
             dw_sq(ag[g].hi[c], ag[g].lo[c], in[u] ? s[u] : 0.f);
-            if (K > 1) dw_sq(as[g].hi[c], as[g].lo[c], in[u] ? x0[u] : 0.f);
+            if (kMulti<KT>) dw_sq(as[g].hi[c], as[g].lo[c], in[u] ? x0[u] : 0.f);
             if (SS) dw_sq(as[g].hi[c], as[g].lo[c], in[u] ? y[u] : 0.f);
             if (RW) dw_sq(aw[g].hi[c], aw[g].lo[c], in[u] ? y[u] : 0.f);
         }
@@ -1105,7 +1124,7 @@ __device__ __noinline__ D3 tile_shifted(uint32_t stage, int chunk, const Tab &ta
         ps = ff_add(ps, dw_pair(as[1]));
         pw = ff_add(pw, dw_pair(aw[1]));
     }
-    const bool bad = lane < n && !(dw_lane_ok(pg) && (!(K > 1 || SS) || dw_lane_ok(ps)) &&
+    const bool bad = lane < n && !(dw_lane_ok(pg) && (!(kMulti<KT> || SS) || dw_lane_ok(ps)) &&
                                    (!RW || dw_lane_ok(pw)));
     D3 r = {ff_to_double(pg), ff_to_double(ps), ff_to_double(pw)};
     if (__any_sync(kFull, bad)) {  // as tile_cols_fp64: again, every square exact in fp64
@@ -1115,9 +1134,9 @@ __device__ __noinline__ D3 tile_shifted(uint32_t stage, int chunk, const Tab &ta
             const float x0 = lds1(at_k[0] + o);
             float s = x0;
             for (int k = 1; k < K; ++k) s = __fadd_rn(s, lds1(at(k) + o));
-            if (K > 1) s = mean1<KT>(s, sc);
+            if (kMulti<KT>) s = mean1<KT>(s, mk);
             r.g = __fma_rn((double)s, (double)s, r.g);
-            if (K > 1) r.s = __fma_rn((double)x0, (double)x0, r.s);
+            if (kMulti<KT>) r.s = __fma_rn((double)x0, (double)x0, r.s);
             if (SS) {
                 const double y = (double)lds1(at_s + o);
                 r.s = __fma_rn(y, y, r.s);
@@ -1158,7 +1177,7 @@ __device__ __forceinline__ void reduce_tile(uint32_t stage, int chunk, const Row
         const D3 d = tile_shifted<KT, WM, RW, SS>(stage, chunk, ptr.tab, ptr.t, q.begin,
                                                          (int)(q.end - q.begin), sc);
         accd[0] = d.g;
-        accd[1] = (K > 1 || SS) ? d.s : d.g;  // K = 1: replica 0 is the mean
+        accd[1] = (kMulti<KT> || SS) ? d.s : d.g;  // K = 1: replica 0 is the mean
         accd[2] = d.w;
         accf[0] = accf[1] = accf[2] = 0.f;
         acce[0] = acce[1] = acce[2] = 0;
@@ -1198,7 +1217,7 @@ __device__ __forceinline__ void reduce_tile(uint32_t stage, int chunk, const Row
                 }
                 if (!PR) {
                     fg = __fadd_rn(fg, pg);
-                    if (K > 1 || SS) fs = __fadd_rn(fs, ps);
+                    if (kMulti<KT> || SS) fs = __fadd_rn(fs, ps);
                     if (RW) fw = __fadd_rn(fw, pw);
                 }
             }
@@ -1266,7 +1285,7 @@ __device__ __forceinline__ void reduce_tile(uint32_t stage, int chunk, const Row
             }
             if (!PR) {
                 fg = __fadd_rn(fg, pg);
-                if (K > 1 || SS) fs = __fadd_rn(fs, ps);
+                if (kMulti<KT> || SS) fs = __fadd_rn(fs, ps);
                 if (RW) fw = __fadd_rn(fw, pw);
             }
         }
@@ -1285,11 +1304,11 @@ __device__ __forceinline__ void reduce_tile(uint32_t stage, int chunk, const Row
                     s = __fadd_rn(s, SH ? lds1(stage + (uint32_t)(4 * k * chunk) + o)
                                         : __ldcg(ptr[k] + j));
             }
-            if (K > 1) {
-                s = mean1<KT>(s, sc);
+            if (kMulti<KT>) {
+                s = mean1<KT>(s, mean_k(sc));
                 if (WM) out0[j] = s;
             }
-            if (K > 1) rs = __fma_rn((double)x0, (double)x0, rs);
+            if (kMulti<KT>) rs = __fma_rn((double)x0, (double)x0, rs);
             rg = __fma_rn((double)s, (double)s, rg);
             if (RW || SS) {  // role K
                 const float y = SH ? lds1((RW ? sw_s : ss_s) + o)
@@ -1302,7 +1321,7 @@ __device__ __forceinline__ void reduce_tile(uint32_t stage, int chunk, const Row
     if (PR) {
         // The warp is converged again here (the loops above end in every lane).
         const float2 pg = dw_pair(ag), ps = dw_pair(as), pw = dw_pair(aw);
-        const bool bad = lane < ncols && !(dw_lane_ok(pg) && (!(K > 1 || SS) || dw_lane_ok(ps)) &&
+        const bool bad = lane < ncols && !(dw_lane_ok(pg) && (!(kMulti<KT> || SS) || dw_lane_ok(ps)) &&
                                            (!RW || dw_lane_ok(pw)));
         double cg, cs, cw;
         if (__any_sync(kFull, bad)) {
@@ -1316,18 +1335,18 @@ __device__ __forceinline__ void reduce_tile(uint32_t stage, int chunk, const Row
             cw = ff_to_double(pw);
         }
         accd[0] = __dadd_rn(cg, rg);
-        accd[1] = (K > 1 || SS) ? __dadd_rn(cs, rs) : accd[0];  // K = 1: replica 0 is the mean
+        accd[1] = (kMulti<KT> || SS) ? __dadd_rn(cs, rs) : accd[0];  // K = 1: replica 0 is the mean
         accd[2] = RW ? __dadd_rn(cw, rw) : 0.0;
     } else {
         // The warp is converged again here; ncols is the same in every lane.
         int eg = 0, es = 0, ew = 0;
         // One vote per tile; the warp maxima only when some lane is out of range.  A lane
         // without columns (lane >= ncols) has nothing to check.
-        const bool lane_ok = lane >= ncols || (sq_in_range(fg) && (!(K > 1 || SS) || sq_in_range(fs)) &&
+        const bool lane_ok = lane >= ncols || (sq_in_range(fg) && (!(kMulti<KT> || SS) || sq_in_range(fs)) &&
                                                (!RW || sq_in_range(fw)));
         if (ncols > 0 && !__all_sync(kFull, lane_ok)) {
             eg = sq_range_exp(fg);
-            if (K > 1 || SS) es = sq_range_exp(fs);
+            if (kMulti<KT> || SS) es = sq_range_exp(fs);
             if (RW) ew = sq_range_exp(fw);
             if (eg | es | ew) {
                 const F3 r = tile_cols_scaled<KT, RW, SS>(stage, chunk, ncols, sc, pow2f(eg),
@@ -1335,11 +1354,11 @@ __device__ __forceinline__ void reduce_tile(uint32_t stage, int chunk, const Row
                 if (eg) fg = r.g;
                 if (es) fs = r.s;
                 if (ew) fw = r.w;
-                const bool own = K > 1 || SS;
+                const bool own = kMulti<KT> || SS;
                 ecode = scale_code(eg) | scale_code(own ? es : eg) << 2 | scale_code(ew) << 4;
             }
         }
-        const bool own_s = K > 1 || SS;  // K = 1: replica 0 is the mean
+        const bool own_s = kMulti<KT> || SS;  // K = 1: replica 0 is the mean
         accf[0] = fg;
         acce[0] = eg;
         accd[0] = rg;
@@ -1797,7 +1816,14 @@ __global__ void __launch_bounds__(32 * kFinWarps) k_finish(const __grid_constant
 // Pointer roles: 0 = gbar, 1 = w, then m (HM), then the per-element gradscale (PE).
 // Stage streams: gbar, w, then m (HM), then the per-element scale (PE, scaled).
 
-__device__ __forceinline__ void sgd1(float g, float c, float &w, float &m, const Scalars &sc,
+// The step's scalars by value: an out-of-line function that stores through float pointers would
+// have to load them again after every store (the shifted update's tiles took 7000 cycles, and 
+// @@ so).
+struct Sgd {
+    float lr, mu, wd;
+};
+__device__ __forceinline__ Sgd sgd_of(const Scalars &sc) { return {sc.lr, sc.mu, sc.wd}; }
+__device__ __forceinline__ void sgd1(float g, float c, float &w, float &m, const Sgd &sc,
                                      bool has_m) {
     const float gt = __fmul_rn(c, g);
     const float d = __fadd_rn(gt, __fmul_rn(sc.wd, w));
@@ -1814,10 +1840,10 @@ template <bool HM>
 __device__ __forceinline__ float update4(float4 g4, float4 w4, float4 m4, float4 cc, float *wp,
                                          float *mp, const Scalars &sc, float pw) {
     pw = sq4(pw, w4);
-    sgd1(g4.x, cc.x, w4.x, m4.x, sc, HM);
-    sgd1(g4.y, cc.y, w4.y, m4.y, sc, HM);
-    sgd1(g4.z, cc.z, w4.z, m4.z, sc, HM);
-    sgd1(g4.w, cc.w, w4.w, m4.w, sc, HM);
+    sgd1(g4.x, cc.x, w4.x, m4.x, sgd_of(sc), HM);
+    sgd1(g4.y, cc.y, w4.y, m4.y, sgd_of(sc), HM);
+    sgd1(g4.z, cc.z, w4.z, m4.z, sgd_of(sc), HM);
+    sgd1(g4.w, cc.w, w4.w, m4.w, sgd_of(sc), HM);
     st_stream(wp, w4);
     if (HM) st_stream(mp, m4);
     return pw;
@@ -1848,6 +1874,7 @@ __device__ __noinline__ double update_shifted(uint32_t stage, const Tab &tab, in
     const uint32_t at_c = use_se ? at(HM ? 3 : 2) : 0u;
     float *wp = ptr[1] + begin;
     float *mp = HM ? ptr[2] + begin : nullptr;
+    const Sgd sgd = sgd_of(sc);
     Dw4 aw;
     dw_zero(aw);
     // One step from element j0 on; the elements past the end count as 0.
@@ -1867,7 +1894,7 @@ __device__ __noinline__ double update_shifted(uint32_t stage, const Tab &tab, in
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             if (SW) dw_sq(aw.hi[u], aw.lo[u], in[u] ? w[u] : 0.f);
-            sgd1(g[u], c[u], w[u], m[u], sc, HM);
+            sgd1(g[u], c[u], w[u], m[u], sgd, HM);
             if (in[u]) {
                 __stcs(wp + j0 + 32 * u, w[u]);
                 if (HM) __stcs(mp + j0 + 32 * u, m[u]);
@@ -2065,7 +2092,7 @@ __global__ void __launch_bounds__(Ring2<SH>::kThreads, 1)
                     if (use_se) c_t = lds1(o + se_off);
                 }
                 if (SW) awt = __fma_rn((double)w_t, (double)w_t, awt);
-                sgd1(g_t, c_t, w_t, m_t, sc, HM);
+                sgd1(g_t, c_t, w_t, m_t, sgd_of(sc), HM);
                 wp[jj] = w_t;
                 if (HM) mp[jj] = m_t;
             }
