@@ -571,7 +571,7 @@ def run_ours(args, wl):
             one_step()
     step.set_trace_events(None)
     torch.cuda.synchronize()
-    # kernel boundaries: [0] k_reduce [1] k_combine (pass 1) [2] k_update [3] k_combine [4]
+    # kernel boundaries: [0] k_reduce [1] (LARS: k_lars) [2] k_update [3] k_finish [4]
     t_red = [e[0].elapsed_time(e[1]) for e in evs]
     t_cmb1 = [e[1].elapsed_time(e[2]) for e in evs]
     t_upd = [e[2].elapsed_time(e[3]) for e in evs]
