@@ -3034,6 +3034,7 @@ int tula_ags_update_scale(const float *const *g_small, const float *const *g_lar
     if (rc) return rc;
     const WsLayout L = ws_layout(n, pl);
     Scalars sc = make_scalars(hp, 1, n, hp->workspace, L, kModeScale);
+    sc.stats = nullptr;  // the rows of the steps that hp is also used for
     auto fill = [&](int p, const float **dst) {
         dst[0] = g_large[p];
         dst[1] = g_small[p];
