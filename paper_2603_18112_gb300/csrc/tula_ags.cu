@@ -612,6 +612,15 @@ __device__ __forceinline__ void bulk_g2s_hint(uint32_t dst, const void *src, uin
         "l"(src), "r"(bytes), "r"(smem_addr(bar)), "l"(policy)
         : "memory");
 }
+// Fetches `bytes` from src into L2: a hint, which reads nothing into the kernel.
+__device__ __forceinline__ void bulk_prefetch(const void *src, uint32_t bytes, bool hint,
+                                              uint64_t policy) {
+    if (hint)
+        asm volatile("cp.async.bulk.prefetch.L2.global.L2::cache_hint [%0], %1, %2;" ::"l"(src),
+                     "r"(bytes), "l"(policy));
+    else
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes));
+}
 // One fp32 global -> shared, asynchronously, by this lane; cp_async_wait() waits for every such
 // copy of this lane.
 __device__ __forceinline__ void cp_async4(uint32_t dst, const float *src) {
@@ -835,10 +844,12 @@ struct Stream {
         base = sc.claim_base;
         hint = sc.evict_first != 0;
         policy = policy_evict_first();
-        // cp.async reads through L1: nothing there from before this kernel.
-        if constexpr (SH) __threadfence();
         const unsigned v = (unsigned)warp * gridDim.x + blockIdx.x;
         return v < nc ? (int)v : -1;
+    }
+    // cp.async (shifted tiles' ends) reads through L1: nothing stays there from before this.
+    __device__ __forceinline__ void forget_l1() const {
+        if constexpr (SH) __threadfence();
     }
     // Claims the tile after the one just issued: after, because the warp may stop for the
     // atomic's round trip here (its tile is on its way meanwhile; claimed before the copies, it
@@ -884,6 +895,21 @@ struct Stream {
         issue_edge_tile(stage + (uint32_t)lane * part, stream ? tc.mine : nullptr, tc.aligned,
                         q.begin, (int)(q.end - q.begin), tc.numel - q.begin, arm, mine, bar, hint,
                         policy);
+    }
+    // Has L2 fetch tile c, to be issued later; of a shifted one what lies between its first and
+    // last 16-byte boundary.
+    template <typename Tab>
+    __device__ __forceinline__ void prefetch(const Tab &tab, int c, int chunk, int role, int ns) {
+        const TilePos q = tc.at(tab, c, chunk, role, ns);
+        if ((int)(threadIdx.x & 31) >= ns) return;
+        int n = (int)(q.end - q.begin);
+        const float *src = tc.mine + q.begin;
+        if constexpr (SH) {
+            const int up = (int)(-(reinterpret_cast<uintptr_t>(src) >> 2) & 3u);
+            src += up;
+            n -= up;
+        }
+        if (n >= 4) bulk_prefetch(src, 16u * (uint32_t)(n >> 2), hint, policy);
     }
     __device__ __forceinline__ void copy(const TilePos &q, int lane, int chunk) {
         const uint32_t bytes = 16u * (uint32_t)tc.nv;
@@ -1449,20 +1475,15 @@ template <int KT, bool WM, bool RW, bool SS, bool PR, bool SH, bool Small>
 __global__ void __launch_bounds__(Ring1Of<KT, RW, SH>::kThreads, 1)
     k_reduce(const __grid_constant__ TableOf<Small> tab, const __grid_constant__ Scalars sc) {
     extern __shared__ __align__(128) unsigned char smem[];
-    // The first launch of a step's pass that does not read w issues its first tiles at once: the
-    // only kernel that lets it start early is the previous call's k_finish, once all before that
-    // one had completed.  What it writes, the mean and the accumulators, waits for k_finish, which
-    // reads the accumulators.  A first launch that reads w waits whole.  The next kernel may start
-    // when that wait has passed; a later launch of the pass (more tensors than one parameter block
-    // holds) therefore finds all but its predecessor in the pass complete.  It shares no tensor
-    // with that one, and takes the other of two tile counters, so it only has to complete after it:
-    // its warps wait once their first tile is done.
+    // The first launch of a pass reads and writes nothing before its wait: the kernel ahead of it
+    // may be the caller's own, still writing the gradients, and may have let its dependents start.
+    // Until then it sets up its barriers, finds its first tiles in the table and has L2 fetch them,
+    // which puts no value into the kernel (ResNet-18, K = 4: 70.7 us a step, 71.6 without).  The
+    // next kernel may start when that wait has passed; a later launch of the pass (more tensors than
+    // one parameter block holds) therefore finds all but its predecessor in the pass complete.  It
+    // shares no tensor with that one, and takes the other of two tile counters, so it only has to
+    // complete after it: its warps wait once their first tile is done.
     const bool first = tab.seq == 0;
-    const bool early = !RW && !SS && sc.mode == kModeStep;
-    if (first && !early) {
-        grid_wait();
-        grid_launch_dependents();
-    }
     const int lane = threadIdx.x & 31;
     const int K = KT > 0 ? KT : sc.K;
     const int chunk = tab.chunk;
@@ -1473,12 +1494,14 @@ __global__ void __launch_bounds__(Ring1Of<KT, RW, SH>::kThreads, 1)
     int c = st.start(smem, tab.nc, sc.tiles + 2 * (tab.seq & 1), sc);
     TilePos q = {};
     if (RW && sc.keep_w && lane == K) st.hint = false;
-    if (c >= 0) q = st.issue(tab, c, chunk, role, ns);
-    st.claim();
-    if (first && early) {
+    if (first) {
+        if (c >= 0) st.prefetch(tab, c, chunk, role, ns);
         grid_wait();
         grid_launch_dependents();
     }
+    st.forget_l1();
+    if (c >= 0) q = st.issue(tab, c, chunk, role, ns);
+    st.claim();
     bool to_wait = !first;
     const bool step_g2 = sc.mode == kModeStep;  // |gbar|^2 also goes into |G|^2
     // The partial sums of a batch of kPend tiles are reduced across the warp together
@@ -1760,10 +1783,8 @@ __global__ void __launch_bounds__(32 * kFinWarps) k_finish(const __grid_constant
     const int n = sc.n_total;
     const bool step = sc.mode == kModeStep;
     grid_wait();
-    // After a step, the next call's reduction may start now: it only reads replicas, and claims
-    // tiles, until this kernel has completed.  (After the other calls it would find their pass's
-    // counters not re-armed yet.)
-    if (step) grid_launch_dependents();
+    // The next call's first kernel may start now; it reads and writes nothing before its own wait.
+    grid_launch_dependents();
     if (t == 0 && lane == 0) {
         const int pass = step ? 1 : 0;
         sc.tiles[pass] = sc.tiles[2 + pass] = 0u;
@@ -1973,6 +1994,7 @@ __global__ void __launch_bounds__(Ring2<SH>::kThreads, 1)
     Stream<Ring2<SH>, SH> st;
     int c = st.start(smem, tab.nc, sc.tiles + 2 * (tab.seq & 1) + 1, sc);
     TilePos q = {};
+    st.forget_l1();
     if (c >= 0) q = st.issue(tab, c, chunk, role, ns, early ? kEarlyFrom : 0);
     st.claim();
     if (early) {

@@ -1,6 +1,8 @@
 """GPU tests of what a caller may do around the calls: options set for another call, a sharded
 step that is dropped, kernels of the caller's own ahead of a step, buffers side by side."""
-import numpy as np
+import ctypes
+import subprocess
+
 import pytest
 import torch
 
@@ -46,3 +48,93 @@ def test_update_scale_leaves_the_statistics_alone(gran):
     assert torch.equal(st.stats, rows)
     changed = elem if gran == T.TULA_SCALE_PER_ELEMENT else [st.scale]
     assert all(bool((t != 1).any()) for t in changed)
+
+
+# Lets its dependents start at once, and writes its output some 300 us later: the way a GEMM with
+# programmatic dependent launch may write a weight gradient.
+_LATE_WRITER = r"""
+__global__ void late_writer(float *dst, const float *src, long long n) {
+    asm volatile("griddepcontrol.launch_dependents;");
+    unsigned long long t0, t;
+    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t0));
+    for (int i = 0; i < 100000; ++i) {
+        asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+        if (t - t0 > 300000ull) break;
+        __nanosleep(500);
+    }
+    for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < n;
+         j += (long long)gridDim.x * blockDim.x)
+        dst[j] = src[j];
+}
+extern "C" int write_late(float *dst, const float *src, long long n, void *stream) {
+    late_writer<<<64, 256, 0, (cudaStream_t)stream>>>(dst, src, n);
+    return (int)cudaGetLastError();
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def write_late(tmp_path_factory):
+    from paper_2603_18112_gb300 import build
+    d = tmp_path_factory.mktemp("late_writer")
+    (d / "late_writer.cu").write_text(_LATE_WRITER)
+    nvcc = build.nvcc_path()
+    subprocess.run([nvcc, *build.ARCH, "-shared", "-Xcompiler", "-fPIC", "-cudart", "shared",
+                    "-Xlinker", f"-rpath={build.cuda_lib_dir(nvcc)}", str(d / "late_writer.cu"),
+                    "-o", str(d / "late_writer.so")], check=True)
+    fn = ctypes.CDLL(str(d / "late_writer.so")).write_late
+    fn.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_longlong, ctypes.c_void_p]
+
+    def run(dst, src):
+        assert dst.numel() == src.numel()
+        rc = fn(dst.data_ptr(), src.data_ptr(), dst.numel(),
+                torch.cuda.current_stream().cuda_stream)
+        assert rc == 0
+    return run
+
+
+@pytest.mark.parametrize("shift", [0, 1])
+@pytest.mark.parametrize("call", ["step", "lars", "sharded", "stats", "scale", "scale_elem"])
+def test_inputs_written_by_a_kernel_that_lets_its_dependents_start(call, shift, write_late):
+    """The caller's kernel just ahead of a call allows programmatic dependent launch and writes the
+    gradients after that; the call reads what it has written, bit for bit the results of a call
+    made after everything had completed."""
+    wl = _workload(331)
+    K = 2
+    ps = _normal_pset((1, 5, 1000, 30001, 200000))
+    elem = [torch.zeros(n, device="cuda") for n in ps.numels]
+    runs = []
+    for late in (False, True):
+        buf = W.allocate(wl, "cuda", K=K, pset=ps, align=1 if shift else 64, shift=shift)
+        both = torch.zeros(2 * buf.total, device="cuda")  # every replica in one buffer
+        buf.g_flats = [both[:buf.total], both[buf.total:]]
+        buf.g = [W._views(f, buf.offsets, ps.shapes, buf.numels) for f in buf.g_flats]
+        W.fill_state(buf, wl)
+        st = T.AGSOptimizerStep(buf.w, buf.g, buf.m, lars_trust=0.01, scale_elem=elem,
+                                rule=T.TULA_RULE_LARS if call == "lars" else T.TULA_RULE_AGS)
+        share = st.new_g2_share()
+        rows = torch.zeros_like(st.stats)
+        for seed_step in (1, 2, 3):
+            W.fill_grads(buf, wl, step=seed_step)
+            src = both.clone()
+            if late:
+                both.fill_(3.0)
+            torch.cuda.synchronize()
+            if late:
+                write_late(both, src)
+            if call in ("step", "lars"):
+                st.step(wl.lr, wl.momentum, wl.weight_decay)
+            elif call == "sharded":
+                st.shard_reduce(wl.momentum, share)
+                st.shard_update(wl.lr, wl.momentum, wl.weight_decay, share)
+            elif call == "stats":
+                T.tula_layer_stats(buf.w, buf.g, rows, st.workspace)
+            else:
+                st.hp.granularity = int(call == "scale_elem")
+                T.tula_ags_update_scale(buf.g[1], buf.g[0], st.hp)
+            torch.cuda.synchronize()
+        assert st.error() == 0
+        runs.append([both, buf.w_flat, buf.m_flat, st.state, st.stats, st.scale, rows,
+                     *(t.clone() for t in elem)])
+    for a, b in zip(*runs):
+        assert torch.equal(a, b)
