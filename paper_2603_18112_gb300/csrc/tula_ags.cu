@@ -1732,11 +1732,13 @@ __device__ __forceinline__ double share_to_double(const unsigned long long *shar
 }
 
 // Pass 1 of a sharded step, after the reduction: this rank's share of |G|^2 out of the global
-// accumulator, which is re-armed.  One warp.
+// accumulator, which is re-armed, as the reduction's tile counters are: the update may never come
+// (a step dropped for its |G|^2).  One warp.
 __global__ void __launch_bounds__(32) k_share(const __grid_constant__ Scalars sc,
                                               unsigned long long *share) {
     grid_wait();
     const int lane = threadIdx.x & 31;
+    if (lane < 2) sc.tiles[2 * lane] = 0u;
     unsigned long long *const a[1] = {sc.gacc};
     unsigned long long w[1];
     acc_words<1, kGCopies>(a, true, w);

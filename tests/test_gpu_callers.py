@@ -138,3 +138,37 @@ def test_inputs_written_by_a_kernel_that_lets_its_dependents_start(call, shift, 
                      *(t.clone() for t in elem)])
     for a, b in zip(*runs):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("K", [1, 4])
+@pytest.mark.parametrize("after", ["sharded", "whole", "stats"])
+def test_a_dropped_sharded_step(K, after):
+    """Pass 1 of a sharded step whose update never comes (a step dropped for its |G|^2): a step
+    taken next on the same workspace -- in two halves or whole, over more tiles than there are
+    streaming warps -- has its mean, |G|^2, w and m as if the dropped one had not been, and
+    tula_layer_stats takes every tile (|w|^2, which the dropped step has not touched)."""
+    wl = _workload(311)
+    ps = _normal_pset((6_000_003, 7, 40000, 64))
+    runs = []
+    for dropped in (False, True):
+        buf = W.allocate(wl, "cuda", K=K, pset=ps)
+        W.fill_state(buf, wl)
+        st = T.AGSOptimizerStep(buf.w, buf.g, buf.m, grid_ctas=1, stats=False)
+        share = st.new_g2_share()
+        if dropped:
+            W.fill_grads(buf, wl, step=1)
+            st.shard_reduce(wl.momentum, share)
+        W.fill_grads(buf, wl, step=2)
+        rows = torch.zeros(ps.n_tensors, T.TULA_STATS_LEN, dtype=torch.float64, device="cuda")
+        if after == "sharded":
+            st.shard_reduce(wl.momentum, share)
+            st.shard_update(wl.lr, wl.momentum, wl.weight_decay, share)
+        elif after == "whole":
+            st.step(wl.lr, wl.momentum, wl.weight_decay)
+        else:
+            T.tula_layer_stats(buf.w, buf.g, rows, st.workspace)
+        torch.cuda.synchronize()
+        assert st.error() == 0
+        runs.append([buf.g_flats[0], buf.w_flat, buf.m_flat, st.state, rows[:, T.TULA_STAT_W_SQ]])
+    for a, b in zip(*runs):
+        assert torch.equal(a, b)
