@@ -374,8 +374,51 @@ __device__ __forceinline__ float2 dw_pair(const Dw4 &a) {
     const float2 c23 = ff_add(make_float2(a.hi[2], a.lo[2]), make_float2(a.hi[3], a.lo[3]));
     return ff_add(c01, c23);
 }
-__device__ __forceinline__ bool dw_lane_ok(float2 v) {
-    return v.x >= 0x1p-77f && v.x <= 3.0e38f;  // false for 0, tiny sums, inf and NaN
+__device__ __forceinline__ bool dw_lane_ok(float hi) {
+    return hi >= 0x1p-77f && hi <= 3.0e38f;  // false for 0, tiny sums, inf and NaN
+}
+
+// Triples: the same sum with the errors of its high parts added exactly, too, for tiles whose norms
+// hold fp64's precision (misaligned tensors).  Each error joins the middle part by TwoSum, and what
+// that rounds off is added up in the low part, so N squares err by at most about (N u)^3 of their
+// sum (cascaded summation: Ogita, Rump and Oishi, SIAM J. Sci. Comput. 26, 2005): 4 (N u)^3 with the
+// low part's own roundings, 2^-51.4 for the four chains of N <= 72 of the longest tile, where an
+// fp64 sum of a lane's 288 squares errs by up to 2^-45.  (72 random squares, the worst of 200 draws:
+// triples 2^-53, fp64 2^-50, pairs 2^-46.)  22 fp32 operations a square instead of the pairs' 13:
+// 125 us a step of packed buckets (17.3 M elements, K = 4), 118 with pairs.  Overflow and underflow
+// show as for pairs.
+struct Tw4 {
+    float hi[4], md[4], lo[4];
+};
+__device__ __forceinline__ void tw_zero(Tw4 &a) {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) a.hi[c] = a.md[c] = a.lo[c] = 0.f;
+}
+__device__ __forceinline__ void tw_sq(Tw4 &a, int c, float x) {
+    const float p = __fmul_rn(x, x);
+    const float2 t = two_sum(a.hi[c], p);
+    const float2 m = two_sum(a.md[c], t.y);
+    const float2 e = two_sum(m.x, __fmaf_rn(x, x, -p));
+    a.hi[c] = t.x;
+    a.md[c] = e.x;
+    a.lo[c] = __fadd_rn(a.lo[c], __fadd_rn(m.y, e.y));
+}
+// The four triples added in a fixed tree into the first; then as a double, with the high part for
+// dw_lane_ok.
+__device__ __forceinline__ void tw_add(Tw4 &a, int c, int d) {
+    const float2 t = two_sum(a.hi[c], a.hi[d]);
+    const float2 m = two_sum(a.md[c], a.md[d]);
+    const float2 e = two_sum(m.x, t.y);
+    a.hi[c] = t.x;
+    a.md[c] = e.x;
+    a.lo[c] = __fadd_rn(__fadd_rn(a.lo[c], a.lo[d]), __fadd_rn(m.y, e.y));
+}
+__device__ __forceinline__ double tw_total(Tw4 &a, float &high) {
+    tw_add(a, 0, 1);
+    tw_add(a, 2, 3);
+    tw_add(a, 0, 2);
+    high = a.hi[0];
+    return __dadd_rn((double)a.hi[0], __dadd_rn((double)a.md[0], (double)a.lo[0]));
 }
 
 // Exact powers of two (k within the normal range of the type).
@@ -773,9 +816,9 @@ struct TensorCache {
 // them.)  The up to three elements at each end of a tensor outside those granules, and the last
 // n % 4 elements of an aligned tensor, come by 4-byte cp.async into the same places.  Only the
 // kernels for launches with such a tensor (SH) hold this code: in the others it cost 0.4 % (ResNet-50)
-// to 5 % (1024 small layers) of a step, and they load an aligned tensor's tail directly.  Before,
-// misaligned tensors were loaded one element at a time and squared in fp64: 17.3 M elements in 128
-// tensors, K = 4, the gradients packed, took 548 us a step; now 117 us, against 101 us aligned.
+// to 5 % (1024 small layers) of a step, and they load an aligned tensor's tail directly.  17.3 M
+// elements in 128 tensors, K = 4, the gradients packed, take 125 us a step, against 101 us aligned;
+// loaded one element at a time and squared in fp64 they took 548.
 
 // A shifted tile, or the last tile of an aligned tensor of n % 4 != 0 elements: this lane's stream
 // (mine; nullptr: none) of n elements from `begin` of a tensor with `rest` elements from there on.
@@ -1055,10 +1098,9 @@ __device__ __noinline__ F3 tile_cols_scaled(uint32_t stage, int chunk, int nv, c
 
 // A tile of a tensor off a 16-byte boundary (see issue_edge_tile() for where its elements lie): lane l
 // takes elements l, l + 32, ..., U at a time, with conflict-free 4-byte loads from shared
-// memory and coalesced 4-byte stores of the mean.  The squares are float-float pairs in either
-// mode: the elements of such tensors used to be squared in fp64, and these sums keep that
-// precision (relative error ~1e-15 a lane) without GB300's slow FP64 pipe.  Returns the lane's
-// sums; out of line, so that the streaming loop of aligned tensors keeps its shape.
+// memory and coalesced 4-byte stores of the mean.  The squares are added as triples in either
+// mode, so that these norms hold fp64's precision.  Returns the lane's sums; out of line, so that
+// the streaming loop of aligned tensors keeps its shape.
 template <int KT, bool WM, bool RW, bool SS, typename Tab>
 __device__ __noinline__ D3 tile_shifted(uint32_t stage, int chunk, const Tab &tab, int t,
                                         long long begin, int n, const Scalars &sc) {
@@ -1083,15 +1125,12 @@ __device__ __noinline__ D3 tile_shifted(uint32_t stage, int chunk, const Tab &ta
     const uint32_t at_w = RW ? at(K) : 0u;
     const uint32_t at_s = SS ? at(K) : 0u;
     float *out = ptr[0] + begin;
-    // U elements per lane and step: their U independent chains hide one another's latency.
-    constexpr int U = KT >= 1 && KT <= 0 ? 8 : 4;
-    Dw4 ag[U / 4], as[U / 4], aw[U / 4];
-#pragma unroll
-    for (int g = 0; g < U / 4; ++g) {
-        dw_zero(ag[g]);
-        dw_zero(as[g]);
-        dw_zero(aw[g]);
-    }
+    // Four elements per lane and step: their independent chains hide one another's latency.
+    constexpr int U = 4;
+    Tw4 ag, as, aw;
+    tw_zero(ag);
+    tw_zero(as);
+    tw_zero(aw);
     // One step from element j0 on; the elements past the end count as 0.
     auto step = [&](int j0, auto whole) {
         constexpr bool kWhole = decltype(whole)::value;
@@ -1119,24 +1158,20 @@ __device__ __noinline__ D3 tile_shifted(uint32_t stage, int chunk, const Tab &ta
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) y[u] = RW || SS ? lds1((RW ? at_w : at_s) + o[u]) : 0.f;
-#pragma unroll
-        for (int u4 = 0; u4 < U; u4 += 4) {
-            if (kMulti<KT>) {
-                const float4 m = mean4<KT>(make_float4(s[u4], s[u4 + 1], s[u4 + 2], s[u4 + 3]), mk);
-                s[u4] = m.x;
-                s[u4 + 1] = m.y;
-                s[u4 + 2] = m.z;
-                s[u4 + 3] = m.w;
-            }
+        if (kMulti<KT>) {
+            const float4 m = mean4<KT>(make_float4(s[0], s[1], s[2], s[3]), mk);
+            s[0] = m.x;
+            s[1] = m.y;
+            s[2] = m.z;
+            s[3] = m.w;
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int g = u / 4, c = u % 4;
             if (kMulti<KT> && WM && in[u]) out[j0 + 32 * u] = s[u];
-            dw_sq(ag[g].hi[c], ag[g].lo[c], in[u] ? s[u] : 0.f);
-            if (kMulti<KT>) dw_sq(as[g].hi[c], as[g].lo[c], in[u] ? x0[u] : 0.f);
-            if (SS) dw_sq(as[g].hi[c], as[g].lo[c], in[u] ? y[u] : 0.f);
-            if (RW) dw_sq(aw[g].hi[c], aw[g].lo[c], in[u] ? y[u] : 0.f);
+            tw_sq(ag, u, in[u] ? s[u] : 0.f);
+            if (kMulti<KT>) tw_sq(as, u, in[u] ? x0[u] : 0.f);
+            if (SS) tw_sq(as, u, in[u] ? y[u] : 0.f);
+            if (RW) tw_sq(aw, u, in[u] ? y[u] : 0.f);
         }
     };
     int j = lane;
@@ -1144,15 +1179,10 @@ __device__ __noinline__ D3 tile_shifted(uint32_t stage, int chunk, const Tab &ta
     for (; j - lane + 32 * U <= n; j += 32 * U) step(j, std::true_type{});
     if (j - lane < n) step(j, std::false_type{});
     __syncwarp();
-    float2 pg = dw_pair(ag[0]), ps = dw_pair(as[0]), pw = dw_pair(aw[0]);
-    if constexpr (U == 8) {
-        pg = ff_add(pg, dw_pair(ag[1]));
-        ps = ff_add(ps, dw_pair(as[1]));
-        pw = ff_add(pw, dw_pair(aw[1]));
-    }
-    const bool bad = lane < n && !(dw_lane_ok(pg) && (!(kMulti<KT> || SS) || dw_lane_ok(ps)) &&
-                                   (!RW || dw_lane_ok(pw)));
-    D3 r = {ff_to_double(pg), ff_to_double(ps), ff_to_double(pw)};
+    float hg, hs, hw;
+    D3 r = {tw_total(ag, hg), tw_total(as, hs), tw_total(aw, hw)};
+    const bool bad = lane < n && !(dw_lane_ok(hg) && (!(kMulti<KT> || SS) || dw_lane_ok(hs)) &&
+                                   (!RW || dw_lane_ok(hw)));
     if (__any_sync(kFull, bad)) {  // as tile_cols_fp64: again, every square exact in fp64
         r = {0.0, 0.0, 0.0};
         for (int j = lane; j < n; j += 32) {
@@ -1347,8 +1377,9 @@ __device__ __forceinline__ void reduce_tile(uint32_t stage, int chunk, const Row
     if (PR) {
         // The warp is converged again here (the loops above end in every lane).
         const float2 pg = dw_pair(ag), ps = dw_pair(as), pw = dw_pair(aw);
-        const bool bad = lane < ncols && !(dw_lane_ok(pg) && (!(kMulti<KT> || SS) || dw_lane_ok(ps)) &&
-                                           (!RW || dw_lane_ok(pw)));
+        const bool bad = lane < ncols && !(dw_lane_ok(pg.x) &&
+                                           (!(kMulti<KT> || SS) || dw_lane_ok(ps.x)) &&
+                                           (!RW || dw_lane_ok(pw.x)));
         double cg, cs, cw;
         if (__any_sync(kFull, bad)) {
             const D3 f = tile_cols_fp64<KT, RW, SS>(stage, chunk, ncols, sc);
@@ -1882,7 +1913,7 @@ __device__ __noinline__ float w_cols_scaled(uint32_t w_stage, int nv, float f) {
 }
 
 // A tile of a tensor off a 16-byte boundary, as tile_shifted() of pass 1: four elements per lane
-// and step.  Returns the lane's |w|^2 (float-float pairs, to fp64 once) when the statistics want it.
+// and step.  Returns the lane's |w|^2 (triples, to fp64 once) when the statistics want it.
 template <bool HM, bool PE, bool SW, typename Tab>
 __device__ __noinline__ double update_shifted(uint32_t stage, const Tab &tab, int t, long long begin, int n, float ct, bool use_se,
                                               const Scalars &sc) {
@@ -1898,8 +1929,8 @@ __device__ __noinline__ double update_shifted(uint32_t stage, const Tab &tab, in
     float *wp = ptr[1] + begin;
     float *mp = HM ? ptr[2] + begin : nullptr;
     const Sgd sgd = sgd_of(sc);
-    Dw4 aw;
-    dw_zero(aw);
+    Tw4 aw;
+    tw_zero(aw);
     // One step from element j0 on; the elements past the end count as 0.
     auto step = [&](int j0, auto whole) {
         constexpr bool kWhole = decltype(whole)::value;
@@ -1916,7 +1947,7 @@ __device__ __noinline__ double update_shifted(uint32_t stage, const Tab &tab, in
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            if (SW) dw_sq(aw.hi[u], aw.lo[u], in[u] ? w[u] : 0.f);
+            if (SW) tw_sq(aw, u, in[u] ? w[u] : 0.f);
             sgd1(g[u], c[u], w[u], m[u], sgd, HM);
             if (in[u]) {
                 __stcs(wp + j0 + 32 * u, w[u]);
@@ -1930,9 +1961,9 @@ __device__ __noinline__ double update_shifted(uint32_t stage, const Tab &tab, in
     if (j0 - lane < n) step(j0, std::false_type{});
     __syncwarp();
     if (!SW) return 0.0;
-    const float2 pw = dw_pair(aw);
-    double r = ff_to_double(pw);
-    if (__any_sync(kFull, lane < n && !dw_lane_ok(pw))) {
+    float high;
+    double r = tw_total(aw, high);
+    if (__any_sync(kFull, lane < n && !dw_lane_ok(high))) {
         r = 0.0;
         for (int j = lane; j < n; j += 32) {
             const double y = (double)lds1(at_w + 4u * (uint32_t)j);

@@ -518,8 +518,8 @@ def test_default_steps_over_the_whole_float_range():
 
 @pytest.mark.parametrize("K", [1, 4])
 def test_default_steps_misaligned_over_the_whole_float_range(K):
-    """The same range on misaligned tensors, where every element is loaded one by one (fp64
-    squares), and with K = 1 and 4 (other tile sizes and stream counts)."""
+    """The same range on misaligned tensors, whose squares are added as triples (in fp64 where those
+    cannot hold them), and with K = 1 and 4 (other tile sizes and stream counts)."""
     ps = _extreme_pset((1, K if K > 1 else 1))
     wl = _extreme_workload(121 + K, ps)
     for shift in (0, 1):
@@ -814,9 +814,9 @@ def test_branch_at_the_rounding_boundary_of_delta(delta):
 def test_streams_at_different_alignments(K, rule, gran, monkeypatch):
     """Tensors packed back to back, every role starting at its own offset within 16 bytes (the
     weights, the momentum and each replica at others), with sizes around a granule, a row of lanes
-    and a tile: the mean bitwise, everything else as the oracle.  Such tiles keep float-float sums:
-    norms are within 75 * 2^-46 = 1.1e-12 of the oracle's (a lane and component adds at most
-    9216 / 128 = 72 squares and the two tree steps after them, below 2^-46 each)."""
+    and a tile: the mean bitwise, everything else as the oracle.  Such tiles keep triples: norms are
+    within 2^-50 of the exact ones (test_norms_of_misaligned_tensors_hold_fp64), the oracle's
+    within 2^-52."""
     sizes = [1, 2, 3, 4, 5, 6, 7, 8, 9, 31, 33, 127, 128, 129, 131, 1021]
     for t in (T.tula_ags_chunk_elems(1, K), T.tula_ags_chunk_elems(2, 3),
               T.tula_ags_chunk_elems(3, K + 1)):
@@ -853,7 +853,7 @@ def test_streams_at_different_alignments(K, rule, gran, monkeypatch):
     assert moved.sum() > pair.n // 2
     assert_stats_close(got, ref, "layer_stats")
     for col in (T.TULA_STAT_W_SQ, T.TULA_STAT_G_SQ, T.TULA_STAT_G0_SQ):
-        assert_norm_close(got[moved, col], ref[moved, col], f"col {col}", rtol=75 * 2.0 ** -46)
+        assert_norm_close(got[moved, col], ref[moved, col], f"col {col}", rtol=1.25 * 2.0 ** -50)
     assert pair.gpu.error() == 0
 
 
@@ -920,3 +920,54 @@ def test_tensors_farther_apart_than_a_32_bit_offset(K, monkeypatch):
         pair.step(1, 1.0)
         pair.step(1, 1.0)
         assert pair.flags == [0, 1]
+
+
+@pytest.mark.parametrize("K", [1, 4])
+def test_norms_of_misaligned_tensors_hold_fp64(K):
+    """Squared norms of tensors off a 16-byte boundary against the exact sums of exact squares.
+    Of every 128 elements one is large, so that a single lane's running sum of up to 72 squares
+    makes the norm.  Its bound: the triple adds N <= 72 squares within 4 (72 * 2^-24)^3 = 2^-51.4
+    and is rounded to fp64 twice, the accumulators round once and so does the reference: below
+    2^-50.  A step that refreshes the gradscale adds the lanes in an fp64 tree of five more
+    roundings: below 2^-49."""
+    rng = np.random.default_rng(241 + K)
+    tile = T.tula_ags_chunk_elems(1, K)
+    sizes = [tile, 3 * tile + 8, 4000, 776] * 3  # every one at the same place within 16 bytes
+    ps = W.ParamSet("sparse")
+    for n in sizes:
+        ps.add((n,), W.KIND_NORMAL)
+    wl = W.workload("stress_k4", seed=241, zero_patterns=False)
+    buf = W.allocate(wl, "cuda", K=K, align=1, shift=1, pset=ps)
+
+    def fill(views, p):
+        for t in views:
+            x = rng.uniform(1e-6, 2e-6, t.numel())
+            x[p::128] = rng.uniform(0.5, 2.0, x[p::128].size)
+            t.copy_(torch.from_numpy(x.astype(np.float32)))
+
+    for p in range(ps.n_tensors):
+        fill([buf.w[p], *(g[p] for g in buf.g)], p)
+
+    def square(x):
+        return math.fsum((x.astype(np.float64) ** 2).tolist())
+
+    g_h = [W.to_numpy(g) for g in buf.g]
+    mean = [O.replica_mean([g_h[k][p] for k in range(K)]) for p in range(ps.n_tensors)]
+    ref = np.zeros((ps.n_tensors, 3))
+    ref[:, T.TULA_STAT_W_SQ] = [square(x) for x in W.to_numpy(buf.w)]
+    ref[:, T.TULA_STAT_G_SQ] = [square(x) for x in mean]
+    ref[:, T.TULA_STAT_G0_SQ] = [square(x) for x in g_h[0]]
+    snap = _inputs_snapshot(buf)
+    step = T.AGSOptimizerStep(buf.w, buf.g, buf.m)
+    rows = torch.zeros_like(step.stats)
+    T.tula_layer_stats(buf.w, buf.g, rows, step.workspace)
+    got = {"layer_stats": (rows.cpu().numpy(), 2.0 ** -50)}
+    for refresh in (False, True)[:min(K, 2)]:
+        _restore(buf, snap)
+        step.step(0.1, 0.9, 0.0, refresh_scale=refresh)
+        rtol = 2.0 ** -(49 if refresh else 50)
+        got[f"step, refresh {refresh}"] = (step.stats.cpu().numpy(), rtol)
+        assert_norm_close(step.state[0].item(), math.fsum(ref[:, T.TULA_STAT_G_SQ]), "|G|^2", rtol)
+    for what, (stats, rtol) in got.items():
+        for col in (T.TULA_STAT_W_SQ, T.TULA_STAT_G_SQ, T.TULA_STAT_G0_SQ):
+            assert_norm_close(stats[:, col], ref[:, col], f"{what} col {col}", rtol=rtol)
