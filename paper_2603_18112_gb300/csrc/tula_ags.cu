@@ -890,7 +890,9 @@ struct Stream {
         const unsigned v = (unsigned)warp * gridDim.x + blockIdx.x;
         return v < nc ? (int)v : -1;
     }
-    // cp.async (shifted tiles' ends) reads through L1: nothing stays there from before this.
+    // cp.async (the ends of shifted tiles) reads through L1, 32 bytes at a time, which bring the
+    // neighbouring elements along: whatever L1 holds from before a wait is given up by a fence after
+    // it, before elements that another kernel has written meanwhile are read this way.
     __device__ __forceinline__ void forget_l1() const {
         if constexpr (SH) __threadfence();
     }
@@ -2033,6 +2035,7 @@ __global__ void __launch_bounds__(Ring2<SH>::kThreads, 1)
     if (early) {
         grid_wait();
         grid_launch_dependents();
+        st.forget_l1();  // a role's first tiles may share a sector with the mean's
         if (c >= 0) st.issue_below(q, kEarlyFrom, ns, chunk);
         rearm_pass1();
         scaled = take_branch();

@@ -172,3 +172,44 @@ def test_a_dropped_sharded_step(K, after):
         runs.append([buf.g_flats[0], buf.w_flat, buf.m_flat, st.state, rows[:, T.TULA_STAT_W_SQ]])
     for a, b in zip(*runs):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("roles", ["wgm", "mgw", "gwm"])
+def test_roles_side_by_side_in_one_buffer(roles):
+    """The weights, the gradients and the momentum of each tensor back to back in one buffer, none
+    at a 16-byte boundary: the update copies ends of w and m, with whatever shares their 32 bytes,
+    while the reduction still writes the mean.  Element by element the results are those of aligned
+    buffers, bit for bit."""
+    K = 2
+    sizes = [1, 2, 3, 5, 6, 7, 9, 11, 13, 127, 2049, 4099, 9217, 20001] * 8
+    ps = _normal_pset(sizes)
+    wl = _workload(351)
+    plain = W.allocate(wl, "cuda", K=K, pset=ps)
+    W.fill_state(plain, wl)
+    flat = torch.zeros(1 + 4 * sum(sizes), device="cuda")
+    views = {"w": [], "g": [[], []], "m": []}
+    at = 1
+    for n in sizes:
+        for role in roles:
+            for out in views["g"] if role == "g" else [views[role]]:
+                out.append(flat[at:at + n])
+                at += n
+    assert at == flat.numel()
+    for a, b in zip(plain.w, views["w"]):
+        b.copy_(a)
+    kw = dict(force_branch=T.TULA_BRANCH_SCALED, scale=torch.linspace(0.5, 2.0, len(sizes),
+                                                                      device="cuda"))
+    steps = [T.AGSOptimizerStep(plain.w, plain.g, plain.m, **kw),
+             T.AGSOptimizerStep(views["w"], views["g"], views["m"], **kw)]
+    for i in range(4):
+        W.fill_grads(plain, wl, step=i)
+        for a, b in zip(plain.g, views["g"]):
+            for x, y in zip(a, b):
+                y.copy_(x)
+        for st in steps:
+            st.step(wl.lr, wl.momentum, wl.weight_decay)
+        torch.cuda.synchronize()
+        assert all(st.error() == 0 for st in steps)
+        for a, b in ((plain.w, views["w"]), (plain.m, views["m"]), (plain.g[0], views["g"][0])):
+            for x, y in zip(a, b):
+                assert torch.equal(x, y)
