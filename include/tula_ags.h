@@ -170,7 +170,8 @@ int tula_ags_workspace_size(const int64_t *numels, int n_tensors, int K, size_t 
  *   numels[p] >= 0         element counts (0 = skipped); all tensors together may span
  *                          fewer than 2^31 tiles of min(tula_ags_chunk_elems(1, K + 1),
  *                          tula_ags_chunk_elems(2, 4)) elements (K + 2 in place of K + 1
- *                          when K = 1; an empty tensor counts as one tile): about 3.3e12
+ *                          when K = 1; an empty tensor counts as one tile), and tiles and
+ *                          tensors of numels[p] % 4 != 0 together at most 2^31: about 3.3e12
  *                          elements for K <= 4, 1.9e12 at K = 8, 8.2e11 at K = 16, more
  *                          than any GB300 holds; a longer list gives TULA_ERR_ARG
  * Per element, with c the coefficient of the rule (Algorithm 1, Eq. 8):
@@ -228,7 +229,7 @@ int tula_ags_plan_destroy(tula_ags_plan *plan);
  * partials, word 22 the number of NaN partials, word 23 zero.  Integer addition has no order, so
  * every rank takes the same |G|^2, Delta and branch, equal bit for bit to those of one
  * tula_ags_step over all tensors (tiles are cut per tensor, so each tensor's norms are the same
- * wherever it lives); the ranks together may span fewer than 2^31 pass-1 tiles.
+ * wherever it lives); the limits on tiles and tensors hold for the ranks together.
  * Arguments as tula_ags_step, with the rank's tensors; hp (workspace sized for the rank's
  * tensors, state, scale, layer_stats) must be the same in both calls, and no other call may use
  * the workspace between them.  g2_share, g2_total: device uint64 [TULA_G2_SHARE_WORDS], 8-byte

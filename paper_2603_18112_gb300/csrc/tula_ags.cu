@@ -472,14 +472,17 @@ __device__ __forceinline__ float4 mul4(float4 v, float f) {
 // Range: the partials are fp32 tile sums scaled by 2^k (k in {0, -200, 144}, sq_range_exp) or
 // fp64 sums of exact squares of fp32 numbers, so their bits lie within 2^-352 .. 2^273; a tensor
 // of up to 2^31 tiles, or all tensors together, stays below 2^305; 21 digits from 2^-352 cover
-// 2^-352 .. 2^320.  Each word takes at most two adds (< 2^32 each) per tile, so its high half
-// cannot overflow for fewer than 2^31 tiles.  A partial that is inf or NaN (an inf or NaN
-// element) sets a flag in the last word instead: the norm is then inf, or NaN.
+// 2^-352 .. 2^320.  To one word a tile adds less than 2 * 2^32: one partial adds to a word once,
+// less than 2^32, and the three limbs of a shifted tile's sum together no more than two such adds
+// (limbs_max_add).  Only the last tile of a tensor of n % 4 != 0 elements may add up to 4 * 2^32,
+// its fp32 sum and the squares of up to three tail elements.  A word therefore stays below 2^64
+// while tiles and such tensors together number at most 2^31 (valid_numels).  A partial that is inf
+// or NaN (an inf or NaN element) sets a flag in the last word instead: the norm is then inf, or NaN.
 //
 // Copies: the tiles of one tensor land close together in time, and every tile of a step adds
 // into |G|^2, so one word would take an atomic every few ns, about what an L2 slice can do for
 // one address.  Each accumulator therefore has copies, picked by the CTA, that the reading warp
-// adds up (exact; all copies together still take fewer than 2^32 adds per word).
+// adds up (exact: the bound on a word holds for all copies together).
 constexpr int kAccDigits = 21;
 constexpr int kAccWords = 24;             // digits, two spare words, the flags
 constexpr int kAccFlags = kAccWords - 1;  // bit 0: an inf partial, bit 1: a NaN partial
@@ -1455,6 +1458,24 @@ __device__ __forceinline__ void add_tail(const Scalars &sc, int tg, const double
         if (a == 0 && sc.mode == kModeStep) acc_add_f64(gacc_of(sc), d);
     }
 }
+// The most that the limbs of add_shifted, at bits r, r + 26 and r + 52 of a word, add to any one
+// word between them.
+constexpr unsigned long long limbs_max_add() {
+    unsigned long long most = 0;
+    for (int r = 0; r < 32; ++r) {
+        unsigned long long word[5] = {};
+        for (int i = 0; i < 3; ++i) {
+            const unsigned long long limb = 32ull * ((i == 2 ? 1ull << 27 : 1ull << 26) - 1ull);
+            const int at = r + 26 * i, w = at >> 5, b = at & 31;
+            const unsigned long long low = limb << b, top = (1ull << 32) - (1ull << b);
+            word[w] += low < top ? low : top;
+            word[w + 1] += low >> 32;
+        }
+        for (unsigned long long x : word) most = x > most ? x : most;
+    }
+    return most;
+}
+static_assert(limbs_max_add() <= 2ull << 32, "a shifted tile adds to a word as two partials do");
 // The lanes' fp64 sums d[0 .. R) (>= 0, finite or not) of a shifted tile into R accumulators, and
 // the first one into `also` as well (unless NULL).  An fp64 tree across the warp took 4000 cycles of
 // a tile's 13,000 on GB300's slow FP64 pipe, so the lanes are added as integers: relative to the
@@ -2344,17 +2365,20 @@ WsLayout ws_layout(int n_tensors, const Plan &) {
     return L;
 }
 
-// The tile index of either pass must fit an int, which also keeps every accumulator word's
-// carries within its high half (at most two adds below 2^32 per tile).
+// The tile index of either pass must fit an int; and the tiles and the tensors of n % 4 != 0
+// elements together number at most 2^31, which keeps every accumulator word below 2^64.
 bool valid_numels(const int64_t *numels, int n, int K, Plan *pl) {
     if (!numels || n < 1 || K < 1 || K > TULA_MAX_K) return false;
     const int t1 = chunk1_min(K), t2 = chunk2_min();
     Plan p;
+    long long tails = 0;
     for (int i = 0; i < n; ++i) {
         if (numels[i] < 0) return false;
         p.c1 += tiles_of(numels[i], t1);
         p.c2 += tiles_of(numels[i], t2);
+        tails += (numels[i] & 3) != 0;
         if (p.c1 >= (1LL << 31) || p.c2 >= (1LL << 31)) return false;
+        if (std::max(p.c1, p.c2) + tails > (1LL << 31)) return false;
     }
     *pl = p;
     return true;

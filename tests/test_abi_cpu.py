@@ -101,6 +101,20 @@ def test_size_limit(lib, K):
         assert e.value.code == T.TULA_ERR_ARG
 
 
+@pytest.mark.parametrize("K", [1, 4, 16])
+def test_size_limit_with_tails(lib, K):
+    """The squares of a tensor's last n % 4 elements are added one by one, up to two more adds to
+    a word of its accumulators: tiles and such tensors together may number at most 2^31."""
+    tile = min(T.tula_ags_chunk_elems(1, K + 2 if K == 1 else K + 1), T.tula_ags_chunk_elems(2, 4))
+    limit, half = (2 ** 31 - 1) * tile, 2 ** 30 * tile
+    for numels in ([limit - 1], [half - 1, limit - half], [half - tile - 1, limit - half - 3]):
+        assert T.tula_ags_workspace_size(numels, K) > 0
+    for numels in ([half - 1, limit - half - 3], [half, 1, 2, limit - half - 2 * tile]):
+        with pytest.raises(T.TulaError) as e:
+            T.tula_ags_workspace_size(numels, K)
+        assert e.value.code == T.TULA_ERR_ARG
+
+
 def _call_step(lib, n=2, K=1, params=None, grads=None, moms=None, numels=None, hp=None,
                momentum=0.9):
     P = ctypes.c_void_p
