@@ -98,18 +98,60 @@ def test_rules(rule, gran, mom):
 
 @pytest.mark.parametrize("rule", [T.TULA_RULE_AGS, T.TULA_RULE_LARS])
 def test_many_tensors_span_several_launches(rule):
-    """1000 tensors with K = 16 need several parameter blocks per pass (LARS: pass 1 reading w,
-    through its own ring and tile size)."""
+    """1800 tensors with K = 16 need several parameter blocks per pass (LARS: pass 1 reading w,
+    through its own ring and tile size): 446 (421) of them fill a block of the reduction, 1734 one
+    of the update."""
     rng = np.random.default_rng(5)
     ps = W.ParamSet("many")
-    for n in rng.integers(1, 5000, size=1000):
+    for n in rng.integers(1, 5000, size=1800):
         ps.add((int(n),), W.KIND_NORMAL)
     wl = W.workload("stress_k16", seed=31)
     pair = Pair(wl, pset=ps, rule=rule, lars_trust=0.01)
     before = T.tula_ags_launch_count()
     for i, mult in enumerate((1.0, 1.0)):
         pair.step(i + 1, mult, refresh=(i == 0))
-    assert T.tula_ags_launch_count() - before >= 2 * 2 * 2
+    lars = rule == T.TULA_RULE_LARS
+    assert T.tula_ags_launch_count() - before == 2 * (5 + 2 + 1 + lars)
+
+
+@pytest.mark.parametrize("grid", [0, 2])
+@pytest.mark.parametrize("layout", ["aligned", "packed", "mixed"])
+@pytest.mark.parametrize("rule,gran,mom,n,blocks", [
+    (T.TULA_RULE_AGS, T.TULA_SCALE_PER_TENSOR, True, 5300, (3, 4)),
+    (T.TULA_RULE_AGS, T.TULA_SCALE_PER_TENSOR, False, 5300, (3, 3)),
+    (T.TULA_RULE_AGS, T.TULA_SCALE_PER_ELEMENT, True, 4300, (2, 4)),
+    (T.TULA_RULE_LARS, T.TULA_SCALE_PER_TENSOR, True, 5300, (4, 4)),
+])
+def test_later_launches_of_a_pass(rule, gran, mom, n, blocks, layout, grid):
+    """Two to four launches of each pass, which overlap, take two tile counters in turn and start
+    claiming where the one before the last stopped (a grid of 2 leaves every launch more tiles than
+    warps).  packed: every tensor off a 16-byte boundary; mixed: the first block's tensors aligned,
+    the others not.  The launches of each pass are counted through the two halves of a sharded
+    step."""
+    rng = np.random.default_rng(251)
+    ps = W.ParamSet("later")
+    for i, size in enumerate(rng.integers(1, 41, size=n)):
+        size = int(size) if i % 64 else 3001
+        ps.add((4 * size if layout == "mixed" and i < 2300 else size,), W.KIND_NORMAL)
+    wl = W.workload("stress_k4", seed=251, factor_range=(1e-3, 1e1), zero_patterns=False)
+    pair = Pair(wl, K=2, pset=ps, rule=rule, granularity=gran, with_momentum=mom, lars_trust=0.01,
+                align=64 if layout == "aligned" else 1, shift=1 if layout == "packed" else 0,
+                grid_ctas=grid)
+    odd = [any(t.data_ptr() % 16 for t in (pair.buf.w[p], pair.buf.g[0][p], pair.buf.g[1][p]))
+           for p in range(n)]
+    assert sum(odd) > n // 4 if layout != "aligned" else not any(odd)
+    assert not any(odd[:2300]) if layout == "mixed" else True
+    for seed_step, mult in ((1, 1.0), (1, 1.0)):
+        pair.step(seed_step, mult)
+    assert pair.flags == [0, 1]
+    assert pair.gpu.error() == 0
+    counts, share = [T.tula_ags_launch_count()], pair.gpu.new_g2_share()
+    pair.gpu.shard_reduce(pair.momentum, share)
+    counts.append(T.tula_ags_launch_count())
+    pair.gpu.shard_update(wl.lr, pair.momentum, wl.weight_decay, share)
+    counts.append(T.tula_ags_launch_count())
+    lars = rule == T.TULA_RULE_LARS
+    assert [counts[1] - counts[0] - 1, counts[2] - counts[1] - 1 - lars] == list(blocks)
 
 
 def test_zero_gradients_and_weights():
@@ -177,19 +219,34 @@ def test_layer_stats(K):
         assert torch.equal(a, b)  # read-only
 
 
+@pytest.mark.parametrize("layout", ["aligned", "packed", "apart", "many"])
 @pytest.mark.parametrize("gran", [T.TULA_SCALE_PER_TENSOR, T.TULA_SCALE_PER_ELEMENT])
-def test_update_scale(gran):
+def test_update_scale(gran, layout):
+    """UpdateGradScale against the oracle.  packed: tensors back to back, every role at the same
+    place within 16 bytes; apart: each role at its own; many: more tensors than a launch holds."""
     wl = W.workload("resnet20", seed=61)
-    buf = W.allocate(wl, "cuda", K=2, pset=_ragged_pset(extra=(7, 300001)))
+    ps = _ragged_pset(extra=(7, 300001), K=1)
+    if layout == "many":
+        for i in range(4000):
+            ps.add((1 + i % 37,), W.KIND_NORMAL)
+    align = 64 if layout == "aligned" else 1
+    buf = W.allocate(wl, "cuda", K=2, pset=ps, align=align, shift=int(layout != "aligned"))
     W.fill_grads(buf, wl, step=1)
-    gs, gl = buf.g[0], buf.g[1]
+
+    def moved(flat, shift):
+        out = torch.zeros(flat.numel() + 8, device="cuda")[shift:shift + flat.numel()]
+        return W._views(out.copy_(flat), buf.offsets, ps.shapes, buf.numels)
+
+    shifts = (1, 2, 3) if layout == "apart" else (0, 0, 0)
+    gs, gl = moved(buf.g_flats[0], shifts[0]), moved(buf.g_flats[1], shifts[1])
+    se = moved(torch.zeros_like(buf.g_flats[0]), shifts[2])
+    assert any(t.data_ptr() % 16 for t in gs) == (layout != "aligned")
     hp = T.tula_ags_default_hparams(4)
     hp.granularity = gran
     n = buf.pset.n_tensors
     scale = torch.zeros(n, dtype=torch.float32, device="cuda")
     ws = T.new_workspace(buf.numels, 1)
     hp.scale, hp.workspace, hp.workspace_bytes = scale.data_ptr(), ws.data_ptr(), ws.numel()
-    se = [torch.zeros_like(t) for t in gs]
     keep = None
     if gran == T.TULA_SCALE_PER_ELEMENT:
         keep = T._tensor_ptrs(se)
@@ -453,12 +510,14 @@ def test_lars_steps_over_the_whole_float_range():
     pair.step(2, 1.0)
 
 
-def test_update_scale_over_the_whole_float_range():
+@pytest.mark.parametrize("shift", [0, 1])
+def test_update_scale_over_the_whole_float_range(shift):
     """UpdateGradScale per tensor (precise norms of g_small and g_large) over the same range,
-    with s_max out of the way: each scale within 2 ulp of the oracle's fp64 ratio."""
+    with s_max out of the way: each scale within 2 ulp of the oracle's fp64 ratio, on aligned and
+    on misaligned tensors."""
     ps = _extreme_pset((1, 2))
     wl = _extreme_workload(105, ps)
-    buf = W.allocate(wl, "cuda", K=2, pset=ps)
+    buf = W.allocate(wl, "cuda", K=2, pset=ps, align=1 if shift else 64, shift=shift)
     W.fill_grads(buf, wl, step=1)
     gs, gl = buf.g[1], buf.g[0]
     n = buf.pset.n_tensors
@@ -632,20 +691,23 @@ def test_checkpoint_and_resume_through_the_host():
 
 
 @pytest.mark.parametrize("name,rule", [("resnet50", T.TULA_RULE_AGS), ("resnet18", T.TULA_RULE_LARS),
-                                       ("ragged_k4", T.TULA_RULE_AGS)])
+                                       ("ragged_k4", T.TULA_RULE_AGS), ("packed_k4", T.TULA_RULE_AGS),
+                                       ("packed_k4", T.TULA_RULE_LARS)])
 def test_sharded_step_equals_the_whole_step(name, rule):
     """A step sharded over two ranks (each owning whole tensors) run on one GPU, one shard after
     the other: each rank's pass 1 exports its share of |G|^2, the shares are summed as integers,
     and each rank finishes from the sum.  Tiles are cut per tensor and the sums are exact, so the
     mean, every norm, |G|^2, Delta, the branch, w, m and the gradscale equal those of one step
     over all tensors bit for bit -- whichever order the shares are added in."""
-    if name == "ragged_k4":
+    packed = name == "packed_k4"  # tensors back to back, off 16-byte boundaries
+    if packed or name == "ragged_k4":
         wl = W.workload("stress_k4", seed=161, factor_range=(0.1, 10.0), zero_patterns=False)
         ps = _ragged_pset(K=4)
     else:
         wl, ps = W.workload(name), None
     K = 4 if ps is not None else wl.K
-    a, b = (W.allocate(wl, "cuda", K=K, pset=ps) for _ in range(2))
+    a, b = (W.allocate(wl, "cuda", K=K, pset=ps, align=1 if packed else 64, shift=int(packed))
+            for _ in range(2))
     for buf in (a, b):
         W.fill_state(buf, wl)
     n = a.pset.n_tensors
@@ -687,7 +749,7 @@ def test_plan_steps_equal_direct_steps(case):
     if case == "many_k2":
         rng = np.random.default_rng(171)
         ps = W.ParamSet("many")
-        for n in rng.integers(1, 3000, size=800):   # several parameter blocks per pass
+        for n in rng.integers(1, 600, size=5300):   # 3 parameter blocks of pass 1, 4 of the update
             ps.add((int(n),), W.KIND_NORMAL)
         K = 2
     else:
