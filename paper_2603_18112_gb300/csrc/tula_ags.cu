@@ -184,10 +184,10 @@ using TableOf = Table<Small ? 8 * 1024 : kParamBudget>;
 static_assert(sizeof(TableOf<true>) == 8 * 1024 && sizeof(TableOf<false>) == kParamBudget, "as sized");
 
 struct Scalars {
-    int K, rule, gran, force, refresh, mode, n_total, read_w;
-    int pow2K, evict_first, early_w, keep_w;  // evict_first: TMA loads ask L2 to drop their lines
-                                              // first, keep_w: but not pass 1's of w; early_w: the
-                                              // update follows this call's pass 1
+    int K, rule, force, refresh, mode, n_total, read_w;
+    int evict_first, early_w, keep_w;  // evict_first: TMA loads ask L2 to drop their lines first,
+                                       // keep_w: but not pass 1's of w; early_w: the update
+                                       // follows this call's pass 1
     float delta, eps, s_max, static_s, lars_trust, lr, mu, wd, invK, Kf;
     float *scale;
     double *state;
@@ -244,19 +244,13 @@ __device__ __forceinline__ float4 add4(float4 a, float4 b) {
 // Eq. 1c: divide the k-ascending sum by K (exact reciprocal when K is a power of 2).  K by value,
 // for the same reason as Sgd.
 struct MeanK {
-    int pow2K;
     float invK, Kf;
 };
-__device__ __forceinline__ MeanK mean_k(const Scalars &sc) { return {sc.pow2K, sc.invK, sc.Kf}; }
+__device__ __forceinline__ MeanK mean_k(const Scalars &sc) { return {sc.invK, sc.Kf}; }
 template <int KT>
 __device__ __forceinline__ float mean1(float s, const MeanK &sc) {
-    if constexpr (KT > 0 && (KT & (KT - 1)) == 0) {
-        return __fmul_rn(s, 1.0f / (float)KT);
-    } else if constexpr (KT > 0) {
-        return __fdiv_rn(s, (float)KT);
-    } else {
-        return sc.pow2K ? __fmul_rn(s, sc.invK) : __fdiv_rn(s, sc.Kf);
-    }
+    static_assert((KT & (KT - 1)) == 0, "a power of two, or 0: known at run time");
+    return KT > 0 ? __fmul_rn(s, 1.0f / (float)(KT > 0 ? KT : 1)) : __fdiv_rn(s, sc.Kf);
 }
 // s / K for a K known only at run time, correctly rounded (Markstein, IBM J. Res. Dev. 34, 1990):
 // with y = fl(1 / K) and q = fl(s y), the remainder r = s - K q is exact in one fused operation and
@@ -274,7 +268,7 @@ __device__ __forceinline__ float mean_fast(float s, const MeanK &sc) {
 template <int KT>
 __device__ __forceinline__ float4 mean4(float4 s, const MeanK &sc) {
     if (KT == 0 && mean_in_range(s.x) && mean_in_range(s.y) && mean_in_range(s.z) &&
-        mean_in_range(s.w))  // (K a power of two as well: its remainders are 0)
+        mean_in_range(s.w))
         return make_float4(mean_fast(s.x, sc), mean_fast(s.y, sc), mean_fast(s.z, sc),
                            mean_fast(s.w, sc));
     return make_float4(mean1<KT>(s.x, sc), mean1<KT>(s.y, sc), mean1<KT>(s.z, sc),
@@ -1018,7 +1012,7 @@ constexpr bool kMulti = KT != 1;
 // One float4 column of a tile: mean, squares.  x0 = replica 0, s = sum.
 template <int KT, bool WM, bool RW, bool SS, bool PR>
 __device__ __forceinline__ void column1(float4 x0, float4 s, float4 wv, float4 sv, float *out,
-                                        const Scalars &sc, int K, Dw4 &ag, Dw4 &as, Dw4 &aw,
+                                        const Scalars &sc, Dw4 &ag, Dw4 &as, Dw4 &aw,
                                         float &pg, float &ps, float &pw) {
     if (kMulti<KT>) {
         s = mean4<KT>(s, mean_k(sc));
@@ -1214,13 +1208,13 @@ __device__ __noinline__ D3 tile_shifted(uint32_t stage, int chunk, const Tab &ta
 
 // Per-lane partial sums of one tile (not yet reduced across the warp).  Precise mode (PR):
 // accd holds the lane's fp64 sums.  Default mode: accf holds the lane's fp32 sums over the
-// tile's float4 columns, scaled by 2^(2 acce) (acce is the same in every lane), and accd the
-// lane's fp64 sums over the elements taken one by one (tail, shifted tile).
+// tile's float4 columns, scaled by 2^(2 e) with e coded in `ecode` (the same in every lane), accd
+// the lane's fp64 sums over the elements taken one by one (tail, shifted tile).
 template <int KT, bool WM, bool RW, bool SS, bool PR, bool SH, typename Tab>
 __device__ __forceinline__ void reduce_tile(uint32_t stage, int chunk, const Row<Tab> ptr,
                                             float *out0, const TilePos &q, int nv, bool aligned,
                                             const Scalars &sc, double (&accd)[kAcc], float (&accf)[kAcc],
-                                            int (&acce)[kAcc], unsigned &ecode, bool &tail) {
+                                            unsigned &ecode, bool &tail) {
     const int lane = threadIdx.x & 31;
     const int K = KT > 0 ? KT : sc.K;
     const uint32_t sw_s = stage + (uint32_t)(K * chunk * 4);
@@ -1233,7 +1227,7 @@ __device__ __forceinline__ void reduce_tile(uint32_t stage, int chunk, const Row
     double rg = 0.0, rs = 0.0, rw = 0.0;  // exact fp64 sums of the tail
     const int ncols = nv;                 // the float4 columns (nv is reused below)
     tail = false;                         // the tile has elements taken one by one
-    ecode = 0u;                           // scale_code of acce[a] in bits 2a, 2a + 1
+    ecode = 0u;                           // scale_code of sum a's exponent in bits 2a, 2a + 1
     if (SH && !aligned) {
         const D3 d = tile_shifted<KT, WM, RW, SS>(stage, chunk, ptr.tab, ptr.t, q.begin,
                                                          (int)(q.end - q.begin), sc);
@@ -1241,7 +1235,6 @@ __device__ __forceinline__ void reduce_tile(uint32_t stage, int chunk, const Row
         accd[1] = (kMulti<KT> || SS) ? d.s : d.g;  // K = 1: replica 0 is the mean
         accd[2] = d.w;
         accf[0] = accf[1] = accf[2] = 0.f;
-        acce[0] = acce[1] = acce[2] = 0;
         tail = true;
         return;
     }
@@ -1272,8 +1265,8 @@ __device__ __forceinline__ void reduce_tile(uint32_t stage, int chunk, const Row
                         float4 s = x[0];
 #pragma unroll
                         for (int k = 1; k < KT; ++k) s = add4(s, x[k]);
-                        column1<KT, WM, RW, SS, PR>(x[0], s, wv, sv, out + 4 * v, sc, K, ag, as,
-                                                    aw, pg, ps, pw);
+                        column1<KT, WM, RW, SS, PR>(x[0], s, wv, sv, out + 4 * v, sc, ag, as, aw,
+                                                    pg, ps, pw);
                     }
                 }
                 if (!PR) {
@@ -1311,8 +1304,8 @@ __device__ __forceinline__ void reduce_tile(uint32_t stage, int chunk, const Row
                         s = add4(s, lds4(stage + (uint32_t)((k * chunk + 4 * v) * 4)));
                     const float4 wv = RW ? lds4(sw_s + (uint32_t)(16 * v)) : x0;
                     const float4 sv = SS ? lds4(ss_s + (uint32_t)(16 * v)) : x0;
-                    column1<KT, WM, RW, SS, PR>(x0, s, wv, sv, out + 4 * v, sc, K, ag, as, aw, pg, ps,
-                                                pw);
+                    column1<KT, WM, RW, SS, PR>(x0, s, wv, sv, out + 4 * v, sc, ag, as, aw, pg,
+                                                ps, pw);
                 }
             } else {
 #pragma unroll 1
@@ -1339,7 +1332,7 @@ __device__ __forceinline__ void reduce_tile(uint32_t stage, int chunk, const Row
                     for (int u = 0; u < U; ++u) {
                         const int v = v0 + 32 * (u0 + u);
                         if (v < nv)
-                            column1<KT, WM, RW, SS, PR>(x0[u], s[u], wv[u], sv[u], out + 4 * v, sc, K,
+                            column1<KT, WM, RW, SS, PR>(x0[u], s[u], wv[u], sv[u], out + 4 * v, sc,
                                                         ag, as, aw, pg, ps, pw);
                     }
                 }
@@ -1422,13 +1415,10 @@ __device__ __forceinline__ void reduce_tile(uint32_t stage, int chunk, const Row
         }
         const bool own_s = kMulti<KT> || SS;  // K = 1: replica 0 is the mean
         accf[0] = fg;
-        acce[0] = eg;
         accd[0] = rg;
         accf[1] = own_s ? fs : fg;
-        acce[1] = own_s ? es : eg;
         accd[1] = own_s ? rs : rg;
         accf[2] = fw;
-        acce[2] = ew;
         accd[2] = rw;
     }
 }
@@ -1589,11 +1579,10 @@ __global__ void __launch_bounds__(Ring1Of<KT, RW, SH>::kThreads, 1)
             const Row<TableOf<Small>> ptr{tab, q.t};
             double accd[kAcc];
             float accf[kAcc];
-            int acce[kAcc];
             unsigned tcode;
             bool tile_tail;
             reduce_tile<KT, WM, RW, SS, PR, SH>(st.stage, chunk, ptr, st.tc.stream(0), q, st.tc.nv, st.tc.aligned, sc,
-                                            accd, accf, acce, tcode, tile_tail);
+                                            accd, accf, tcode, tile_tail);
             __syncwarp();
             const int tg = q.tg;
             const bool shifted = SH && !st.tc.aligned;
@@ -2636,12 +2625,10 @@ Scalars make_scalars(const tula_ags_hparams *hp, int K, int n, void *ws, const W
     sc.K = K;
     sc.mode = mode;
     sc.n_total = n;
-    sc.pow2K = (K & (K - 1)) == 0;
     sc.invK = 1.0f / (float)K;
     sc.Kf = (float)K;
     if (hp) {
         sc.rule = hp->rule;
-        sc.gran = hp->granularity;
         sc.force = hp->force_branch;
         sc.refresh = hp->refresh_scale;
         sc.delta = hp->delta;
