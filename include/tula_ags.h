@@ -48,9 +48,10 @@
  *     coefficient (gradscale refresh, LARS) split every square exactly into two
  *     fp32 parts, add them as float-float pairs (off a 16-byte boundary: as triples) per
  *     lane and in fp64 across lanes (relative error below 72 * 2^-46 = 1.1e-12, about
- *     1e-15 on ordinary data; triples below 2^-49), then exactly across tiles; a tile whose pairs cannot hold that (a
- *     square that overflows, or sums below 2^-77) is redone with exact fp64
- *     squares, so these norms keep that precision over the whole fp32 range.
+ *     1e-15 on ordinary data; triples below 2^-49), then exactly across tiles; a tile
+ *     whose sums cannot hold that (a square that overflows, or sums below 2^-77) is
+ *     redone with exact fp64 squares, so these norms keep that precision over the
+ *     whole fp32 range.
  */
 #ifndef TULA_AGS_H
 #define TULA_AGS_H
@@ -75,7 +76,9 @@ extern "C" {
 #define TULA_ERR_SCRATCH_LIMIT (-5) /* tula_ags_step_static_scratch: the tensor list needs more
                                        scratch than TULA_STATIC_SCRATCH_BYTES */
 #define TULA_ERR_NO_MEMORY (-6)   /* host memory for launch tables or a plan could not be
-                                     allocated; nothing was enqueued */
+                                     allocated.  A step builds its update's tables after its
+                                     reduction has been enqueued: as after TULA_ERR_CUDA, zero
+                                     the workspace again before reusing it */
 
 #define TULA_MAX_K 16
 
@@ -156,7 +159,8 @@ typedef struct tula_ags_hparams {
 void tula_ags_default_hparams(tula_ags_hparams *hp, int K);
 
 /* Bytes of workspace needed for this list of tensor sizes and K replicas (host only): about
- * 1.6 KB per tensor (accumulators and per-tensor sums), whatever the tensors' sizes. */
+ * 1.6 KB per tensor (accumulators, a coefficient and 32 unused bytes), whatever the tensors'
+ * sizes. */
 int tula_ags_workspace_size(const int64_t *numels, int n_tensors, int K, size_t *bytes);
 
 /*

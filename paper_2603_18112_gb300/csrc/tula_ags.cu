@@ -127,9 +127,9 @@ enum Mode { kModeStep = 0, kModeStats = 1, kModeScale = 2 };
 // One launch's tensors: sizes, first tiles and pointers, in a parameter block of Bytes bytes.  The
 // arrays lie one after the other in `raw`, `np` pointers per tensor: a pointer is its role's base
 // plus a 32-bit offset in fp32 elements (a 16 GB window), with 16 more bits when some role's
-// tensors lie farther apart (`wide`).  8 to 12 bytes per tensor and 8 per pointer, as the table was
-// before, took 4096 tensors with K = 16 through 21 launches of pass 1 instead of 10, and left more
-// of the block to miss the constant cache on.
+// tensors lie farther apart (`wide`).  6 bytes per tensor and 4 per pointer put 4096 tensors with
+// K = 16 through 10 launches of pass 1 (whole pointers and sizes: 21), and leave less of the block
+// to miss the constant cache on.
 constexpr int kHints = 160;
 constexpr int kMaxRoles = TULA_MAX_K + 1;
 struct TableHead {
@@ -784,23 +784,24 @@ struct TensorCache {
 // Each warp streams for itself: it has one stage of shared memory and one mbarrier, waits for the
 // tile in it, computes, and issues its next tile into the same stage as soon as every lane has read
 // the last one, before it adds that tile's sums up.  Lane i < ns fetches stream i's pointer (role
-// roles[i]) and issues that stream's copy to offset i * chunk floats of the stage.  While one warp
+// i) and issues that stream's copy to offset i * chunk floats of the stage.  While one warp
 // of a CTA computes, the others' copies are in flight; nothing is handed from warp to warp.
-// A producer warp that issues for all of them, as here before, is what bounded the passes: one
-// warp issues a bulk copy every ~27 ns (the lanes of one instruction go in turn), so 16 streams
-// of 2 KB took 0.83 us of a 36 KB stage's 0.80 us at the HBM rate, and 8 streams delayed every
-// refill.  Streams read this way alone run at 6.95-6.99 TB/s whatever the copy size (512 B to
-// 18 KB), against 6.09 TB/s with one producer warp and 16 copies of 2 KB.
+// One producer warp for all of them would bound the passes: a warp issues a bulk copy every ~27 ns
+// (the lanes of one instruction go in turn), so 16 streams of 2 KB would take 0.83 us of a 36 KB
+// stage's 0.80 us at the HBM rate, and 8 streams delay every refill.  Streams read this way alone
+// run at 6.95-6.99 TB/s whatever the copy size (512 B to 18 KB), against 6.09 TB/s with one
+// producer warp and 16 copies of 2 KB.
 //
 // Dealing: a launch has V = gridDim.x * kWarps streaming warps; warp v first takes tile v, then,
 // when there are more tiles than warps, tiles claimed one at a time from a global counter
-// (ctr[0]), the claim made a whole tile ahead so that its round trip is never waited for.  SMs
-// stream at unequal rates; with 36 KB tiles claims run at 7.19-7.25 TB/s where a fixed deal runs
-// at 6.95.  (Tiles under ~18 KB would be bound by the counter: one atomic every 1.5-2.8 ns.)  A
-// launch of nc tiles that claims makes exactly nc claims (nc - V tiles and one past the end for
-// each warp), so the host knows where the next launch on the counter begins, and nobody waits at
-// the end of a launch to re-arm it: the update does that for pass 1, k_finish for pass 2.  (A fence
-// and a ticket per warp for it took about 1 us at the end of each pass.)  Where a tile is
+// (ctr[0]), the claim made a whole tile ahead so that its round trip passes while the tile issued
+// before it is on its way (claim()).  SMs stream at unequal rates; with 36 KB tiles claims run at
+// 7.19-7.25 TB/s where a fixed deal runs at 6.95.  (Tiles under ~18 KB would be bound by the
+// counter: one atomic every 1.5-2.8 ns.)  A launch of nc tiles that claims makes exactly nc claims
+// (nc - V tiles and one past the end for each warp), so the host knows where the next launch on the
+// counter begins, and nobody waits at the end of a launch to re-arm it: the update does that for
+// pass 1 (k_share in a sharded step), k_finish for pass 2 and for the calls without an update.  (A
+// fence and a ticket per warp would take about 1 us at the end of each pass.)  Where a tile is
 // processed never changes its result: each tile's partial sums are added exactly, in integers,
 // into its tensor's accumulators.
 //
@@ -812,10 +813,10 @@ struct TensorCache {
 // elements of the neighbouring tiles along, which another warp may be updating; nobody reads
 // them.)  The up to three elements at each end of a tensor outside those granules, and the last
 // n % 4 elements of an aligned tensor, come by 4-byte cp.async into the same places.  Only the
-// kernels for launches with such a tensor (SH) hold this code: in the others it cost 0.4 % (ResNet-50)
-// to 5 % (1024 small layers) of a step, and they load an aligned tensor's tail directly.  17.3 M
-// elements in 128 tensors, K = 4, the gradients packed, take 125 us a step, against 101 us aligned;
-// loaded one element at a time and squared in fp64 they took 548.
+// kernels for launches with such a tensor (SH) hold this code: in the others it would cost 0.4 %
+// (ResNet-50) to 5 % (1024 small layers) of a step, and they load an aligned tensor's tail
+// directly.  17.3 M elements in 128 tensors, K = 4, the gradients packed, take 125 us a step,
+// against 101 us aligned, and 548 loaded one element at a time and squared in fp64.
 
 // A shifted tile, or the last tile of an aligned tensor of n % 4 != 0 elements: this lane's stream
 // (mine; nullptr: none) of n elements from `begin` of a tensor with `rest` elements from there on.
@@ -1095,8 +1096,8 @@ __device__ __noinline__ F3 tile_cols_scaled(uint32_t stage, int chunk, int nv, c
     return r;
 }
 
-// A tile of a tensor off a 16-byte boundary (see issue_edge_tile() for where its elements lie): lane l
-// takes elements l, l + 32, ..., U at a time, with conflict-free 4-byte loads from shared
+// A tile of a tensor off a 16-byte boundary (see issue_edge_tile() for where its elements lie):
+// lane l takes elements l, l + 32, ..., four at a time, with conflict-free 4-byte loads from shared
 // memory and coalesced 4-byte stores of the mean.  The squares are added as triples in either
 // mode, so that these norms hold fp64's precision.  Returns the lane's sums; out of line, so that
 // the streaming loop of aligned tensors keeps its shape.
@@ -1279,9 +1280,9 @@ __device__ __forceinline__ void reduce_tile(uint32_t stage, int chunk, const Row
         }
     }
     if (nv >= 0) {
-        // Ragged tile, or K known only at run time.  The latter takes U columns together, replica by
-        // replica, so that U loads are always in flight: one column at a time, every load waited
-        // for the one before, and K = 6 took 234 us a ResNet-50 step, 213 with this.
+        // Ragged tile, or K known only at run time.  The latter takes U columns together, replica
+        // by replica, so that U loads are always in flight (ResNet-50, K = 6: 213 us a step, and
+        // 234 one column at a time, each load waiting for the one before).
         constexpr int U = PR ? 2 : 4;
         // The tail's loads go first (not SH, K known: one lane per element), to land meanwhile.
         constexpr bool kTailFirst = !SH && KT > 0;
@@ -1466,9 +1467,10 @@ constexpr unsigned long long limbs_max_add() {
     return most;
 }
 static_assert(limbs_max_add() <= 2ull << 32, "a shifted tile adds to a word as two partials do");
+
 // The lanes' fp64 sums d[0 .. R) (>= 0, finite or not) of a shifted tile into R accumulators, and
-// the first one into `also` as well (unless NULL).  An fp64 tree across the warp took 4000 cycles of
-// a tile's 13,000 on GB300's slow FP64 pipe, so the lanes are added as integers: relative to the
+// the first one into `also` as well (unless NULL).  An fp64 tree across the warp takes 4000 cycles
+// of a tile's 13,000 on GB300's slow FP64 pipe, so the lanes are added as integers: relative to the
 // warp's largest exponent a sum is a fixed-point number of 79 bits, limbs of 26, 26 and 27, and
 // each limb's warp total (below 2^32) takes one instruction.  What lies below 2^-78 of the largest
 // sum is cut off, less than an fp64 addition's own rounding.  The totals are exact integers and go
@@ -1498,8 +1500,10 @@ __device__ __noinline__ void add_shifted(const double (&d)[R], unsigned long lon
         const int shift = top - e;
         // Bits 78 .. 26: m >> shift; bits 25 .. 0: the first 26 of those that cuts off.
         const unsigned long long hi = shift < 64 ? m >> shift : 0ull;
-        const unsigned long long cut = shift == 0 ? 0ull
-                                       : shift < 64 ? m << (64 - shift) : shift < 128 ? m >> (shift - 64) : 0ull;
+        const unsigned long long cut = shift == 0    ? 0ull
+                                       : shift < 64  ? m << (64 - shift)
+                                       : shift < 128 ? m >> (shift - 64)
+                                                     : 0ull;
         const unsigned low = (unsigned)(cut >> 38);
         const unsigned l0 = __reduce_add_sync(kFull, low);
         const unsigned l1 = __reduce_add_sync(kFull, (unsigned)(hi & 0x3ffffffull));
@@ -1581,8 +1585,8 @@ __global__ void __launch_bounds__(Ring1Of<KT, RW, SH>::kThreads, 1)
             float accf[kAcc];
             unsigned tcode;
             bool tile_tail;
-            reduce_tile<KT, WM, RW, SS, PR, SH>(st.stage, chunk, ptr, st.tc.stream(0), q, st.tc.nv, st.tc.aligned, sc,
-                                            accd, accf, tcode, tile_tail);
+            reduce_tile<KT, WM, RW, SS, PR, SH>(st.stage, chunk, ptr, st.tc.stream(0), q, st.tc.nv,
+                                                st.tc.aligned, sc, accd, accf, tcode, tile_tail);
             __syncwarp();
             const int tg = q.tg;
             const bool shifted = SH && !st.tc.aligned;
@@ -1656,10 +1660,9 @@ __global__ void __launch_bounds__(Ring1Of<KT, RW, SH>::kThreads, 1)
 // Delta (Eq. 5) and the branch of Algorithm 1 for the step record; the update has taken the same
 // branch from the same accumulator (step_branch).  No warp waits for another.
 //
-// Everything here used to stand between the passes, in a kernel of its own.  The update then
-// waited for it: 9.9 us from the end of the reduction to the update's first tile on ResNet-50,
-// 3.7 of them the record's fp64 division.  Only LARS, whose coefficients are ratios of this
-// step's norms, still has a kernel there (k_lars).
+// Between the passes it would keep the update waiting: 9.9 us from the end of the reduction to the
+// update's first tile on ResNet-50, 3.7 of them the record's fp64 division.  Only LARS, whose
+// coefficients are ratios of this step's norms, has a kernel there (k_lars).
 
 // The square roots of three norms (lanes 0-2 in one fp64 sequence) and the two ratios of a
 // tensor (lanes 0 and 1): UpdateGradScale's |g_s| / (|g_l| + eps) and |w| / |gbar| (LARS, the
@@ -1927,7 +1930,8 @@ __device__ __noinline__ float w_cols_scaled(uint32_t w_stage, int nv, float f) {
 // A tile of a tensor off a 16-byte boundary, as tile_shifted() of pass 1: four elements per lane
 // and step.  Returns the lane's |w|^2 (triples, to fp64 once) when the statistics want it.
 template <bool HM, bool PE, bool SW, typename Tab>
-__device__ __noinline__ double update_shifted(uint32_t stage, const Tab &tab, int t, long long begin, int n, float ct, bool use_se,
+__device__ __noinline__ double update_shifted(uint32_t stage, const Tab &tab, int t,
+                                              long long begin, int n, float ct, bool use_se,
                                               const Scalars &sc) {
     constexpr uint32_t part = (uint32_t)(4 * Ring2<false>::tile_elems(2 + (HM ? 1 : 0) + (PE ? 1 : 0)) +
                                          kShiftBytes);
@@ -1999,7 +2003,8 @@ __global__ void __launch_bounds__(Ring2<SH>::kThreads, 1)
     // step (whatever ran between its two calls).  The next kernel may start when that wait has
     // passed: the next step's reduction reads the mean this step's has written.  A later launch of
     // the pass only has to complete after the one before, as in k_reduce; what it reads was final
-    // when that one let it start, and it reads it through L2 (its own wait comes later).
+    // when that one let it start, and it reads it from L2 (its own wait comes later): by TMA and
+    // ld.cg, and the ends of shifted tiles through an L1 that it has given up (forget_l1).
     const bool first = tab.seq == 0;
     const bool early = !PE && first && sc.early_w;
     if (first && !early) {
@@ -2147,8 +2152,8 @@ __global__ void __launch_bounds__(Ring2<SH>::kThreads, 1)
             }
             if constexpr (SH) {
                 if (!st.tc.aligned)
-                    awt = update_shifted<HM, PE, SW>(stage, tab, q.t, q.begin, (int)(q.end - q.begin), ct,
-                                                     use_se, sc);
+                    awt = update_shifted<HM, PE, SW>(stage, tab, q.t, q.begin,
+                                                     (int)(q.end - q.begin), ct, use_se, sc);
             }
             const bool tile_tail = 4 * (long long)nv < n;  // the same in every lane
             if (in_tail) {
@@ -2200,7 +2205,10 @@ __global__ void __launch_bounds__(Ring2<SH>::kThreads, 1)
             int idx;
             const float f = warp_reduce_scatter<kPend>(pend, idx);
             if ((lane & 7) == 0) {
-                const int tg = idx == 0 ? ptensor[0] : idx == 1 ? ptensor[1] : idx == 2 ? ptensor[2] : ptensor[3];
+                const int tg = idx == 0   ? ptensor[0]
+                               : idx == 1 ? ptensor[1]
+                               : idx == 2 ? ptensor[2]
+                                          : ptensor[3];
                 if (tg >= 0)
                     acc_add_f32(acc2_of(sc, tg), f,
                                 -2 * scale_exp((ecode >> (2 * idx)) & 3u));
@@ -2461,9 +2469,9 @@ struct TableCache {
     }
 };
 
-// The pointers of a pass's launches: fill(p, ptrs) writes tensor p's np pointers.
-// What the tables of tensors [0, n) need: whether every role's pointers lie within 16 GB of its
-// lowest, and whether some non-empty tensor has a pointer off a 16-byte boundary.
+// What the tables of tensors [0, n) need: each role's lowest pointer, whether all of its pointers
+// lie within 16 GB of that, and whether some non-empty tensor has a pointer off a 16-byte boundary.
+// fill(p, ptrs) writes tensor p's np pointers.
 struct Pointers {
     unsigned long long base[kMaxRoles] = {};
     bool wide = false, shifted = false;
@@ -2602,7 +2610,8 @@ int launch_streaming(const StreamKernels &k, int n, const int64_t *numels, int c
         if (blocks->small)
             rc = launch_block(k.small, b.get(), threads, k.smem, sc, grid_override, stream, base);
         else if (static_cast<const FullTab *>(b.get())->shifted)
-            rc = launch_block(k.shifted, b.get(), threads, k.smem_shifted, sc, grid_override, stream, base);
+            rc = launch_block(k.shifted, b.get(), threads, k.smem_shifted, sc, grid_override,
+                              stream, base);
         else
             rc = launch_block(k.full, b.get(), threads, k.smem, sc, grid_override, stream, base);
         if (rc) return rc;
@@ -2779,8 +2788,6 @@ int tula_ags_workspace_error(const void *workspace, size_t workspace_bytes,
 
 namespace {
 
-// Every host-side check of a step's arguments except the workspace: TULA_OK or the status
-// tula_ags_step returns.  Nothing is enqueued before it passes.
 // The options of a step (hp apart from its workspace, and the momentum) against the buffers the
 // step has: momentum buffers (has_mom) and per-element gradscales (has_se).
 int check_step_options(const tula_ags_hparams *hp, float momentum, bool has_mom, bool has_se) {
@@ -2820,6 +2827,8 @@ int check_step_tensors(float *const *param_ptrs, float *const *grad_ptrs, float 
     return TULA_OK;
 }
 
+// Every host-side check of a step's arguments except the workspace: TULA_OK or the status
+// tula_ags_step returns.  Nothing is enqueued before it passes.
 int check_step_args(float *const *param_ptrs, float *const *grad_ptrs, float *const *mom_ptrs,
                     const int64_t *numels, int n_tensors, float momentum,
                     const tula_ags_hparams *hp, Plan *pl) {
@@ -3185,9 +3194,9 @@ extern "C" int tula_ags_step_static_scratch(float *const *param_ptrs, float *con
     void *scratch = nullptr;
     rc = static_scratch_address(&scratch);
     if (rc) return rc;
-    // The array keeps the last call's contents: zero the tile counters and the accumulators before this call's kernels.  The error
-    // word between them is left alone, so that a wait that ran out stays reported until
-    // tula_ags_static_scratch_error reads it.
+    // The array keeps the last call's contents: zero the tile counters and the accumulators before
+    // this call's kernels.  The error word is left alone, so that a wait that ran out stays reported
+    // until tula_ags_static_scratch_error reads it.
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     char *b = static_cast<char *>(scratch);
     cudaError_t e = cudaMemsetAsync(b, 0, L.err, s);

@@ -418,8 +418,8 @@ class AGSOptimizerStep:
 
     def set_trace_events(self, events):
         """Up to five cudaEvent_t handles (or None) recorded at the kernel boundaries of a
-        step: before the reduction, after it, after its combine, after the update, after the
-        update's combine."""
+        step: before the reduction, after it, before the update (after LARS's coefficients), after
+        the update, after the kernel that finishes the norms and the step record."""
         for i in range(5):
             ev = events[i] if events is not None and i < len(events) else None
             self.hp.trace_events[i] = (ev.cuda_event if hasattr(ev, "cuda_event") else ev) or None
