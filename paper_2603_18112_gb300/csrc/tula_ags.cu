@@ -27,8 +27,8 @@
 // stream issued by one lane each, and claim tiles from a global counter (SMs
 // stream at unequal rates).  Tile partials are fp32 sums within a tile
 // (float-float pairs per lane in the precise mode for norms that feed a
-// coefficient), range-checked per tile, and leave the tile only as exact integer
-// additions into the accumulators.
+// coefficient, triples for misaligned tensors), range-checked per tile, and leave
+// the tile only as exact integer additions into the accumulators.
 //
 // Every mbarrier wait is bounded; a wait that runs out sets an error word in
 // the workspace (tula_ags_workspace_error) and the CTA drains its copies in
@@ -1398,8 +1398,9 @@ __device__ __forceinline__ void reduce_tile(uint32_t stage, int chunk, const Row
         int eg = 0, es = 0, ew = 0;
         // One vote per tile; the warp maxima only when some lane is out of range.  A lane
         // without columns (lane >= ncols) has nothing to check.
-        const bool lane_ok = lane >= ncols || (sq_in_range(fg) && (!(kMulti<KT> || SS) || sq_in_range(fs)) &&
-                                               (!RW || sq_in_range(fw)));
+        const bool lane_ok =
+            lane >= ncols || (sq_in_range(fg) && (!(kMulti<KT> || SS) || sq_in_range(fs)) &&
+                              (!RW || sq_in_range(fw)));
         if (ncols > 0 && !__all_sync(kFull, lane_ok)) {
             eg = sq_range_exp(fg);
             if (kMulti<KT> || SS) es = sq_range_exp(fs);
@@ -1923,7 +1924,8 @@ __device__ __forceinline__ float update4(float4 g4, float4 w4, float4 m4, float4
 // or lose their precision to underflow.  Out of line, like tile_cols_scaled.
 __device__ __noinline__ float w_cols_scaled(uint32_t w_stage, int nv, float f) {
     float a = 0.f;
-    for (int v = threadIdx.x & 31; v < nv; v += 32) a = sq4(a, mul4(lds4(w_stage + (uint32_t)(16 * v)), f));
+    for (int v = threadIdx.x & 31; v < nv; v += 32)
+        a = sq4(a, mul4(lds4(w_stage + (uint32_t)(16 * v)), f));
     return a;
 }
 
@@ -2424,7 +2426,8 @@ long long l2_bytes() {
 
 // Launch with programmatic stream serialization: the kernel may begin while
 // the previous kernel in the stream finishes; its griddepcontrol.wait orders
-// every memory access after that kernel's completion.
+// what follows after that kernel's completion (what k_update and the later
+// launches of a pass read before theirs is said there).
 template <typename... KArgs, typename... Args>
 int launch_pdl(void (*kernel)(KArgs...), int grid, int threads, int smem, cudaStream_t s,
                Args &&...args) {
